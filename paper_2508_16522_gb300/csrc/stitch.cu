@@ -118,10 +118,12 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
   const uint32_t n = (uint32_t)p.n;
   int nl = 0;          // kept ready items (warp-uniform)
   uint32_t pend = 0;   // executed, not yet counted (warp-uniform)
-  uint64_t idle_since = 0, last_check = 0;
+  uint64_t idle_since = 0, last_check = 0, last_status = 0;
   unsigned long long seen = 0;
   uint32_t backoff = 32;
   uint32_t my_t = kNoTk;  // this lane's claimed ring ticket
+  // ring items need no ordering unless a body reads its predecessors' results
+  // or tickets are compared (counters and trigger records: see exec.cu)
 
   for (;;) {
     uint64_t item = kEmpty64;
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
     // 1. this lane's ticket, once published
     bool waiting = my_t != kNoTk;
     if (waiting && my_t < p.ring_cap) {
-      const uint64_t vv = ld_acquire_u64(p.ring + my_t);
+      const uint64_t vv = FENCE || TICKETS ? ld_acquire_u64(p.ring + my_t) : ld_relaxed_item(p.ring + my_t);
       if (vv != kEmpty64) {
         item = vv;
         my_t = kNoTk;
@@ -167,11 +169,20 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
       }
       int stop = 0;
       if (lane == 0) {
-        const unsigned long long ex = ld_relaxed_u64(&ctrl->executed);
-        if (ld_relaxed_u32(&ctrl->status) != 0u || ex >= (unsigned long long)p.total) {
+        // the shared words, read at most every microsecond per idle warp (all of
+        // them reading at every pass would pile onto one L2 line)
+        const uint64_t now = globaltimer_ns();
+        const bool look = now - last_status >= 1000u;
+        unsigned long long ex = seen;
+        uint32_t st = 0u;
+        if (look) {
+          last_status = now;
+          ex = ld_relaxed_u64(&ctrl->executed);
+          st = ld_relaxed_u32(&ctrl->status);
+        }
+        if (st != 0u || ex >= (unsigned long long)p.total) {
           stop = 1;
-        } else {
-          const uint64_t now = globaltimer_ns();
+        } else if (look) {
           if (idle_since == 0) {
             idle_since = last_check = now;
             seen = ex;
@@ -300,7 +311,8 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
           if ((uint64_t)base + (uint64_t)nover > (uint64_t)p.ring_cap) {
             if (lane == 0) atomicCAS(&ctrl->status, 0u, (uint32_t)RT_ERR_OOM);
           } else if (ready && rank >= room) {
-            st_release_u64(p.ring + base + (rank - room), nit);
+            if (FENCE || TICKETS) st_release_u64(p.ring + base + (rank - room), nit);
+            else st_relaxed_u64(p.ring + base + (rank - room), nit);
           }
         }
         nl += rcount < room ? rcount : room;
