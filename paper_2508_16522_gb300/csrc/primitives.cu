@@ -169,6 +169,9 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const K* keys, int
     const int64_t k = base + j * kRadixThreads + threadIdx.x;
     kv[j] = k < n ? keys[k] : K(0);
   }
+#pragma unroll
+  for (int j = 0; j < kRadixIpt; ++j)
+    if (base + j * kRadixThreads + threadIdx.x < n) atomicAdd(&h[(uint32_t)(kv[j] >> shift) & mask], 1u);
   __syncthreads();
   hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
@@ -207,6 +210,14 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   uint64_t vv[HAS_V ? kRadixIpt : 1];
   uint32_t rk[kRadixIpt];
   const unsigned lt = lanemask_lt();
+  // every key's load in flight before the ranking, whose warp barriers would hold
+  // each round's loads back until the round before it is done (two passes over the
+  // 343M entries of the 1M-launch trace: 9.9 -> 7.1 ms)
+#pragma unroll
+  for (int r = 0; r < kRadixIpt; ++r) {
+    const int64_t idx = wbase + r * 32 + lane;
+    kv[r] = idx < n ? keys[idx] : K(0);
+  }
 #pragma unroll
   for (int r = 0; r < kRadixIpt; ++r) {
     int64_t idx = wbase + r * 32 + lane;
@@ -244,6 +255,13 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   for (int w = 0; w < kRadixWarps; ++w) wpre += w < warp ? wsum[w] : 0u;
   bstart[threadIdx.x] = wpre + incl - tot;
   if (threadIdx.x == kRadixThreads - 1) bstart[256] = wpre + incl;
+  if (HAS_V) {
+#pragma unroll
+    for (int r = 0; r < kRadixIpt; ++r) {
+      const int64_t idx = wbase + r * 32 + lane;
+      vv[HAS_V ? r : 0] = idx < n ? vals[idx] : 0ull;
+    }
+  }
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < kRadixIpt; ++r) {
@@ -264,9 +282,6 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     keys_out[dst] = k;
     if (HAS_V) vals_out[dst] = sv[i];
   }
-#pragma unroll
-  for (int j = 0; j < kRadixIpt; ++j)
-    if (base + j * kRadixThreads + threadIdx.x < n) atomicAdd(&h[(uint32_t)(kv[j] >> shift) & mask], 1u);
 }
 
 template <typename K, bool HAS_V>
@@ -305,14 +320,6 @@ int radix_sort(K* keys, K* keys_alt, uint64_t* vals, uint64_t* vals_alt, int64_t
   int64_t nb = (n + kRadixTile - 1) / kRadixTile;
   int64_t h = 256 * nb;
   uint32_t* hist = (uint32_t*)ws;
-  // every key's load in flight before the ranking, whose warp barriers would hold
-  // each round's loads back until the round before it is done (two passes over the
-  // 343M entries of the 1M-launch trace: 9.9 -> 7.1 ms)
-#pragma unroll
-  for (int r = 0; r < kRadixIpt; ++r) {
-    const int64_t idx = wbase + r * 32 + lane;
-    kv[r] = idx < n ? keys[idx] : K(0);
-  }
   uint32_t* offs = hist + h;
   uint32_t* sws = offs + h + 1;
   K* kin = keys;
@@ -352,13 +359,6 @@ template int radix_sort<uint64_t>(uint64_t*, uint64_t*, uint64_t*, uint64_t*, in
 // kernel, e.g. the serving kernel).
 void preload_primitives() {
   cudaFuncAttributes a;
-  if (HAS_V) {
-#pragma unroll
-    for (int r = 0; r < kRadixIpt; ++r) {
-      const int64_t idx = wbase + r * 32 + lane;
-      vv[HAS_V ? r : 0] = idx < n ? vals[idx] : 0ull;
-    }
-  }
   cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t>);
   cudaFuncGetAttributes(&a, k_scan_reduce<uint64_t>);
   cudaFuncGetAttributes(&a, k_scan_down<uint32_t>);
