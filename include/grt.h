@@ -139,8 +139,9 @@ typedef struct {
   float ms_sweep_kernel;  /* the interference sweep kernel alone */
   int32_t csr_by_buckets; /* 1: the CSR was built from per-source buckets (every row held at most
                              1024 candidate pairs), 0: from a radix sort of all the pairs */
-  int32_t pair_filter_bits; /* dense inputs (16+ binned entries per task): log2 of the slots of the
-                               pair-key filter the first sweep wrote through (a pair found again in
+  int32_t pair_filter_bits; /* dense inputs (16+ binned entries per task): log2 of the most slots the
+                               pair filter may have (as many, a power of two, for each task), which
+                               the first sweep wrote through (a pair found again in
                                another tile is not written again); 0: no filter */
   int32_t pad1;
   /* diagnostic counters of the last executor launch: batches, tasks, edges,

@@ -142,12 +142,12 @@ struct rt_graph {
   DevBuf err;  // uint32 device-side validation bits
   bool pending_validate = false;
   // analysis
-  DevBuf rect_task, cnt, keys, keys_alt, pay, pay_alt, seg_b, seg_e, pairs, pairs_alt, flags, upos;
+  DevBuf rect_task, cnt, keys, keys_alt, pay, pay_alt, tiles, pairs, pairs_alt, flags, upos;
   DevBuf col, row_ptr, indeg, count, rootpos, root_items, ws, misc, adj;
   DevBuf adjx;          // the owned executor's extension records, built on its first run after an analysis
   bool adjx_ok = false;
   int32_t max_outdeg = 0;  // largest out-degree of the analysed graph
-  DevBuf tflags;  // per tile: dropped a pair in the first sweep / in the rerun
+  int32_t max_span = 0, last_root = 0;  // its longest edge (target - source) and last root
   DevBuf pfilt;   // dense inputs: the first sweep's pair-key filter
   int pair_filter_bits = 0;  // log2 of its slots in the last analysis (0: not used)
   DevBuf bucket;  // CSR by buckets: per-task counts, offsets, distinct counts, long-row list, control words
@@ -168,6 +168,7 @@ struct rt_graph {
   int32_t st_R = 0;  // replays of the last stitched run with tickets
   // execution
   DevBuf ring, ctrl, gtable, done_g, tickets;
+  DevBuf spill;  // a run inside one block: its ready queue past the shared memory
   uint32_t* hpin = nullptr;  // pinned readback area (64 words)
   bool analyzed = false, dirty = false, status_pending = false;
   int64_t n_edges = 0, n_roots = 0, n_entries = 0, n_pairs = 0;
@@ -191,10 +192,10 @@ namespace {
 template <class G, class F>
 void for_each_buf(G* g, F f) {
   auto bufs = {&g->req_off, &g->lo, &g->hi, &g->priv, &g->pred_off, &g->pred, &g->body_arg, &g->stage32, &g->err,
-                &g->rect_task, &g->cnt, &g->keys, &g->keys_alt, &g->pay, &g->pay_alt, &g->seg_b, &g->seg_e,
+                &g->rect_task, &g->cnt, &g->keys, &g->keys_alt, &g->pay, &g->pay_alt, &g->tiles,
                 &g->pairs, &g->pairs_alt, &g->flags, &g->upos, &g->col, &g->row_ptr, &g->indeg, &g->count,
                 &g->rootpos, &g->root_items, &g->ws, &g->misc, &g->adj, &g->adjx, &g->bucket, &g->ring, &g->ctrl,
-                &g->gtable, &g->done_g, &g->tickets, &g->tflags, &g->pfilt, &g->ev_pred_off, &g->ev_pred,
+                &g->gtable, &g->done_g, &g->tickets, &g->spill, &g->pfilt, &g->ev_pred_off, &g->ev_pred,
                 &g->ev_head, &g->ev_pending, &g->ev_nodes, &g->ev_ring, &g->ev_ctrl, &g->ksink, &g->st_count,
                 &g->st_ring, &g->st_ctrl, &g->st_tickets, &g->st_err};
   for (auto* b : bufs) f(*b);
@@ -389,6 +390,30 @@ rt_status rt_graph_destroy(rt_graph_t g) {
 // ---------------------------------------------------------------------------
 namespace {
 
+const char* err_bits_text(uint32_t e) {
+  if (e & 32u) return "a rectangle lies outside its own graph's domain";
+  if (e & 2u) return "a rectangle has lo > hi or lies outside the domain";
+  if (e & 4u) return "a privilege is not read/write/reduce";
+  if (e & 1u) return "req_off does not start at 0, decreases, or does not end at the rect count";
+  if (e & 8u) return "a predecessor is not an earlier task (or pred_off is malformed)";
+  if (e & 16u) return "a body_arg lies outside the state buffer";
+  return "invalid launch data";
+}
+
+// offsets that start at 0 and do not decrease (one pass without branches)
+bool offsets_ok(const int32_t* off, int32_t n) {
+  int bad = off[0] != 0;
+  for (int32_t i = 0; i < n; ++i) bad |= off[i + 1] < off[i];
+  return !bad;
+}
+
+// From this many launches, rectangles and predecessors on, a host batch's
+// contents are checked on the device once they are there (the host loop takes
+// about 1 ns each, 1.2 ms for a 1024 x 300 graph's predecessors; the copy,
+// kernel and wait about 60 us). The offsets, which say how much there is to
+// copy, are checked here first.
+constexpr int64_t kDeviceCheck = 65536;
+
 // T: the coordinate type of lo and hi (int64_t, or int32_t for rt_launch_batch32)
 template <class T>
 rt_status host_validate(const rt_graph* g, int32_t n, const int32_t* req_off, const T* lo, const T* hi,
@@ -428,6 +453,18 @@ rt_status copy_in(void* dst, const void* src, size_t bytes, cudaStream_t s) {
   if (!bytes) return RT_OK;
   CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s));
   return RT_OK;
+}
+
+// memory of the current device (a kernel may not reach another device's, which a
+// copy does)
+bool kernel_reads(const void* p) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
 rt_status ensure_pinned(rt_graph* g) {
@@ -486,6 +523,14 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
   const int D = g->dims.ndim;
   int64_t R = 0, Pb = 0;
   int32_t first[2] = {0, 0};
+  bool check_now = false;  // a host batch checked on the device before this call returns
+  auto on_host = [&]() -> rt_status {
+    if (c32)
+      return host_validate(g, n, req_off, static_cast<const int32_t*>(lo), static_cast<const int32_t*>(hi), priv,
+                           pred_off, pred, body_arg);
+    return host_validate(g, n, req_off, static_cast<const int64_t*>(lo), static_cast<const int64_t*>(hi), priv, pred_off,
+                         pred, body_arg);
+  };
   if (!dev) {
     R = req_off[n];
     Pb = pred_off ? pred_off[n] : 0;
@@ -494,12 +539,13 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     if (R < 0 || Pb < 0) return fail(RT_ERR_INVALID, "negative rect or pred count");
     if (R > 0 && (!lo || !hi || !priv)) return fail(RT_ERR_INVALID, "rect arrays are NULL");
     if (!on_device_check) {
-      if (c32)
-        CKR(host_validate(g, n, req_off, static_cast<const int32_t*>(lo), static_cast<const int32_t*>(hi), priv,
-                          pred_off, pred, body_arg));
-      else
-        CKR(host_validate(g, n, req_off, static_cast<const int64_t*>(lo), static_cast<const int64_t*>(hi), priv,
-                          pred_off, pred, body_arg));
+      check_now = (int64_t)n + R + Pb >= kDeviceCheck && offsets_ok(req_off, n) && (!pred_off || offsets_ok(pred_off, n));
+      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+      if (check_now && (cudaStreamIsCapturing(g->s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) {
+        cudaGetLastError();
+        check_now = false;
+      }
+      if (!check_now) CKR(on_host());
     }
   }
   CKR(ensure_device());
@@ -507,12 +553,13 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
   cudaStream_t s = g->s;
   if (dev) {
     // the batch's sizes live on the device: read both ends of the offset arrays
-    CK(cudaMemcpyAsync(g->hpin + 0, req_off, 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(g->hpin + 1, req_off + n, 4, cudaMemcpyDeviceToHost, s));
-    if (pred_off) {
-      CK(cudaMemcpyAsync(g->hpin + 2, pred_off, 4, cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(g->hpin + 3, pred_off + n, 4, cudaMemcpyDeviceToHost, s));
+    const int32_t* const at[4] = {req_off, req_off + n, pred_off, pred_off ? pred_off + n : nullptr};
+    ReportArgs ra;
+    for (int k = 0; k < (pred_off ? 4 : 2); ++k) {
+      if (kernel_reads(at[k])) ra.add(g->hpin + k, at[k]);
+      else CK(cudaMemcpyAsync(g->hpin + k, at[k], 4, cudaMemcpyDefault, s));
     }
+    launch_report(ra, s);
     CK(cudaStreamSynchronize(s));
     first[0] = (int32_t)g->hpin[0];
     R = (int32_t)g->hpin[1];
@@ -529,10 +576,12 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
 
   const int32_t n0 = g->n;
   const int64_t R0 = g->R, P0 = g->P;
-  // offsets: position 0 of the batch is the previous end, so copy [1..n]
+  const bool had_pred = g->has_pred, had_body_arg = g->has_body_arg;
+  // offsets: position 0 of the batch is the previous end, so copy [1..n] (a
+  // first batch's own 0 with them)
   CKR(g->req_off.reserve((size_t)(n0 + n + 1) * 4, s, (size_t)(n0 + 1) * 4));
-  if (n0 == 0) CK(cudaMemsetAsync(g->req_off.p, 0, 4, s));
-  CKR(copy_in(g->req_off.as<int32_t>() + n0 + 1, req_off + 1, (size_t)n * 4, s));
+  if (n0 == 0) CKR(copy_in(g->req_off.p, req_off, (size_t)(n + 1) * 4, s));
+  else CKR(copy_in(g->req_off.as<int32_t>() + n0 + 1, req_off + 1, (size_t)n * 4, s));
   launch_add_offset(g->req_off.as<int32_t>() + n0 + 1, n, (int32_t)R0, s);
   if (R > 0) {
     CKR(g->lo.reserve((size_t)(R0 + R) * D * 8, s, (size_t)R0 * D * 8));
@@ -577,11 +626,15 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     }
     g->has_body_arg = true;
   }
-  if (on_device_check) {
+  if (on_device_check || check_now) {
     if (!g->err.p) {
       CKR(g->err.reserve(256, s));
       CK(cudaMemsetAsync(g->err.p, 0, 4, s));
     }
+    // word 0 gathers the deferred checks' findings until the analysis, word 1 is
+    // this call's own
+    uint32_t* err = g->err.as<uint32_t>() + (check_now ? 1 : 0);
+    if (check_now) CK(cudaMemsetAsync(err, 0, 4, s));
     if (bp)  // each rectangle checked against its own graph's domain, then moved into its band
       launch_band_place(g->req_off.as<int32_t>() + n0, n, bp->task_first, bp->G, bp->box, D,
                         g->lo.as<int64_t>() + R0 * D, g->hi.as<int64_t>() + R0 * D, R, g->err.as<uint32_t>(), s);
@@ -590,8 +643,21 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
                     g->hi.as<int64_t>() + R0 * D, g->priv.as<uint8_t>() + R0, R,
                     g->has_pred ? g->pred_off.as<int32_t>() + n0 : nullptr, g->pred.as<int32_t>(), P0,
                     P0 + Pb, n0, body_arg ? g->body_arg.as<int32_t>() + n0 : nullptr, limit, g->dims,
-                    g->err.as<uint32_t>(), s);
-    g->pending_validate = true;
+                    err, s);
+    if (check_now) {
+      ReportArgs ra;
+      ra.add(g->hpin + 4, err);
+      launch_report(ra, s);
+      CK(cudaStreamSynchronize(s));
+      if (g->hpin[4] != 0u) {  // nothing was appended; the host check names the fault
+        g->has_pred = had_pred;
+        g->has_body_arg = had_body_arg;
+        CKR(on_host());
+        return fail(RT_ERR_INVALID, "device validation: %s", err_bits_text(g->hpin[4]));
+      }
+    } else {
+      g->pending_validate = true;
+    }
   }
   CK(cudaGetLastError());
   trace("launch_batch: copies enqueued");
@@ -607,15 +673,10 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
 // ---------------------------------------------------------------------------
 namespace {
 
-const char* err_bits_text(uint32_t e) {
-  if (e & 32u) return "a rectangle lies outside its own graph's domain";
-  if (e & 2u) return "a rectangle has lo > hi or lies outside the domain";
-  if (e & 4u) return "a privilege is not read/write/reduce";
-  if (e & 1u) return "req_off does not start at 0, decreases, or does not end at the rect count";
-  if (e & 8u) return "a predecessor is not an earlier task (or pred_off is malformed)";
-  if (e & 16u) return "a body_arg lies outside the state buffer";
-  return "invalid launch data";
-}
+// the sweep by windows: least mean share of its tile that an entry covers, and
+// (without the pair filter) least mean entries per tile
+constexpr double kWindowCover = 0.2;
+constexpr int kWindowTileEntries = 64;
 
 rt_status reserve_ws(rt_graph* g, size_t bytes) { return g->ws.reserve(bytes + 1024, g->s); }
 
@@ -634,26 +695,53 @@ rt_status run_analysis(rt_graph* g) {
   const int64_t ntiles = (int64_t)d.ntx * d.nty;
   trace("analyze: start");
   CKR(g->misc.reserve(256, s));
+  CK(cudaMemsetAsync(g->misc.p, 0, 256, s));
   trace("analyze: misc reserved");
   unsigned long long* cursor = reinterpret_cast<unsigned long long*>(g->misc.p);
   uint32_t* tile_counter = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 64);
+  // control words, zeroed above: 0 the pair cursor, 64 and 68 tile counters, 96
+  // tiles left by the sweep by windows, 100 the longest row, 104 long rows, 128
+  // pairs of the tiles to sweep again, 160 the rectangles' cells, 192
+  // the largest out-degree, the longest edge and the last root
+  uint32_t* nbail = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 96);
+  uint32_t* bmax = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 100);
+  uint32_t* bnbig = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 104);
+  unsigned long long* rerun = reinterpret_cast<unsigned long long*>(g->misc.as<char>() + 128);
+  unsigned long long* area = reinterpret_cast<unsigned long long*>(g->misc.as<char>() + 160);
+  uint32_t* shape = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 192);
   volatile uint64_t* h64 = reinterpret_cast<volatile uint64_t*>(g->hpin);  // 32 x u64
+  // CSR by buckets: counts [n+1], offsets [n+1], distinct counts [n+1], long
+  // rows [n+1]
+  CKR(g->bucket.reserve((size_t)4 * (n + 1) * 4, s));
+  uint32_t* bcnt = g->bucket.as<uint32_t>();
+  uint32_t* boff = bcnt + (n + 1);
+  uint32_t* bucnt = boff + (n + 1);
+  uint32_t* bbig = bucnt + (n + 1);
 
   // ---- 1-3: binning ------------------------------------------------------
   int64_t M = 0;
   const uint32_t* skeys = nullptr;
   const uint64_t* spay = nullptr;
+  // per tile: its segment of the sorted entries, and whether it dropped a pair
+  // in the first sweep / in the rerun (or was left by the sweep by windows)
+  uint32_t *seg_b = nullptr, *seg_e = nullptr;
+  uint8_t *flags1 = nullptr, *flags2 = nullptr;
   if (R > 0) {
     CKR(g->rect_task.reserve((size_t)R * 4, s));
     CKR(g->cnt.reserve((size_t)(R + 1) * 8, s));
     CKR(reserve_ws(g, scan_ws_elems<uint64_t>(R) * 8));
-    launch_bin_count(g->req_off.as<int32_t>(), n, g->lo.as<int64_t>(), g->hi.as<int64_t>(), R, d,
-                     g->rect_task.as<int32_t>(), g->cnt.as<uint64_t>(), s);
+    launch_bin_count(g->req_off.as<int32_t>(), n, R, g->lo.as<int64_t>(), g->hi.as<int64_t>(), d,
+                     g->rect_task.as<int32_t>(), g->cnt.as<uint64_t>(), area, bcnt, s);
     scan_exclusive<uint64_t>(g->cnt.as<uint64_t>(), g->cnt.as<uint64_t>(), R, g->ws.as<uint64_t>(), s);
-    CK(cudaMemcpyAsync((void*)&h64[0], g->cnt.as<uint64_t>() + R, 8, cudaMemcpyDeviceToHost, s));
   }
   h64[1] = 0;
-  if (g->pending_validate) CK(cudaMemcpyAsync((void*)&h64[1], g->err.p, 4, cudaMemcpyDeviceToHost, s));
+  ReportArgs ra1;
+  if (R > 0) {
+    ra1.add((void*)&h64[0], g->cnt.as<uint64_t>() + R, true);
+    ra1.add((void*)&h64[4], area, true);
+  }
+  if (g->pending_validate) ra1.add((void*)&h64[1], g->err.p);
+  launch_report(ra1, s);
   trace("analyze: bin count enqueued");
   if (R > 0 || g->pending_validate) CK(cudaStreamSynchronize(s));
   trace("analyze: bin count synced");
@@ -668,8 +756,11 @@ rt_status run_analysis(rt_graph* g) {
     CKR(g->keys_alt.reserve((size_t)M * 4, s));
     CKR(g->pay.reserve((size_t)M * 8, s));
     CKR(g->pay_alt.reserve((size_t)M * 8, s));
-    CKR(g->seg_b.reserve((size_t)ntiles * 4, s));
-    CKR(g->seg_e.reserve((size_t)ntiles * 4, s));
+    CKR(g->tiles.reserve((size_t)ntiles * 10, s));
+    seg_b = g->tiles.as<uint32_t>();
+    seg_e = seg_b + ntiles;
+    flags1 = reinterpret_cast<uint8_t*>(seg_e + ntiles);
+    flags2 = flags1 + ntiles;
     CKR(reserve_ws(g, radix_ws_bytes(M)));
     trace("analyze: entry buffers reserved");
     launch_bin_expand(g->rect_task.as<int32_t>(), g->lo.as<int64_t>(), g->hi.as<int64_t>(),
@@ -682,9 +773,8 @@ rt_status run_analysis(rt_graph* g) {
                                           g->ws.p, s);
     skeys = flip ? g->keys_alt.as<uint32_t>() : g->keys.as<uint32_t>();
     spay = flip ? g->pay_alt.as<uint64_t>() : g->pay.as<uint64_t>();
-    CK(cudaMemsetAsync(g->seg_b.p, 0, (size_t)ntiles * 4, s));
-    CK(cudaMemsetAsync(g->seg_e.p, 0, (size_t)ntiles * 4, s));
-    launch_segments(skeys, M, g->seg_b.as<uint32_t>(), g->seg_e.as<uint32_t>(), s);
+    CK(cudaMemsetAsync(flags1, 0, (size_t)ntiles * 2, s));
+    launch_segments(skeys, M, ntiles, seg_b, seg_e, s);
     if (prof) CK(cudaEventRecord(g->ev[EV_SORTE], s));
   } else if (prof) {
     CK(cudaEventRecord(g->ev[EV_BIN], s));
@@ -705,68 +795,119 @@ rt_status run_analysis(rt_graph* g) {
   const int sweep_blocks =
       (int)std::max<int64_t>(std::min<int64_t>((ntiles + sweep_warps - 1) / sweep_warps, (int64_t)g_dev.num_sms * 8), 1);
   const unsigned long long W = (unsigned long long)sweep_blocks * (unsigned long long)sweep_warps;
-  const unsigned long long guess = M > 0 ? std::max<unsigned long long>(2ull * M, 1ull << 16) : 0ull;
+  unsigned long long guess = M > 0 ? std::max<unsigned long long>(2ull * M, 1ull << 16) : 0ull;
   uint32_t chunk = 32;
   while (chunk < 512 && 2ull * chunk * W <= guess) chunk <<= 1;
-  unsigned long long cap = (unsigned long long)Pe + (M > 0 ? guess + W * chunk : 0ull);
+  // dense inputs (16 or more binned entries per task): the first sweep passes
+  // its pairs through a filter of about two slots per entry (2^17 .. 2^27
+  // slots, as many for each target task), so that a pair found again in other
+  // tiles is not written again; skipped when it would pass the graph's memory
+  // cap
+  int fbits = 0, fslots = 0;  // log2 of the slots, in all and per target
+  if (M >= (int64_t)16 * n) {
+    fbits = 17;
+    while (fbits < 27 && (1ll << fbits) < 2 * M) ++fbits;
+    fslots = fbits - bits_for((uint64_t)(n - 1));  // n <= M / 16 < 2^26, so at least 1
+    const size_t fbytes = (size_t)4 << fbits;
+    if (fbytes > g->pfilt.cap && t_capped && over_cap(fbytes - g->pfilt.cap)) fbits = 0;
+    else CKR(g->pfilt.reserve(fbytes, s));
+  }
+  g->pair_filter_bits = fbits;
+  // Entries that cover a fair part of their tiles are swept by windows
+  // (windows.cu): on dense inputs (with the filter), or where each tile holds so
+  // many entries that its one warp is the analysis's longest chain. Thinner
+  // entries make many class cells of a window and many walks back. Its warps
+  // take chunks of about a quarter of a warp's share, and small buffer chunks:
+  // with the filter few pairs are written, and each warp leaves holes in its
+  // last chunk.
+  const double cover = M > 0 ? (double)h64[4] / ((double)M * d.tw * d.th) : 0.0;
+  const bool by_windows = M > 0 && cover >= kWindowCover && (fbits > 0 || M >= (int64_t)kWindowTileEntries * ntiles);
+  if (by_windows && !fbits) guess *= 2;
+  int wblocks = 0, wspan = 16;
+  uint32_t wchunk = 1;
+  if (by_windows) {
+    wblocks = (int)std::min<int64_t>((M + 16 * kWindowWarps - 1) / (16 * kWindowWarps),
+                                     (int64_t)g_dev.num_sms * window_blocks_per_sm(d));
+    const int64_t ww = (int64_t)wblocks * kWindowWarps;
+    wspan = (int)std::min<int64_t>(512, (M / (4 * ww) + 15) / 16 * 16);
+    wspan = std::max(wspan, 16);
+    while (wchunk < 512 && 32ull * wchunk * (unsigned long long)ww <= guess) wchunk <<= 1;
+  }
+  unsigned long long cap =
+      (unsigned long long)Pe +
+      (M > 0 ? guess + W * chunk + (unsigned long long)wblocks * kWindowWarps * wchunk : 0ull);
   CKR(g->pairs.reserve((size_t)std::max<unsigned long long>(cap, 1) * 8, s));
   if (Pe > 0)
     launch_explicit_pairs(g->pred_off.as<int32_t>(), g->pred.as<int32_t>(), n, B, g->pairs.as<uint64_t>(), s);
   int64_t Ptot = Pe;
-  // CSR by buckets: counts [n+1], offsets [n+1], distinct counts [n+1], long
-  // rows [n+1], the longest row and the long-row count
-  CKR(g->bucket.reserve(((size_t)4 * (n + 1) + 64) * 4, s));
-  uint32_t* bcnt = g->bucket.as<uint32_t>();
-  uint32_t* boff = bcnt + (n + 1);
-  uint32_t* bucnt = boff + (n + 1);
-  uint32_t* bbig = bucnt + (n + 1);
-  uint32_t* bmax = bbig + (n + 1);
-  uint32_t* bnbig = bmax + 16;
-  const bool counted = M > 0;  // the sweep's pairs are counted per source before its sync
   h64[6] = 0;
-  if (M > 0) {
-    unsigned long long* rerun = reinterpret_cast<unsigned long long*>(g->misc.as<char>() + 128);
-    CKR(g->tflags.reserve((size_t)ntiles * 2, s));
-    uint8_t* flags1 = g->tflags.as<uint8_t>();
-    uint8_t* flags2 = flags1 + ntiles;
-    CK(cudaMemsetAsync(flags1, 0, (size_t)ntiles * 2, s));
+  if (M == 0 && Pe > 0) {  // explicit dependences alone: counted per source, one sync to learn the longest row
     h64[2] = (uint64_t)Pe;
     CK(cudaMemcpyAsync(cursor, (const void*)&h64[2], 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(tile_counter, 0, 4, s));
-    CK(cudaMemsetAsync(rerun, 0, 8, s));
-    // dense inputs (16 or more binned entries per task): the first sweep passes
-    // its pair keys through a direct-mapped filter of about one slot per entry
-    // (2^16 .. 2^26 slots), so that a pair found again in other tiles is not
-    // written again; skipped when it would pass the graph's memory cap
-    int fbits = 0;
-    if (M >= (int64_t)16 * n) {
-      fbits = 16;
-      while (fbits < 26 && (1ll << fbits) < M) ++fbits;
-      const size_t fbytes = (size_t)8 << fbits;
-      if (fbytes > g->pfilt.cap && t_capped && over_cap(fbytes - g->pfilt.cap)) {
-        fbits = 0;
-      } else {
-        CKR(g->pfilt.reserve(fbytes, s));
-        CK(cudaMemsetAsync(g->pfilt.p, 0xFF, fbytes, s));
-      }
-    }
-    g->pair_filter_bits = fbits;
-    SweepOut o{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, nullptr, flags1, rerun,
-               fbits ? g->pfilt.as<unsigned long long>() : nullptr, fbits};
-    if (prof) CK(cudaEventRecord(g->ev[EV_SW0], s));
-    launch_sweep(spay, g->seg_b.as<uint32_t>(), g->seg_e.as<uint32_t>(), d, o, sweep_blocks, s);
-    if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
-    CK(cudaGetLastError());
-    trace("analyze: sweep enqueued");
-    // the pairs per source and the longest row, before the sync the sweep
-    // needs anyway: they decide between the bucket CSR and the pair sort
-    CK(cudaMemsetAsync(bcnt, 0, (size_t)(n + 1) * 4, s));
-    CK(cudaMemsetAsync(bmax, 0, 4, s));
+    CK(cudaMemsetAsync(bcnt, 0, (size_t)n * 4, s));
     launch_bucket_count(g->pairs.as<uint64_t>(), cursor, cap, B, bcnt, n, bmax, s);
-    CK(cudaMemcpyAsync((void*)&h64[6], bmax, 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync((void*)&h64[3], cursor, 8, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync((void*)&h64[5], rerun, 8, cudaMemcpyDeviceToHost, s));
+    ReportArgs ra;
+    ra.add((void*)&h64[6], bmax);
+    launch_report(ra, s);
     CK(cudaStreamSynchronize(s));
+  }
+  const bool counted = Ptot > 0 || M > 0;  // the pairs are counted per source
+  if (M > 0) {
+    // the pairs per source and the longest row, with the sync that the sweep
+    // needs anyway: they decide between the bucket CSR and the pair sort
+    auto count_pairs = [&]() -> rt_status {
+      launch_bucket_count(g->pairs.as<uint64_t>(), cursor, cap, B, bcnt, n, bmax, s);
+      ReportArgs ra;
+      ra.add((void*)&h64[6], bmax);
+      ra.add((void*)&h64[3], cursor, true);
+      ra.add((void*)&h64[5], rerun, true);
+      ra.add((void*)&h64[7], nbail);
+      launch_report(ra, s);
+      CK(cudaGetLastError());
+      CK(cudaStreamSynchronize(s));
+      return RT_OK;
+    };
+    h64[7] = 0;
+    for (bool win = by_windows;; win = false) {
+      if (win != by_windows) {  // again from the start
+        CK(cudaMemsetAsync(flags1, 0, (size_t)ntiles * 2, s));
+        CK(cudaMemsetAsync(g->misc.p, 0, 160, s));
+        CK(cudaMemsetAsync(bcnt, 0, (size_t)n * 4, s));
+      }
+      if (Pe > 0) {
+        h64[2] = (uint64_t)Pe;
+        CK(cudaMemcpyAsync(cursor, (const void*)&h64[2], 8, cudaMemcpyHostToDevice, s));
+      }
+      if (fbits) CK(cudaMemsetAsync(g->pfilt.p, 0xFF, ((size_t)n << fslots) * 4, s));
+      SweepOut o{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, nullptr, flags1, rerun,
+                 fbits ? g->pfilt.as<uint32_t>() : nullptr, fslots};
+      if (prof) CK(cudaEventRecord(g->ev[EV_SW0], s));
+      if (win) {
+        SweepOut ow = o;
+        ow.chunk = wchunk;
+        ow.tile_counter = tile_counter + 1;
+        launch_window(spay, skeys, seg_b, seg_e, M, wspan, d, ow, flags1, nbail, wblocks, s);
+      } else {
+        launch_sweep(spay, seg_b, seg_e, d, o, sweep_blocks, s);
+      }
+      if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
+      trace("analyze: sweep enqueued");
+      CKR(count_pairs());
+      if (win && (unsigned long long)h64[3] <= cap && h64[7] != 0) {
+        // tiles that the windows left
+        o.only = flags1;
+        o.flag_out = flags2;
+        launch_sweep(spay, seg_b, seg_e, d, o, sweep_blocks, s);
+        if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
+        CK(cudaMemsetAsync(bcnt, 0, (size_t)n * 4, s));
+        CK(cudaMemsetAsync(bmax, 0, 4, s));
+        CKR(count_pairs());
+      }
+      // with windows nothing says which tiles dropped a pair past the buffer's
+      // end (more distinct pairs than twice the entries): swept again from the
+      // start by tiles, which do
+      if (!win || (unsigned long long)h64[3] <= cap) break;
+    }
     trace("analyze: sweep synced");
     Ptot = (int64_t)h64[3];
     if ((unsigned long long)Ptot > cap) {
@@ -778,44 +919,44 @@ rt_status run_analysis(rt_graph* g) {
       // the rerun writes every pair its tiles find: no filter (a pair whose
       // first write fell past the buffer's end may already sit in it)
       SweepOut o2{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, flags1, flags2, rerun, nullptr, 0};
-      launch_sweep(spay, g->seg_b.as<uint32_t>(), g->seg_e.as<uint32_t>(), d, o2, sweep_blocks, s);
+      launch_sweep(spay, seg_b, seg_e, d, o2, sweep_blocks, s);
       if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
       CK(cudaGetLastError());
       // the rerun appended pairs: count again
-      CK(cudaMemsetAsync(bcnt, 0, (size_t)(n + 1) * 4, s));
+      CK(cudaMemsetAsync(bcnt, 0, (size_t)n * 4, s));
       CK(cudaMemsetAsync(bmax, 0, 4, s));
-      launch_bucket_count(g->pairs.as<uint64_t>(), cursor, cap, B, bcnt, n, bmax, s);
-      CK(cudaMemcpyAsync((void*)&h64[6], bmax, 4, cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync((void*)&h64[3], cursor, 8, cudaMemcpyDeviceToHost, s));
-      CK(cudaStreamSynchronize(s));
+      CKR(count_pairs());
       Ptot = (int64_t)h64[3];
       if ((unsigned long long)Ptot > cap) return fail(RT_ERR_OOM, "pair buffer overflowed in the rerun");
     }
   }
-  CKR(g->pairs_alt.reserve((size_t)std::max<int64_t>(Ptot, 1) * 8, s));
   if (Ptot >= (1ll << 31) - 1) return fail(RT_ERR_OOM, "%lld candidate pairs (limit 2^31)", (long long)Ptot);
   if (prof) CK(cudaEventRecord(g->ev[EV_SWEEP], s));
   g->n_pairs = Ptot;
 
   // ---- 5: dedupe + CSR -----------------------------------------------------
   CKR(g->flags.reserve((size_t)(Ptot + 1) * 4, s));
-  CKR(g->upos.reserve((size_t)(Ptot + 1) * 4, s));
   CKR(g->col.reserve((size_t)std::max<int64_t>(Ptot, 1) * 4, s));
   CKR(g->row_ptr.reserve((size_t)(n + 1) * 4, s));
   CKR(g->indeg.reserve((size_t)n * 4, s));
   CKR(g->count.reserve((size_t)n * 4, s));
   CKR(g->rootpos.reserve((size_t)(n + 1) * 4, s));
   CKR(g->root_items.reserve((size_t)n * 8, s));
-  CKR(reserve_ws(g, std::max(radix_ws_bytes(Ptot),
-                             scan_ws_elems<uint32_t>(std::max<int64_t>(Ptot, n) + 1) * 4)));
   // rows of at most kBucketMaxRow pairs: buckets per source, each sorted and
   // deduplicated in place; longer rows: an LSD radix sort of all the pairs
   const bool by_buckets = counted && (uint32_t)(h64[6] & 0xffffffffull) <= (uint32_t)kBucketMaxRow;
+  if (by_buckets) {
+    CKR(reserve_ws(g, scan_ws_elems<uint32_t>((int64_t)n + 1) * 4));
+  } else {
+    CKR(g->pairs_alt.reserve((size_t)std::max<int64_t>(Ptot, 1) * 8, s));
+    CKR(g->upos.reserve((size_t)(Ptot + 1) * 4, s));
+    CKR(reserve_ws(g, std::max(radix_ws_bytes(Ptot), scan_ws_elems<uint32_t>(std::max<int64_t>(Ptot, n) + 1) * 4)));
+  }
   const uint32_t* n_edges_at;
   if (by_buckets) {
     launch_bucket_build(g->pairs.as<uint64_t>(), Ptot, B, n, bcnt, boff, bucnt, bbig, bnbig, g->flags.as<uint32_t>(),
                         g->row_ptr.as<uint32_t>(), g->ws.as<uint32_t>(), g->col.as<int32_t>(), g->indeg.as<int32_t>(),
-                        s);
+                        (uint32_t)(h64[6] & 0xffffffffull), s);
     if (prof) CK(cudaEventRecord(g->ev[EV_SORTP], s));
     n_edges_at = g->row_ptr.as<uint32_t>() + n;
   } else {
@@ -833,20 +974,18 @@ rt_status run_analysis(rt_graph* g) {
     n_edges_at = g->upos.as<uint32_t>() + Ptot;
   }
   g->csr_by_buckets = by_buckets;
-  launch_roots(g->indeg.as<int32_t>(), n, g->rootpos.as<uint32_t>(), s);
-  scan_exclusive<uint32_t>(g->rootpos.as<uint32_t>(), g->rootpos.as<uint32_t>(), n, g->ws.as<uint32_t>(), s);
-  launch_roots_emit(g->indeg.as<int32_t>(), g->rootpos.as<uint32_t>(), n, 0, 0, g->root_items.as<uint64_t>(),
-                    g->count.as<int32_t>(), s);
   CKR(g->adj.reserve((size_t)n * 32, s));
-  uint32_t* maxdeg = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 192);
-  CK(cudaMemsetAsync(maxdeg, 0, 4, s));
-  launch_pack_adj(g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), g->indeg.as<int32_t>(), n, g->adj.as<int4>(),
-                  maxdeg, s);
+  scan_zeros(g->indeg.as<uint32_t>(), g->rootpos.as<uint32_t>(), n, g->ws.as<uint32_t>(), s);
+  launch_finish_tasks(g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), g->indeg.as<int32_t>(),
+                      g->rootpos.as<uint32_t>(), n, g->count.as<int32_t>(), g->root_items.as<uint64_t>(),
+                      g->adj.as<int4>(), shape, s);
   g->adjx_ok = false;
   if (prof) CK(cudaEventRecord(g->ev[EV_CSR], s));
-  CK(cudaMemcpyAsync(g->hpin + 8, n_edges_at, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(g->hpin + 9, g->rootpos.as<uint32_t>() + n, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(g->hpin + 10, maxdeg, 4, cudaMemcpyDeviceToHost, s));
+  ReportArgs ra3;
+  ra3.add(g->hpin + 8, n_edges_at);
+  ra3.add(g->hpin + 9, g->rootpos.as<uint32_t>() + n);
+  for (int k = 0; k < 3; ++k) ra3.add(g->hpin + 10 + k, shape + k);
+  launch_report(ra3, s);
   trace("analyze: csr enqueued");
   CK(cudaStreamSynchronize(s));
   trace("analyze: csr synced");
@@ -854,6 +993,8 @@ rt_status run_analysis(rt_graph* g) {
   g->n_edges = g->hpin[8];
   g->n_roots = g->hpin[9];
   g->max_outdeg = (int32_t)g->hpin[10];
+  g->max_span = (int32_t)g->hpin[11];
+  g->last_root = (int32_t)g->hpin[12];
   g->analyze_timed = prof;
   return RT_OK;
 }
@@ -2020,10 +2161,14 @@ extern "C" rt_status rt_copy_csr(rt_graph_t g, int32_t* row_ptr, int32_t* col, i
     }
     return RT_OK;
   }
-  CK(cudaStreamSynchronize(g->s));
-  if (row_ptr) CK(cudaMemcpy(row_ptr, g->row_ptr.p, (size_t)(g->n + 1) * 4, cudaMemcpyDefault));
-  if (col && g->n_edges) CK(cudaMemcpy(col, g->col.p, (size_t)g->n_edges * 4, cudaMemcpyDefault));
-  if (indeg) CK(cudaMemcpy(indeg, g->indeg.p, (size_t)g->n * 4, cudaMemcpyDefault));
+  // on the legacy stream, whatever the graph's: the copies then follow all work
+  // that the caller has issued on blocking streams, as cudaMemcpy's do
+  if (g->s != nullptr) CK(cudaStreamSynchronize(g->s));
+  cudaStream_t s = cudaStreamLegacy;
+  if (row_ptr) CK(cudaMemcpyAsync(row_ptr, g->row_ptr.p, (size_t)(g->n + 1) * 4, cudaMemcpyDefault, s));
+  if (col && g->n_edges) CK(cudaMemcpyAsync(col, g->col.p, (size_t)g->n_edges * 4, cudaMemcpyDefault, s));
+  if (indeg) CK(cudaMemcpyAsync(indeg, g->indeg.p, (size_t)g->n * 4, cudaMemcpyDefault, s));
+  CK(cudaStreamSynchronize(s));
   return RT_OK;
 }
 

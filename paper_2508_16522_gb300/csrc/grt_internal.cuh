@@ -279,6 +279,9 @@ size_t scan_ws_elems(int64_t n);
 template <typename T>
 void scan_exclusive(const T* in, T* out, int64_t n, T* ws, cudaStream_t s);
 
+// out[i] = how many of in[0..i) are zero, out[n] of all
+void scan_zeros(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* ws, cudaStream_t s);
+
 size_t radix_ws_bytes(int64_t n);
 // sorts (keys, vals) by key bits [0, nbits); ping-pongs between the two
 // buffers; returns 1 if the result is in the *_alt buffers
@@ -307,12 +310,13 @@ void launch_widen_bounds(const int32_t* lo32, const int32_t* hi32, int64_t m, in
 // moves it into the graph's band (box: int64 [G][3][ndim] = lo, hi, shift)
 void launch_band_place(const int32_t* req_off, int32_t n, const int32_t* task_first, int32_t G, const int64_t* box,
                        int D, int64_t* lo, int64_t* hi, int64_t R, uint32_t* err, cudaStream_t s);
-void launch_bin_count(const int32_t* req_off, int32_t n, const int64_t* lo, const int64_t* hi,
-                      int64_t R, AnalysisDims d, int32_t* rect_task, uint64_t* cnt, cudaStream_t s);
+void launch_bin_count(const int32_t* req_off, int32_t n, int64_t R, const int64_t* lo, const int64_t* hi,
+                      AnalysisDims d, int32_t* rect_task, uint64_t* cnt, unsigned long long* area,
+                      uint32_t* zero, cudaStream_t s);
 void launch_bin_expand(const int32_t* rect_task, const int64_t* lo, const int64_t* hi,
                        const uint8_t* priv, int64_t R, const uint64_t* off, AnalysisDims d,
                        uint32_t* keys, uint64_t* payload, cudaStream_t s);
-void launch_segments(const uint32_t* keys, int64_t M, uint32_t* seg_begin, uint32_t* seg_end,
+void launch_segments(const uint32_t* keys, int64_t M, int64_t ntiles, uint32_t* seg_begin, uint32_t* seg_end,
                      cudaStream_t s);
 struct SweepOut {
   uint64_t* pairs;
@@ -324,18 +328,25 @@ struct SweepOut {
   const uint8_t* only;       // non-null: sweep only the tiles flagged here
   uint8_t* flag_out;         // non-null: flag the tiles that dropped a pair
   unsigned long long* rerun; // pairs emitted by the tiles that dropped one
-  // optional, dense inputs: a direct-mapped table of 2^filt_bits pair keys
-  // (kEmpty64 = free) through which the flushes of a first sweep pass their
-  // keys; a key found there was emitted before and is not written again. Lossy
-  // only towards keeping duplicates (a slot keeps the last key that reached
-  // it); never set for a rerun, whose tiles must write every pair they find.
-  unsigned long long* filt;
+  // optional, dense inputs: the pair filter (pairs.cuh), 2^filt_bits slots for
+  // each target task; never set for a rerun, whose tiles must write every pair
+  // they find
+  uint32_t* filt;
   int filt_bits;
 };
 int sweep_warps_per_block(int tw, int th);
 size_t sweep_smem_bytes(int tw, int th, int warps);
 void launch_sweep(const uint64_t* payload, const uint32_t* seg_begin, const uint32_t* seg_end,
                   AnalysisDims d, SweepOut o, int blocks, cudaStream_t s);
+// the sweep by windows (windows.cu; the pair filter is optional): chunks of
+// `span` candidates (a multiple of 16) are handed to the warps of `blocks`
+// blocks by o.tile_counter; tiles it leaves to launch_sweep are flagged in bail
+// and counted in *nbail
+constexpr int kWindowWarps = 8;  // per block
+int window_blocks_per_sm(const AnalysisDims& d);
+void launch_window(const uint64_t* payload, const uint32_t* keys, const uint32_t* seg_begin, const uint32_t* seg_end,
+                   int64_t M, int span, AnalysisDims d, SweepOut o, uint8_t* bail, uint32_t* nbail, int blocks,
+                   cudaStream_t s);
 void launch_explicit_pairs(const int32_t* pred_off, const int32_t* pred, int32_t n, int key_bits,
                            uint64_t* pairs, cudaStream_t s);
 void launch_unique_flags(const uint64_t* keys, int64_t P, uint32_t* flags, cudaStream_t s);
@@ -351,10 +362,26 @@ void launch_bucket_count(const uint64_t* pairs, const unsigned long long* cursor
                          int key_bits, uint32_t* cnt, int32_t n, uint32_t* maxrow, cudaStream_t s);
 void launch_bucket_build(const uint64_t* pairs, int64_t P, int key_bits, int32_t n, uint32_t* cnt, uint32_t* off,
                          uint32_t* ucnt, uint32_t* big, uint32_t* nbig, uint32_t* bucket, uint32_t* row_ptr,
-                         uint32_t* scan_ws, int32_t* col, int32_t* indeg, cudaStream_t s);
-void launch_roots(const int32_t* indeg, int32_t n, uint32_t* flags, cudaStream_t s);
-void launch_roots_emit(const int32_t* indeg, const uint32_t* pos, int32_t n, int32_t task_base,
-                       int32_t graph, uint64_t* root_items, int32_t* count, cudaStream_t s);
+                         uint32_t* scan_ws, int32_t* col, int32_t* indeg, uint32_t maxrow, cudaStream_t s);
+// shape[0..2], zeroed by the caller: the largest out-degree, the longest edge
+// (target - source) and the last root
+void launch_finish_tasks(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, const uint32_t* pos,
+                         int32_t n, int32_t* count, uint64_t* root_items, int4* adj, uint32_t* shape,
+                         cudaStream_t s);
+// words copied to pinned host memory by one kernel (at most kReportMax)
+constexpr int kReportMax = 16;
+struct ReportArgs {
+  const void* src[kReportMax];
+  void* dst[kReportMax];
+  uint8_t wide[kReportMax];  // 8 bytes, else 4
+  int n = 0;
+  void add(void* to, const void* from, bool w = false) {
+    dst[n] = to;
+    src[n] = from;
+    wide[n++] = w;
+  }
+};
+void launch_report(const ReportArgs& a, cudaStream_t s);
 
 // maxdeg (nullable, zeroed by the caller): receives the largest out-degree
 void launch_pack_adj(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int64_t n, int4* adj,
@@ -383,6 +410,7 @@ void preload_static();
 void preload_stitch();
 void preload_analysis();
 void preload_sweep();
+void preload_window();
 void preload_exec();
 void preload_serve();
 // the event-based executor (rt_execute_events)

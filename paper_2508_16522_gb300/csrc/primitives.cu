@@ -4,6 +4,8 @@
 // block totals scanned recursively. out[n] receives the total, so arrays are
 // sized n+1; in == out is allowed.
 //
+// Up to kScanOne items one block does it all.
+//
 // Radix sort: 8-bit digits, least significant first. Per pass: a per-block
 // digit histogram, an exclusive scan of the digit-major histogram matrix, and
 // a scatter whose in-block ranks are computed warp by warp with match_any (so
@@ -51,7 +53,13 @@ __device__ T block_exclusive_sum(T v, T* warp_tot, T* block_total) {
   return incl - v + warp_tot[warp];
 }
 
-template <typename T>
+// what a scan adds up: the array's values, or (ZERO) one per zero
+template <bool ZERO, typename T>
+__device__ __forceinline__ T scan_value(T v) {
+  return ZERO ? T(v == T(0)) : v;
+}
+
+template <typename T, bool ZERO>
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const T* in, int64_t n, T* partial) {
   __shared__ T warp_tot[32];
   __shared__ T tot;
@@ -60,13 +68,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const T* in, int64
 #pragma unroll
   for (int j = 0; j < kScanItems; ++j) {
     int64_t k = base + j * kScanThreads + threadIdx.x;  // coalesced
-    if (k < n) s += in[k];
+    if (k < n) s += scan_value<ZERO>(in[k]);
   }
   (void)block_exclusive_sum<T>(s, warp_tot, &tot);
   if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
-template <typename T>
+template <typename T, bool ZERO>
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const T* in, T* out, int64_t n,
                                                            const T* block_base) {
   __shared__ T stage[kScanTile];
@@ -77,7 +85,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const T* in, T* out,
 #pragma unroll
   for (int j = 0; j < kScanItems; ++j) {
     int64_t k = base + j * kScanThreads + threadIdx.x;
-    stage[j * kScanThreads + threadIdx.x] = k < n ? in[k] : T(0);
+    stage[j * kScanThreads + threadIdx.x] = k < n ? scan_value<ZERO>(in[k]) : T(0);
   }
   __syncthreads();
   T v[kScanItems];
@@ -106,6 +114,81 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const T* in, T* out,
     out[n] = total;
   }
 }
+// A short scan in one block: kOneTile items a step, staged in shared memory so
+// that loads and stores coalesce, the next step's loads in flight meanwhile and
+// the running total carried along. Up to kScanOne items it beats the three
+// launches of reduce, scan of the totals and down-sweep (about 3 us each on the
+// device and as much on the host). 512 threads: a block of 1024 at 52 registers
+// would not fit an SM beside a resident serving kernel, and never start.
+constexpr int kOneThreads = 512;
+constexpr int kOneItems = 8;
+constexpr int kOneTile = kOneThreads * kOneItems;
+constexpr int kScanOne = 6 * kOneTile;
+
+template <typename T, bool ZERO>
+__global__ void __launch_bounds__(kOneThreads) k_scan_one(const T* in, T* out, int32_t n) {
+  constexpr int kWarps = kOneThreads / 32;
+  __shared__ T stage[kOneTile];
+  __shared__ T wtot[kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  T next[kOneItems];
+#pragma unroll
+  for (int j = 0; j < kOneItems; ++j) {
+    const int32_t k = j * kOneThreads + tid;
+    next[j] = k < n ? scan_value<ZERO>(in[k]) : T(0);
+  }
+  T carry = 0;
+  for (int32_t base = 0; base < n; base += kOneTile) {
+#pragma unroll
+    for (int j = 0; j < kOneItems; ++j) stage[j * kOneThreads + tid] = next[j];
+    __syncthreads();
+    // in place is allowed: this step's items have been read, none written yet
+    if (base + kOneTile < n) {
+#pragma unroll
+      for (int j = 0; j < kOneItems; ++j) {
+        const int32_t k = base + kOneTile + j * kOneThreads + tid;
+        next[j] = k < n ? scan_value<ZERO>(in[k]) : T(0);
+      }
+    }
+    T v[kOneItems];
+    T sum = 0;
+#pragma unroll
+    for (int j = 0; j < kOneItems; ++j) {
+      v[j] = stage[tid * kOneItems + j];
+      sum += v[j];
+    }
+    T incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    T wi = lane < kWarps ? wtot[lane] : T(0);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T y = __shfl_up_sync(0xffffffffu, wi, o);
+      if (lane >= o) wi += y;
+    }
+    const T before = __shfl_sync(0xffffffffu, wi, warp > 0 ? warp - 1 : 0);
+    T run = carry + (warp > 0 ? before : T(0)) + incl - sum;
+    carry += __shfl_sync(0xffffffffu, wi, 31);
+#pragma unroll
+    for (int j = 0; j < kOneItems; ++j) {
+      stage[tid * kOneItems + j] = run;
+      run += v[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kOneItems; ++j) {
+      const int32_t k = base + j * kOneThreads + tid;
+      if (k < n) out[k] = stage[j * kOneThreads + tid];
+    }
+    __syncthreads();
+  }
+  if (tid == 0) out[n] = carry;
+}
 }  // namespace
 
 template <typename T>
@@ -119,25 +202,39 @@ size_t scan_ws_elems(int64_t n) {
   return total + 1;
 }
 
-template <typename T>
-void scan_exclusive(const T* in, T* out, int64_t n, T* ws, cudaStream_t s) {
+namespace {
+template <typename T, bool ZERO>
+void scan_any(const T* in, T* out, int64_t n, T* ws, cudaStream_t s) {
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(T), s);
     return;
   }
-  int64_t nb = (n + kScanTile - 1) / kScanTile;
-  if (nb == 1) {
-    count_launch();
-    k_scan_down<T><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr);
+  count_launch();
+  if (n <= kScanTile) {
+    k_scan_down<T, ZERO><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr);
     return;
   }
+  if (n <= kScanOne) {
+    k_scan_one<T, ZERO><<<1, kOneThreads, 0, s>>>(in, out, (int32_t)n);
+    return;
+  }
+  const int64_t nb = (n + kScanTile - 1) / kScanTile;
   T* part = ws;
   T* part_scan = ws + nb;
+  k_scan_reduce<T, ZERO><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, part);
+  scan_any<T, false>(part, part_scan, nb, ws + 2 * nb + 1, s);
   count_launch();
-  k_scan_reduce<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, part);
-  scan_exclusive<T>(part, part_scan, nb, ws + 2 * nb + 1, s);
-  count_launch();
-  k_scan_down<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, part_scan);
+  k_scan_down<T, ZERO><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, part_scan);
+}
+}  // namespace
+
+template <typename T>
+void scan_exclusive(const T* in, T* out, int64_t n, T* ws, cudaStream_t s) {
+  scan_any<T, false>(in, out, n, ws, s);
+}
+
+void scan_zeros(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* ws, cudaStream_t s) {
+  scan_any<uint32_t, true>(in, out, n, ws, s);
 }
 
 template size_t scan_ws_elems<uint32_t>(int64_t);
@@ -359,10 +456,15 @@ template int radix_sort<uint64_t>(uint64_t*, uint64_t*, uint64_t*, uint64_t*, in
 // kernel, e.g. the serving kernel).
 void preload_primitives() {
   cudaFuncAttributes a;
-  cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t>);
-  cudaFuncGetAttributes(&a, k_scan_reduce<uint64_t>);
-  cudaFuncGetAttributes(&a, k_scan_down<uint32_t>);
-  cudaFuncGetAttributes(&a, k_scan_down<uint64_t>);
+  cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t, false>);
+  cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t, true>);
+  cudaFuncGetAttributes(&a, k_scan_reduce<uint64_t, false>);
+  cudaFuncGetAttributes(&a, k_scan_down<uint32_t, false>);
+  cudaFuncGetAttributes(&a, k_scan_down<uint32_t, true>);
+  cudaFuncGetAttributes(&a, k_scan_down<uint64_t, false>);
+  cudaFuncGetAttributes(&a, k_scan_one<uint32_t, false>);
+  cudaFuncGetAttributes(&a, k_scan_one<uint32_t, true>);
+  cudaFuncGetAttributes(&a, k_scan_one<uint64_t, false>);
   cudaFuncGetAttributes(&a, k_radix_hist<uint32_t>);
   cudaFuncGetAttributes(&a, k_radix_hist<uint64_t>);
   cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, true>);
@@ -375,6 +477,7 @@ void preload_all() {
   preload_primitives();
   preload_analysis();
   preload_sweep();
+  preload_window();
   preload_exec();
   preload_serve();
   preload_events();

@@ -49,15 +49,15 @@
 // past the buffer's end is flagged with its pair count, for a rerun of just the
 // flagged tiles.
 // On dense inputs a pair is found again in every tile where the two tasks'
-// rectangles meet; there the first sweep passes each flushed key through a
-// direct-mapped table in global memory (one atomic exchange per key) and does
-// not write a key the table already held. The table is lossy only towards
-// keeping duplicates, which the CSR stage removes anyway; the rerun of flagged
-// tiles sweeps without it.
+// rectangles meet; there the first sweep passes each flushed pair through a
+// filter in global memory (pairs.cuh) and does not write one it already held;
+// the rerun of flagged tiles sweeps without it. Dense inputs are mostly swept by
+// windows (windows.cu); this sweep takes the tiles that leaves.
 #include <map>
 #include <mutex>
 
 #include "grt_internal.cuh"
+#include "pairs.cuh"
 
 namespace grt {
 
@@ -192,19 +192,6 @@ __device__ __forceinline__ void put_pair(const WarpSmem& w, const SweepOut& o, u
   }
 }
 
-__device__ __forceinline__ uint64_t pair_key(int src, int dst, int key_bits) {
-  return ((uint64_t)(uint32_t)src << key_bits) | (uint32_t)dst;
-}
-
-// the pair-key filter of dense inputs: the key takes its slot (multiplicative
-// hashing by the 64-bit golden ratio); false when the slot already held it,
-// i.e. some tile emitted this pair before (its write stands, or its tile was
-// flagged for the rerun, which sweeps without the filter)
-__device__ __forceinline__ bool filt_fresh(const SweepOut& o, uint64_t key) {
-  const uint64_t h = (key * 0x9E3779B97F4A7C15ull) >> (64 - o.filt_bits);
-  return atomicExch(o.filt + h, (unsigned long long)key) != (unsigned long long)key;
-}
-
 __device__ __forceinline__ uint64_t entry_at(const Ctx& x, const WarpSmem& w, int p) {
   int q = p - x.pos;
   return (q >= 0 && q < x.cnt) ? w.stage[q] : __ldg(x.L + p);
@@ -242,38 +229,6 @@ __device__ void hash_insert(const WarpSmem& w, const SweepOut& o, int src, int d
 __device__ __forceinline__ void warp_insert(const WarpSmem& w, const SweepOut& o, int src, int dst) {
   unsigned peers = __match_any_sync(kFull, src);
   if (src >= 0 && (peers & lanemask_lt()) == 0) hash_insert(w, o, src, dst);
-}
-
-// Where `need` pairs of one flush go: the first `split` fill the rest of the
-// warp's current chunk (from `a`), the others start a fresh contiguous run of
-// chunks (at `b`). Only a warp's last, partly used chunk is ever left with
-// holes, so the cursor exceeds the pairs written by less than one chunk per
-// warp (convergent).
-struct PairDst {
-  unsigned long long a, b;
-  uint32_t split;
-};
-
-__device__ PairDst reserve_pairs(Ctx& x, const SweepOut& o, uint32_t need) {
-  PairDst d{x.chunk_base, 0ull, need};
-  if (x.chunk_left >= need) {
-    x.chunk_base += need;
-    x.chunk_left -= need;
-    return d;
-  }
-  d.split = x.chunk_left;
-  const uint32_t rest = need - x.chunk_left;
-  const uint32_t k = (rest + o.chunk - 1) / o.chunk;
-  unsigned long long nb = 0;
-  if (x.lane == 0) nb = atomicAdd(o.cursor, (unsigned long long)k * o.chunk);
-  d.b = __shfl_sync(kFull, nb, 0);
-  x.chunk_base = d.b + rest;
-  x.chunk_left = k * o.chunk - rest;
-  return d;
-}
-
-__device__ __forceinline__ unsigned long long pair_pos(const PairDst& d, uint32_t i) {
-  return i < d.split ? d.a + i : d.b + (i - d.split);
 }
 
 // writes the task's distinct predecessors found in this tile (convergent)
