@@ -277,8 +277,14 @@ rt_status rt_execute_kernels(rt_graph_t g, int32_t mode, int32_t iters, int32_t 
  * persistent blocks, warps per block (1..8), how many published ring slots a
  * warp claims at once (1..32; default 8) and how many newly ready successors a
  * warp keeps for its own next batch instead of publishing them (0..64). These
- * are the autotuner's knobs; results do not depend on them. The event-based
- * executor (rt_execute_events) takes the same claim width. */
+ * are the autotuner's knobs; results do not depend on them. With neither blocks
+ * nor warps given, the library also picks the executor under RT_EXEC_RING: a
+ * graph of up to 65534 tasks, or one of any size whose edges span few tasks of
+ * program order, runs inside one block (rt_graph_stats then reports 1 block),
+ * and a larger one whose edges and roots stay within 16384 tasks of program
+ * order over owned chunks; runs with tickets, a held task or the CHECK body
+ * keep the ring. rt_execute_stitched picks owned chunks by the same rule. The
+ * event-based executor (rt_execute_events) takes the same claim width. */
 rt_status rt_graph_exec_config(rt_graph_t g, int32_t blocks, int32_t warps, int32_t claim, int32_t keep);
 
 /* How rt_execute / rt_replay find ready tasks (Algorithm 1's EXECUTE_OP):
@@ -373,7 +379,9 @@ rt_status rt_batch_capture(const rt_graph_desc* desc, int32_t n_graphs, const in
 /* One persistent launch in which every graph of the batch runs `replays` times
  * (1..4096); graph g's replay r+1 starts as soon as its replay r has finished,
  * independently of the other graphs. exec_blocks/exec_warps/claim/keep (0 =
- * default) are the launch shape of rt_graph_exec_config. The batch's counters
+ * default) are the launch shape of rt_graph_exec_config; a batch whose graphs
+ * all fit (as one graph does there) runs each of them inside one block, several
+ * to an SM, whatever the number of blocks and warps given. The batch's counters
  * are reset at the start of every launch. The launch {counter reset, seed,
  * executor, status read-back} is captured as a CUDA graph once per launch
  * shape and relaunched from it afterwards (the first launch of a new or

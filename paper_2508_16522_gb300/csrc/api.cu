@@ -240,6 +240,15 @@ struct rt_batch {
   int policy = RT_EXEC_RING;
   DevBuf task_graph, adjx, scratch;
   bool owned_ready = false;
+  // a batch whose graphs all fit runs each inside one block: four lists of
+  // graphs and every graph's longest edge (host and, from the first such launch
+  // on, device), the queues' spill, the stream of the small blocks
+  bool blocks_fit = false, graph_next = false;
+  int32_t n_list[4] = {0, 0, 0, 0}, max_queue_n = 0;
+  std::vector<int32_t> plan;
+  DevBuf order, spill;
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   int32_t max_outdeg = 0;
 };
 
@@ -1045,25 +1054,73 @@ constexpr int32_t kMaxKernelTasks = 1 << 17;  // rt_execute_kernels: one event p
 constexpr int kKernelStreams = 16;     // hpin word receiving the executor status
 constexpr int kCountersByte = 512;  // hpin byte offset of the executor's diagnostic counters
 
+// Ready successors a warp of a block keeps: a batch of tasks while their edges
+// fit a few decrements per lane (640 mixed Task Bench graphs: 15.1 ms with 32,
+// 25 with 8), few where a task has many (43 captured requests of 19 edges a
+// task: 3.6 ms with 1, 5.2 with 32): a kept task's edges delay the next ones.
+int block_keep(int64_t edges, int64_t tasks) {
+  const int64_t deg = tasks > 0 ? edges / tasks : 0;
+  return deg < 6 ? 32 : (int)std::max<int64_t>(1, 24 / deg);
+}
+
+// ... and takes from the queue at once: one task of many edges, whose row the
+// warp then shares
+int block_claim(int64_t edges, int64_t tasks) { return tasks > 0 && edges / tasks >= 6 ? 1 : 32; }
+
+// the owned executors' extension records, if some task has more successors
+// than its trigger record holds
+rt_status ensure_adjx(rt_graph* g) {
+  if (g->max_outdeg <= kAdjInline || g->adjx_ok) return RT_OK;
+  CKR(g->adjx.reserve((size_t)g->n * 32, g->s));
+  launch_pack_adjx(g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), g->n, g->adjx.as<int4>(), g->s);
+  g->adjx_ok = true;
+  return RT_OK;
+}
+
+// Warps for the owned chunks of a graph (or of one replay of a trace) whose
+// longest edge spans `span` tasks of program order and whose last task without
+// predecessors is `last_root`; 0: not suited. W warps hold a window of 32 W
+// consecutive tasks, so a chain that starts late in program order waits for
+// what comes before it: with every edge and every start inside the window the
+// front of ready tasks is inside it too. A level-ordered graph of width w has
+// edges of w to 2 w. (Random fan-in, 1024 x 300: 0.38 ms, by the ring 1.26 at its
+// default shape and 0.81 at its best; 20 stitched replays of a 1024 x 100
+// stencil 0.23 ms, 1.85 and 0.58. More than one step's warps gained nothing.)
+constexpr int kOwnedMin = 32, kOwnedMax = 256;
+int owned_warps_for(int32_t span, int32_t last_root) {
+  int w = kOwnedMin;
+  while (w < kOwnedMax && 64 * w < span) w *= 2;
+  return span <= 64 * w && last_root < 64 * w ? w : 0;
+}
+
 rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ring_clear) {
   cudaStream_t s = g->s;
-  const bool owned = g->cfg_policy == RT_EXEC_OWNED;  // no ring: every warp polls the countdowns it owns
+  bool owned = g->cfg_policy == RT_EXEC_OWNED;  // no ring: every warp polls the countdowns it owns
   const uint64_t cap = (uint64_t)g->n * (uint64_t)replays + 64;
   if (cap >= 0xFFFFFFF0ull) return fail(RT_ERR_INVALID, "tasks x replays must stay below 2^32 per launch");
-  const bool grow = !owned && (cap * 8 > g->ring.cap || !g->ring.p);
+  // a small graph whose launch shape is left to the library runs inside one
+  // block (not a run that records tickets, holds a task or must reset counters)
+  const bool free_shape = !owned && g->cfg_blocks == 0 && g->cfg_warps == 0 && !(g->desc.flags & RT_GRAPH_TICKETS) &&
+                          !g->dirty && g->hold_task < 0;
+  const bool window = free_shape && block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters);
+  const bool block =
+      window || (free_shape && block_exec_fits(g->n, g->n_roots, g->desc.body, g->desc.spin_iters));
+  // a larger one whose program order follows its dependences closely runs over
+  // owned chunks; a CHECK body's time is its rectangles' cells, which the ring
+  // spreads better
+  const int own_warps = owned_warps_for(g->max_span, g->last_root);
+  const bool auto_owned = free_shape && !block && own_warps > 0 && g->desc.body != RT_BODY_CHECK;
+  if (auto_owned) owned = true;
+  const bool grow = !owned && !block && (cap * 8 > g->ring.cap || !g->ring.p);
   if (grow) {
     drop_replay_graph(g);
     CKR(g->ring.reserve((size_t)cap * 8, s));
   }
-  *ring_clear = owned ? 0 : ((grow || g->dirty) ? (int64_t)(g->ring.cap / 8) : 0);
+  *ring_clear = owned || block ? 0 : ((grow || g->dirty) ? (int64_t)(g->ring.cap / 8) : 0);
   CKR(g->ctrl.reserve(sizeof(ExecCtrl), s));
   CKR(g->done_g.reserve(64, s));
-  const bool wide = owned && g->max_outdeg > kAdjInline;  // some task has successors past its record
-  if (wide && !g->adjx_ok) {
-    CKR(g->adjx.reserve((size_t)g->n * 32, s));
-    launch_pack_adjx(g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), g->n, g->adjx.as<int4>(), s);
-    g->adjx_ok = true;
-  }
+  const bool wide = (owned || window) && g->max_outdeg > kAdjInline;  // some task has successors past its record
+  if (wide) CKR(ensure_adjx(g));
   if (!g->gtable.p) {
     CKR(g->gtable.reserve(sizeof(ExecGraph), s));
   }
@@ -1111,29 +1168,59 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   p.replays = replays;
   p.graphs_target = 1;
   p.timeout_ns = g->desc.timeout_ns;
-  p.claim = g->cfg_claim > 0 ? g->cfg_claim : (owned ? 1 : 8);  // owned: chunks a warp holds at once
-  p.keep = g->cfg_keep > 0 ? g->cfg_keep : 16;
+  p.claim = g->cfg_claim > 0 ? g->cfg_claim : (owned ? 1 : (block ? block_claim(g->n_edges, g->n) : 8));  // owned: chunks a warp holds at once
+  p.keep = g->cfg_keep > 0 ? g->cfg_keep : (block ? block_keep(g->n_edges, g->n) : 16);
+  p.block_n = block ? g->n : 0;
+  p.window = window;
+  p.span = g->max_span;
+  if (block && !window) CKR(g->spill.reserve((size_t)g->n * 2, s));
   p.tickets = (g->desc.flags & RT_GRAPH_TICKETS) ? g->tickets.as<int32_t>() : nullptr;
   p.total_roots = owned ? 0 : (int32_t)g->n_roots;
   p.need_fence = g->desc.body == RT_BODY_COUNTER || g->desc.body == RT_BODY_CHECK;
-  p.policy = g->cfg_policy;
+  p.policy = owned ? RT_EXEC_OWNED : RT_EXEC_RING;
+  if (auto_owned) {
+    p.claim = 1;
+    p.auto_warps = own_warps;
+  }
   *out = p;
   return RT_OK;
+}
+
+// the executor's status and diagnostic counters to pinned host memory
+void report_exec(const ExecParams& p, uint32_t* status, uint32_t* hpin, cudaStream_t s) {
+  ReportArgs ra;
+  ra.add(status, &p.ctrl->status);
+  for (int k = 0; k < kCntCount; ++k)
+    ra.add(reinterpret_cast<char*>(hpin) + kCountersByte + 8 * k, &p.ctrl->counters[k], true);
+  launch_report(ra, s);
 }
 
 rt_status enqueue_run(rt_graph* g, const ExecParams& p, int64_t ring_clear, cudaStream_t s, bool timed) {
   if (g->dirty || g->hold_task >= 0)
     launch_reset_counts(g->count.as<int32_t>(), g->indeg.as<int32_t>(), g->n, g->hold_task, g->hold_extra, s);
   if (timed) CK(cudaEventRecord(g->ev[EV_X0], s));
+  if (p.block_n > 0) {  // initialises itself and writes its status to the host
+    if (timed) CK(cudaEventRecord(g->ev[EV_XK0], s));
+    BlockArgs ba{};
+    ba.spill = g->spill.as<uint16_t>();
+    ba.n_order = 1;
+    ba.status_out = g->hpin + kStatusWord;
+    ba.counters_out = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(g->hpin) + kCountersByte);
+    ba.span = p.span;
+    if (p.window) launch_exec_window(p, ba, 1, p.span <= kSmallSpan, s);
+    else launch_exec_block(p, ba, p.block_n, 1, false, s);
+    if (timed) CK(cudaEventRecord(g->ev[EV_XK1], s));
+    g->exec_blocks = 1;
+    g->exec_warps = p.window && p.span <= kSmallSpan ? block_small_warps() : block_exec_warps();
+    return RT_OK;
+  }
   launch_seed(p, ring_clear, s);
-  const int warps = g->cfg_warps > 0 ? g->cfg_warps : 2;
-  const int blocks = g->cfg_blocks > 0 ? g->cfg_blocks : g_dev.num_sms;
+  const int warps = p.auto_warps > 0 ? 1 : (g->cfg_warps > 0 ? g->cfg_warps : 2);
+  const int blocks = p.auto_warps > 0 ? p.auto_warps : (g->cfg_blocks > 0 ? g->cfg_blocks : g_dev.num_sms);
   if (timed) CK(cudaEventRecord(g->ev[EV_XK0], s));
   launch_exec(p, blocks, warps, s);
   if (timed) CK(cudaEventRecord(g->ev[EV_XK1], s));
-  CK(cudaMemcpyAsync(g->hpin + kStatusWord, &p.ctrl->status, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(reinterpret_cast<char*>(g->hpin) + kCountersByte, p.ctrl->counters,
-                     kCntCount * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  report_exec(p, g->hpin + kStatusWord, g->hpin, s);
   g->exec_blocks = blocks;
   g->exec_warps = warps;
   return RT_OK;
@@ -1438,11 +1525,14 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   CKR(ensure_pinned(g));
   cudaStream_t s = g->s;
   // the second copy must repeat the first
-  CKR(g->st_err.reserve(4, s));
-  CK(cudaMemsetAsync(g->st_err.p, 0, 4, s));
+  CKR(g->st_err.reserve(256, s));
+  CK(cudaMemsetAsync(g->st_err.p, 0, 12, s));
   launch_stitch_check(g->req_off.as<int32_t>(), g->lo.as<int64_t>(), g->hi.as<int64_t>(), g->priv.as<uint8_t>(),
-                      g->dims.ndim, g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), n, g->st_err.as<uint32_t>(), s);
-  CK(cudaMemcpyAsync(g->hpin + kStatusWord, g->st_err.p, 4, cudaMemcpyDeviceToHost, s));
+                      g->dims.ndim, g->row_ptr.as<int32_t>(), g->col.as<int32_t>(), g->indeg.as<int32_t>(), n,
+                      g->st_err.as<uint32_t>(), s);
+  ReportArgs rc;
+  for (int k = 0; k < 3; ++k) rc.add(g->hpin + kStatusWord + k, g->st_err.as<uint32_t>() + k);
+  launch_report(rc, s);
   CK(cudaStreamSynchronize(s));
   CK(cudaGetLastError());
   if (g->hpin[kStatusWord] & 1u)
@@ -1450,16 +1540,18 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   if (g->hpin[kStatusWord] & 2u)
     return fail(RT_ERR_INVALID, "the graph's two halves have different internal edges");
   const bool tickets = (g->desc.flags & RT_GRAPH_TICKETS) != 0;
+  const int wr = owned_warps_for((int32_t)g->hpin[kStatusWord + 1], (int32_t)g->hpin[kStatusWord + 2]);
+  const bool owned = wr > 0 && !tickets && body != RT_BODY_CHECK && g->cfg_blocks == 0 && g->cfg_warps == 0;
   CKR(g->st_count.reserve((size_t)total * 4, s));
-  CKR(g->st_ring.reserve((size_t)total * 8, s));
+  if (!owned) CKR(g->st_ring.reserve((size_t)total * 8, s));
   CKR(g->st_ctrl.reserve(sizeof(ExecCtrl), s));
   if (tickets) CKR(g->st_tickets.reserve((size_t)total * 8, s));
   StitchParams p{};
   p.adj = g->adj.as<int4>();
   p.col = g->col.as<int32_t>();
   p.count = g->st_count.as<int32_t>();
-  p.ring = g->st_ring.as<uint64_t>();
-  p.ring_cap = (uint32_t)total;
+  p.ring = owned ? nullptr : g->st_ring.as<uint64_t>();
+  p.ring_cap = owned ? 0u : (uint32_t)total;
   p.n = n;
   p.R = replays;
   p.claim = std::min(g->cfg_claim > 0 ? g->cfg_claim : 8, 32);
@@ -1486,12 +1578,20 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   p.timeout_ns = g->desc.timeout_ns > 0 ? g->desc.timeout_ns : 2000000000ll;
   const int warps = std::min(g->cfg_warps > 0 ? g->cfg_warps : 2, 8);
   const int blocks = g->cfg_blocks > 0 ? g->cfg_blocks : g_dev.num_sms;
-  CK(cudaMemsetAsync(p.ring, 0xFF, (size_t)total * 8, s));
+  if (!owned) CK(cudaMemsetAsync(p.ring, 0xFF, (size_t)total * 8, s));
   CK(cudaMemsetAsync(p.ctrl, 0, sizeof(ExecCtrl), s));
+  if (owned) CKR(ensure_adjx(g));
   CKR(graph_events(g));
   CK(cudaEventRecord(g->ev[EV_E0], s));
-  launch_stitch(p, g->indeg.as<int32_t>(), g->root_items.as<uint64_t>(), g->rootpos.as<uint32_t>(), blocks, warps,
-                tickets, body == RT_BODY_CHECK || body == RT_BODY_COUNTER, s);
+  if (owned) {
+    // each replay its own warps, up to two warps a scheduler
+    const int groups = std::max(1, std::min(replays, g_dev.num_sms * 8 / wr));
+    launch_stitch_owned(p, g->max_outdeg > kAdjInline ? g->adjx.as<int4>() : nullptr, g->indeg.as<int32_t>(), wr, groups,
+                        body == RT_BODY_COUNTER, s);
+  } else {
+    launch_stitch(p, g->indeg.as<int32_t>(), g->root_items.as<uint64_t>(), g->rootpos.as<uint32_t>(), blocks, warps,
+                  tickets, body == RT_BODY_CHECK || body == RT_BODY_COUNTER, s);
+  }
   CK(cudaEventRecord(g->ev[EV_E1], s));
   CK(cudaMemcpyAsync(g->hpin + kStatusWord, &p.ctrl->status, 4, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
@@ -1626,6 +1726,57 @@ int exec_bps_for(int warps) {
 }
 }  // namespace
 
+namespace {
+// The end of a batch's assembly: its table on the device, every graph's shape
+// (longest edge, last root, largest out-degree) back, one sync, and the plan of
+// its launches: each graph inside one block if all of them fit, in four lists,
+// largest first: counters for a window or for all tasks, blocks of 16 or 4 warps.
+rt_status finish_batch(rt_batch* b, const std::vector<ExecGraph>& table) {
+  cudaStream_t s = b->s;
+  const size_t G = table.size();
+  std::vector<uint32_t> shape(3 * G);
+  DevBuf dshape;
+  CKR(dshape.reserve(3 * G * 4, s));
+  cudaError_t e = cudaMemcpyAsync(b->gtable.p, table.data(), G * sizeof(ExecGraph), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dshape.p, 0, 3 * G * 4, s);
+  launch_batch_shape(b->gtable.as<ExecGraph>(), (int32_t)G, b->row_ptr.as<int32_t>(), b->col.as<int32_t>(),
+                     b->indeg.as<int32_t>(), dshape.as<uint32_t>(), s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(shape.data(), dshape.p, 3 * G * 4, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  dshape.release(s);
+  if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(RT_ERR_CUDA, "batch assembly failed");
+  std::vector<int32_t> by_size;
+  for (size_t k = 0; k < G; ++k)
+    if (table[k].n_tasks > 0) by_size.push_back((int32_t)k);
+  std::stable_sort(by_size.begin(), by_size.end(), [&](int32_t x, int32_t y) {
+    return table[(size_t)x].n_tasks > table[(size_t)y].n_tasks;
+  });
+  std::vector<int32_t> lists[4];
+  b->blocks_fit = true;
+  for (const int32_t k : by_size) {
+    const ExecGraph& X = table[(size_t)k];
+    const int32_t span = (int32_t)shape[3 * (size_t)k];
+    b->max_outdeg = std::max(b->max_outdeg, (int32_t)shape[3 * (size_t)k + 2]);
+    if (block_window_fits(span, (int32_t)shape[3 * (size_t)k + 1], X.body, X.spin_iters)) {
+      lists[span <= kSmallSpan ? 1 : 0].push_back(k);
+    } else if (block_exec_fits(X.n_tasks, X.n_roots, X.body, X.spin_iters)) {
+      lists[X.n_tasks <= kBlockSmall ? 3 : 2].push_back(k);
+      b->max_queue_n = std::max(b->max_queue_n, X.n_tasks);
+    } else {
+      b->blocks_fit = false;
+    }
+  }
+  b->plan.clear();  // the lists one after another, then every graph's longest edge
+  for (int l = 0; l < 4; ++l) {
+    b->n_list[l] = (int32_t)lists[l].size();
+    b->plan.insert(b->plan.end(), lists[l].begin(), lists[l].end());
+  }
+  for (size_t k = 0; k < G; ++k) b->plan.push_back((int32_t)shape[3 * k]);
+  b->dirty = true;  // ring not yet initialised
+  return RT_OK;
+}
+}  // namespace
+
 extern "C" {
 
 rt_status rt_batch_create(const rt_graph_t* graphs, int32_t n_graphs, void* stream, rt_batch_t* out) {
@@ -1716,11 +1867,7 @@ rt_status rt_batch_create(const rt_graph_t* graphs, int32_t n_graphs, void* stre
   if ((st = b->adj.reserve((size_t)std::max<int64_t>(T, 1) * 32, s))) return bail(st);
   launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(),
                   nullptr, s);
-  if (cudaMemcpyAsync(b->gtable.p, table.data(), table.size() * sizeof(ExecGraph), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess)
-    return bail(fail(RT_ERR_CUDA, "batch assembly failed"));
-  b->dirty = true;  // ring not yet initialised
+  if ((st = finish_batch(b, table)) != RT_OK) return bail(st);
   *out = b;
   return RT_OK;
 }
@@ -1835,11 +1982,9 @@ rt_status rt_batch_create_stacked(rt_graph_t g, const int32_t* task_off, int32_t
   }
   launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(),
                   nullptr, s);
-  e = cudaMemcpyAsync(b->gtable.p, table.data(), table.size() * sizeof(ExecGraph), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  st = finish_batch(b, table);
   tmp.release(s);
-  if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return bail(fail(RT_ERR_CUDA, "batch assembly failed"));
-  b->dirty = true;  // ring not yet initialised
+  if (st != RT_OK) return bail(st);
   *out = b;
   return RT_OK;
 }
@@ -1855,9 +2000,7 @@ rt_status enqueue_batch(rt_batch* b, const ExecParams& p, int64_t ring_clear, in
   CK(cudaMemsetAsync(b->count.p, 0, (size_t)b->T * 4, s));
   launch_seed(p, ring_clear, s);
   launch_exec(p, blocks, warps, s);
-  CK(cudaMemcpyAsync(b->hpin, &p.ctrl->status, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(reinterpret_cast<char*>(b->hpin) + 512, p.ctrl->counters, kCntCount * sizeof(unsigned long long),
-                     cudaMemcpyDeviceToHost, s));
+  report_exec(p, b->hpin, b->hpin, s);
   return RT_OK;
 }
 
@@ -1873,9 +2016,61 @@ rt_status enqueue_batch_owned(rt_batch* b, const ExecParams& p, int blocks, int 
   launch_reset_counts(b->count.as<int32_t>(), b->indeg.as<int32_t>(), b->T, -1, 0, s);
   launch_seed(p, 0, s);  // clears the control block and the completion counters
   launch_exec(p, blocks, warps, s);
-  CK(cudaMemcpyAsync(b->hpin, &p.ctrl->status, 4, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(reinterpret_cast<char*>(b->hpin) + 512, p.ctrl->counters, kCntCount * sizeof(unsigned long long),
-                     cudaMemcpyDeviceToHost, s));
+  report_exec(p, b->hpin, b->hpin, s);
+  return RT_OK;
+}
+
+// A batch whose graphs all fit in a block: the large blocks on the launch's
+// stream and the small ones beside them on a second one.
+rt_status prepare_batch_blocks(rt_batch* b) {
+  if (b->order.p) return RT_OK;
+  cudaStream_t s = b->s;
+  if (b->n_list[2] + b->n_list[3] > 0) CKR(b->spill.reserve((size_t)b->T * 2, s));
+  if (b->n_list[0] + b->n_list[1] > 0 && b->max_outdeg > kAdjInline && !b->adjx.p) {
+    CKR(b->adjx.reserve((size_t)b->T * 32, s));
+    launch_pack_adjx(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->T, b->adjx.as<int4>(), s);
+  }
+  if (!b->side) CK(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
+  if (!b->fork) CK(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+  if (!b->join) CK(cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming));
+  CKR(b->order.reserve(b->plan.size() * 4, s));
+  CK(cudaMemcpyAsync(b->order.p, b->plan.data(), b->plan.size() * 4, cudaMemcpyHostToDevice, s));
+  return RT_OK;
+}
+
+rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, cudaStream_t s) {
+  CK(cudaMemsetAsync(p.ctrl, 0, sizeof(ExecCtrl), s));  // status, counters and the launches' next graphs
+  p.adjx = b->adjx.as<int4>();
+  uint32_t* const next[4] = {&p.ctrl->head, &p.ctrl->tail, &p.ctrl->ticket,
+                             reinterpret_cast<uint32_t*>(&p.ctrl->executed)};
+  const int32_t* const n = b->n_list;
+  const bool both = n[0] + n[2] > 0 && n[1] + n[3] > 0;
+  cudaStream_t side = both ? b->side : s;
+  if (both) {
+    CK(cudaEventRecord(b->fork, s));
+    CK(cudaStreamWaitEvent(side, b->fork, 0));
+  }
+  const int32_t* list = b->order.as<int32_t>();
+  const int32_t* const spans = list + (n[0] + n[1] + n[2] + n[3]);
+  for (int l = 0; l < 4; list += n[l++]) {
+    if (n[l] == 0) continue;
+    BlockArgs a{};
+    a.spans = spans;
+    a.spill = b->spill.as<uint16_t>();
+    a.order = list;
+    a.n_order = n[l];
+    a.next = next[l];
+    const bool small = l & 1;
+    const int blocks = std::min(n[l], g_dev.num_sms * (small ? 8 : 2));
+    cudaStream_t on = small ? side : s;
+    if (l < 2) launch_exec_window(p, a, blocks, small, on);
+    else launch_exec_block(p, a, small ? std::min(b->max_queue_n, kBlockSmall) : b->max_queue_n, blocks, small, on);
+  }
+  if (both) {
+    CK(cudaEventRecord(b->join, side));
+    CK(cudaStreamWaitEvent(s, b->join, 0));
+  }
+  report_exec(p, b->hpin, b->hpin, s);
   return RT_OK;
 }
 
@@ -2035,8 +2230,10 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
     CK(cudaGetLastError());
     return RT_OK;  // the ring was not touched: it stays as clean as the last ring launch left it
   }
-  bool clear = b->dirty;
-  if (cap * 8 > b->ring.cap) {
+  const bool in_blocks = b->blocks_fit && b->G_nonempty > 0;
+  if (in_blocks) CKR(prepare_batch_blocks(b));
+  bool clear = !in_blocks && b->dirty;
+  if (!in_blocks && cap * 8 > b->ring.cap) {
     drop_batch_graph(b);
     CKR(b->ring.reserve((size_t)cap * 8, s));
     clear = true;
@@ -2057,23 +2254,34 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
   p.replays = replays;
   p.graphs_target = b->G_nonempty;
   p.timeout_ns = 2000000000ll;
-  p.claim = claim > 0 ? claim : 32;
-  p.keep = keep > 0 ? keep : 32;
+  p.claim = claim > 0 ? claim : (in_blocks ? block_claim(b->E, b->T) : 32);
+  p.keep = keep > 0 ? keep : (in_blocks ? block_keep(b->E, b->T) : 32);
   p.tickets = nullptr;
   p.total_roots = (int32_t)b->Rtot;
   p.need_fence = b->need_fence;
   CK(cudaEventRecord(b->e0, s));
-  if (clear) {
+  if (in_blocks && !b->graph_next) {
+    // the first launch direct: a batch run once does not pay for a CUDA graph
+    b->graph_next = true;
+    CKR(enqueue_batch_blocks(b, p, s));
+  } else if (clear) {
     // a new or dirty ring is cleared whole: a direct launch
     CKR(enqueue_batch(b, p, (int64_t)(b->ring.cap / 8), blocks, warps, s));
   } else {
     // the launch from a cached CUDA graph, captured once per launch shape
-    const int64_t key[7] = {replays, blocks, warps, p.claim, p.keep, (int64_t)(uintptr_t)p.ring, (int64_t)p.ring_cap};
+    const int64_t key[7] = {replays,
+                            in_blocks ? 0 : blocks,
+                            in_blocks ? 0 : warps,
+                            p.claim,
+                            p.keep,
+                            in_blocks ? -2 : (int64_t)(uintptr_t)p.ring,
+                            (int64_t)p.ring_cap};
     if (!b->gexec || memcmp(key, b->gkey, sizeof key) != 0) {
       drop_batch_graph(b);
       if (!b->cap_stream) CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
       CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-      rt_status st = enqueue_batch(b, p, 0, blocks, warps, b->cap_stream);
+      rt_status st = in_blocks ? enqueue_batch_blocks(b, p, b->cap_stream)
+                               : enqueue_batch(b, p, 0, blocks, warps, b->cap_stream);
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamEndCapture(b->cap_stream, &graph);
       if (st != RT_OK) {
@@ -2137,9 +2345,13 @@ rt_status rt_batch_destroy(rt_batch_t b) {
   cudaStreamSynchronize(b->s);
   drop_batch_graph(b);
   DevBuf* bufs[] = {&b->row_ptr, &b->col,  &b->indeg, &b->count, &b->root_items, &b->gtable,  &b->done_g,
-                    &b->ring,    &b->ctrl, &b->adj,   &b->adjx,  &b->task_graph, &b->scratch};
+                    &b->ring,    &b->ctrl, &b->adj,   &b->adjx,  &b->task_graph, &b->scratch,
+                    &b->order,   &b->spill};
   for (DevBuf* x : bufs) x->release(b->s);
   cudaStreamSynchronize(b->s);
+  if (b->side) cudaStreamDestroy(b->side);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
   if (b->hpin) cudaFreeHost(b->hpin);
   if (b->e0) cudaEventDestroy(b->e0);
   if (b->e1) cudaEventDestroy(b->e1);

@@ -209,6 +209,10 @@ struct ExecParams {
   // (task_base, body, buffers) its body runs with; 0 / null for one graph
   int32_t owned_n;
   const int32_t* task_graph;
+  int32_t auto_warps;     // owned policy chosen by the library: its warps (0: the configured shape)
+  int32_t block_n;        // task count of a single graph that runs inside one block (0: grid-wide)
+  int32_t window;         // ... with counters for a window of program order
+  int32_t span;           // a single graph's longest edge
 };
 
 // ---------------------------------------------------------------------------
@@ -396,6 +400,47 @@ void launch_rebase_roots(const uint64_t* src, uint64_t* dst, int32_t n, int32_t 
 void launch_seed(ExecParams p, int64_t ring_clear, cudaStream_t s);
 void launch_exec(ExecParams p, int blocks, int warps, cudaStream_t s);
 int exec_max_blocks_per_sm(int warps);
+// small graphs inside one block each (block_exec.cu). The bounds: task ids of 16
+// bits; 2 bytes of shared memory a task for its countdown and 2 for the first
+// kBlockQueue places of the ready queue, 164 KB in all (a resident server's
+// blocks leave that on every SM); at most kBlockRoots tasks ready at the start
+// and kBlockWork body iterations in all, so that one SM's lanes suffice
+constexpr int32_t kBlockTasks = 65534;
+constexpr int32_t kBlockQueue = 16384;
+constexpr int32_t kBlockSmall = 4096;
+constexpr int64_t kBlockRoots = 1024;
+constexpr int64_t kBlockWork = 1ll << 24;
+bool block_exec_fits(int32_t n, int64_t n_roots, int32_t body, int32_t spin_iters);
+int block_exec_warps();
+int block_small_warps();
+// the same with counters for a window of program order only: graphs whose edges
+// and roots reach at most kWindowSpan tasks (kSmallSpan: blocks of 4 warps, which
+// hold two steps of that width), at most kWindowWork lane-iterations a step (one
+// SM's lanes). 300 steps of a stencil take 0.20 ms on one SM at 400 wide and
+// 0.28 at 600; over owned chunks 0.25 at 1024 (random fan-in: 0.74 against 0.38)
+constexpr int kWindowSlots = 16384;   // counters: 64 KB
+constexpr int kSmallSlots = 2048;
+constexpr int32_t kWindowSpan = 700;
+constexpr int32_t kSmallSpan = 70;
+constexpr int64_t kWindowWork = 1ll << 17;
+bool block_window_fits(int32_t span, int32_t last_root, int32_t body, int32_t spin_iters);
+struct BlockArgs {
+  int32_t span;           // k_exec_window: the graph's longest edge
+  const int32_t* spans;   // ... of each graph of a batch
+  uint16_t* spill;        // the queues' places past kBlockQueue: 16 bits per task of all graphs
+  const int32_t* order;   // a batch: the graphs to run, largest first (null: one graph)
+  int32_t n_order;        // how many (1 for one graph)
+  uint32_t* next;         // ... and the counter that hands them out, zeroed by the caller
+  uint32_t* status_out;   // one graph: status and diagnostic counters, in pinned host memory
+  unsigned long long* counters_out;
+};
+// max_n: the largest graph's tasks; small: blocks of a few warps
+void launch_exec_window(const ExecParams& p, const BlockArgs& a, int blocks, bool small, cudaStream_t s);
+// shape[3g..3g+2] of graph g: longest edge, last root, largest out-degree
+void launch_batch_shape(const ExecGraph* graphs, int32_t G, const int32_t* row_ptr, const int32_t* col,
+                        const int32_t* indeg, uint32_t* shape, cudaStream_t s);
+void launch_exec_block(ExecParams p, const BlockArgs& a, int32_t max_n, int blocks, bool small, cudaStream_t s);
+void preload_block_exec();
 rt_status microbench(double* out, int n_out, cudaStream_t s, const char** why);
 void launch_serve_init(ServeParams p, cudaStream_t s);
 void preload_primitives();
@@ -458,7 +503,11 @@ struct StitchParams {
   int64_t timeout_ns;
 };
 void launch_stitch_check(const int32_t* req_off, const int64_t* lo, const int64_t* hi, const uint8_t* priv, int D,
-                         const int32_t* row_ptr, const int32_t* col, int32_t n, uint32_t* err, cudaStream_t s);
+                         const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int32_t n, uint32_t* err,
+                         cudaStream_t s);
+constexpr int kStitchOwnedWarps = 4;  // per block
+void launch_stitch_owned(const StitchParams& p, const int4* adjx, const int32_t* indeg, int wr, int groups, bool fence,
+                         cudaStream_t s);
 void launch_stitch(const StitchParams& p, const int32_t* indeg, const uint64_t* root_items, const uint32_t* rootpos,
                    int blocks, int warps, bool tickets, bool fence, cudaStream_t s);
 // tasks as whole kernels (rt_execute_kernels)

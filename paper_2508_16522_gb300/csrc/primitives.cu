@@ -479,6 +479,7 @@ void preload_all() {
   preload_sweep();
   preload_window();
   preload_exec();
+  preload_block_exec();
   preload_serve();
   preload_events();
   preload_task_kernel();

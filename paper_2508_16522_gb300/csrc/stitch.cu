@@ -44,7 +44,8 @@ constexpr int kStRound = 4;  // 32-edge groups whose decrements are in flight to
 
 // the second copy repeats the first: same rectangles, same in-copy edges
 __global__ void k_st_check(const int32_t* req_off, const int64_t* lo, const int64_t* hi, const uint8_t* priv,
-                           int D, const int32_t* row_ptr, const int32_t* col, int32_t n, uint32_t* err) {
+                           int D, const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int32_t n,
+                           uint32_t* err) {
   const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n) return;
   const int32_t a0 = req_off[v], a1 = req_off[v + 1], b0 = req_off[n + v], b1 = req_off[n + v + 1];
@@ -70,6 +71,11 @@ __global__ void k_st_check(const int32_t* req_off, const int64_t* lo, const int6
     }
   }
   if (s0 + k != s1) atomicOr(err, 2u);
+  // how far program order strays from the dependences: the longest in-copy
+  // edge (err[1]) and the last task without in-copy predecessors (err[2])
+  const uint32_t far = k > 0 ? (uint32_t)(col[r0 + k - 1] - v) : 0u;
+  if (far > *(volatile uint32_t*)(err + 1)) atomicMax(err + 1, far);
+  if (indeg[v] == 0 && (uint32_t)v > *(volatile uint32_t*)(err + 2)) atomicMax(err + 2, (uint32_t)v);
 }
 
 // counters of every (replay, task), the first ready items and the control
@@ -85,7 +91,7 @@ __global__ void k_st_init(StitchParams p, const int32_t* indeg, const uint64_t* 
   }
   // roots of the two-copy graph: first copy's (no in-copy predecessor) come
   // first, then the second copy's (no predecessor at all)
-  const int64_t a = rootpos[n], b = (int64_t)rootpos[2 * n] - a;
+  const int64_t a = p.ring ? rootpos[n] : 0, b = p.ring ? (int64_t)rootpos[2 * n] - a : 0;
   for (int64_t k = i0; k < a; k += stride) p.ring[k] = (uint32_t)root_items[k];
   for (int64_t k = i0; k < (int64_t)(p.R - 1) * b; k += stride) {
     const int64_t r = 1 + k / b, j = k - (r - 1) * b;
@@ -328,6 +334,117 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
   }
 }
 
+// The same over owned chunks (see k_exec_owned in exec.cu), for traces whose
+// program order follows their dependences closely (see k_st_check's spans).
+// The warps form groups of `wr`; a group takes replays g, g + groups, ... one
+// after another, and warp w of it the chunks w, w + wr, ... of 32 consecutive
+// tasks, one task per lane, polling their counters. A hop costs a reduction and
+// the owner's next poll instead of a trip through the ring, and the replays
+// still overlap: each has its own warps. Every edge leads to a later (replay,
+// task), every warp takes its chunks in that order and all warps are resident,
+// so the first unfinished task is always held with its predecessors done.
+template <bool FENCE>
+__global__ void __launch_bounds__(256) k_stitch_owned(StitchParams p, const int4* adjx, int wr, int groups) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gw = (int)blockIdx.x * (int)(blockDim.x >> 5) + warp;
+  if (gw >= wr * groups) return;
+  ExecCtrl* const ctrl = p.ctrl;
+  const ExecGraph& G = p.G;
+  const int n = p.n, body = G.body, spin = G.spin_iters, nchunks = (n + 31) / 32;
+  const int R4 = adjx != nullptr ? 4 : 2;  // int4s per trigger record
+  const int inl = 4 * R4 - 3;              // successors it holds
+  int r = gw / wr, c = gw % wr;
+  uint64_t idle_since = 0, last_check = 0;
+  unsigned long long seen = 0;
+  while (r < p.R) {
+    if (c >= nchunks) {
+      c = gw % wr;
+      r += groups;
+      continue;
+    }
+    const int v = c * 32 + lane;
+    const bool has = v < n;
+    int32_t* const count = p.count + (int64_t)r * n;  // successor s of (r, v) is count[s], s >= n in replay r + 1
+    const int limit = r + 1 < p.R ? 2 * n : n;        // ... dropped after the last replay
+    int4 q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      q[k] = make_int4(-1, -1, -1, -1);
+      if (k < R4 && has) q[k] = __ldg(k < 2 ? p.adj + 2 * (int64_t)v + k : adjx + 2 * (int64_t)v + (k - 2));
+    }
+    int32_t polled = has ? ld_relaxed_s32(count + v) : 1;
+    unsigned pending = __ballot_sync(kFullT, has);
+    const int tasks = __popc(pending);
+    const int deg = has ? q[0].y : 0;
+    const int dmax = (int)__reduce_max_sync(kFullT, (unsigned)deg);
+    uint32_t backoff = 0;
+    while (pending) {
+      const bool ready = ((pending >> lane) & 1u) && polled == 0;
+      const unsigned rm = __ballot_sync(kFullT, ready);
+      if (!rm) {
+        int stop = 0;
+        if (backoff >= 64 && lane == 0) {
+          const uint64_t now = globaltimer_ns();
+          if (idle_since == 0) {
+            idle_since = last_check = now;
+            seen = ld_relaxed_u64(&ctrl->executed);
+          } else if (now - last_check > 2000u) {
+            last_check = now;
+            const unsigned long long pr = ld_relaxed_u64(&ctrl->executed);
+            if (ld_relaxed_u32(&ctrl->status) != 0u) {
+              stop = 1;
+            } else if (pr != seen) {
+              seen = pr;
+              idle_since = now;
+            } else if (now - idle_since > (uint64_t)p.timeout_ns) {
+              atomicCAS(&ctrl->status, 0u, (uint32_t)RT_ERR_TIMEOUT);
+              stop = 1;
+            }
+          }
+        }
+        if (__shfl_sync(kFullT, stop, 0)) return;
+        if (backoff) __nanosleep(backoff);
+        backoff = backoff ? (backoff < 256 ? backoff * 2 : 256) : 16;
+        if ((pending >> lane) & 1u) polled = ld_relaxed_s32(count + v);
+        continue;
+      }
+      backoff = 0;
+      idle_since = 0;
+      pending &= ~rm;
+      // the next poll is in flight during the work below (late at worst:
+      // counters only go down)
+      if (!FENCE) polled = ((pending >> lane) & 1u) ? ld_relaxed_s32(count + v) : 1;
+      if (FENCE) fence_acq_rel_gpu();  // acquire: the predecessors' effects before the bodies
+      if (ready) {
+        const int64_t slot = (int64_t)r * n + v;
+        if (body == RT_BODY_SPIN) G.out[slot] = (int32_t)spin_body((uint32_t)v, spin);
+        else if (body == RT_BODY_FMA) G.out[slot] = fma_body((uint32_t)v, spin);
+        else if (FENCE) run_body<true>(G, v);
+      }
+      if (FENCE) fence_acq_rel_gpu();  // release: bodies before the decrements
+      if (ready) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (k < R4 && 4 * k - 3 < dmax) {
+            if (k > 0 && q[k].x >= 0 && q[k].x < limit) red_dec_s32(count + q[k].x);
+            if (k > 0 && q[k].y >= 0 && q[k].y < limit) red_dec_s32(count + q[k].y);
+            if (k > 0 && q[k].z >= 0 && q[k].z < limit) red_dec_s32(count + q[k].z);
+            if (q[k].w >= 0 && q[k].w < limit) red_dec_s32(count + q[k].w);
+          }
+        }
+        for (int e = inl; e < deg; ++e) {  // rare: past the record
+          const int s = __ldg(p.col + q[0].x + e);
+          if (s < limit) red_dec_s32(count + s);
+        }
+      }
+      __syncwarp();
+      if (FENCE) polled = ((pending >> lane) & 1u) ? ld_relaxed_s32(count + v) : 1;
+    }
+    if (lane == 0) red_add_u64(&ctrl->executed, (unsigned long long)tasks);  // progress, for the bounded waits
+    c += wr;
+  }
+}
+
 // at most 8 warps of 3.5 KB: under the 48 KB of dynamic shared memory a
 // launch gets without opting in
 template <bool TICKETS, bool FENCE>
@@ -338,10 +455,11 @@ void launch_one(const StitchParams& p, int blocks, int warps, cudaStream_t s) {
 }  // namespace
 
 void launch_stitch_check(const int32_t* req_off, const int64_t* lo, const int64_t* hi, const uint8_t* priv, int D,
-                         const int32_t* row_ptr, const int32_t* col, int32_t n, uint32_t* err, cudaStream_t s) {
+                         const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int32_t n, uint32_t* err,
+                         cudaStream_t s) {
   if (n <= 0) return;
   count_launch();
-  k_st_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(req_off, lo, hi, priv, D, row_ptr, col, n, err);
+  k_st_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(req_off, lo, hi, priv, D, row_ptr, col, indeg, n, err);
 }
 
 void launch_stitch(const StitchParams& p, const int32_t* indeg, const uint64_t* root_items, const uint32_t* rootpos,
@@ -357,10 +475,21 @@ void launch_stitch(const StitchParams& p, const int32_t* indeg, const uint64_t* 
   }
 }
 
+void launch_stitch_owned(const StitchParams& p, const int4* adjx, const int32_t* indeg, int wr, int groups, bool fence,
+                         cudaStream_t s) {
+  count_launch(2);
+  k_st_init<<<1024, 256, 0, s>>>(p, indeg, nullptr, nullptr);
+  const int blocks = (wr * groups + kStitchOwnedWarps - 1) / kStitchOwnedWarps;
+  if (fence) k_stitch_owned<true><<<blocks, kStitchOwnedWarps * 32, 0, s>>>(p, adjx, wr, groups);
+  else k_stitch_owned<false><<<blocks, kStitchOwnedWarps * 32, 0, s>>>(p, adjx, wr, groups);
+}
+
 void preload_stitch() {
   cudaFuncAttributes a;
   cudaFuncGetAttributes(&a, k_st_check);
   cudaFuncGetAttributes(&a, k_st_init);
+  cudaFuncGetAttributes(&a, k_stitch_owned<false>);
+  cudaFuncGetAttributes(&a, k_stitch_owned<true>);
   cudaFuncGetAttributes(&a, k_stitch<false, false>);
   cudaFuncGetAttributes(&a, k_stitch<false, true>);
   cudaFuncGetAttributes(&a, k_stitch<true, false>);
