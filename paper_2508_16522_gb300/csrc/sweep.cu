@@ -65,6 +65,7 @@ namespace {
 constexpr int kHashSlots = 128;
 constexpr int kListCap = 64;
 constexpr int kLaneBuf = 16;     // predecessors one lane buffers in the lane-parallel path
+constexpr int kOccCells = 256;   // tiles up to this many cells find a window's conflicts cell by cell
 constexpr int kSmallCells = 16;  // largest box the lane-parallel path takes
 constexpr int kMaxRounds = 16;   // deeper conflict chains go to the warp-wide path
 constexpr int kLongSpan = 64;    // run spans the whole warp scans together
@@ -93,9 +94,16 @@ __host__ __device__ inline size_t row_table_bytes(int tw) {
   return tw <= kMaxTileSide2D ? (size_t)((32 * 4 * 2 + 8 * tw + 15) & ~15) : 0;
 }
 
+// lane-parallel path: which of the window's candidates cover each class cell
+// (tiles of at most kOccCells)
+__host__ __device__ inline size_t occ_bytes(int tw, int th) {
+  const int C = class_cap(tw, th);
+  return C <= kOccCells ? (size_t)((4 * C + 15) & ~15) : 0;
+}
+
 __host__ __device__ inline size_t per_warp_bytes(int tw, int th) {
   const int C = class_cap(tw, th);
-  return (size_t)16 * C + (size_t)((C + 15) & ~15) + 32 * 8 + kHashSlots * 4 + kListCap * 8 + 16 +
+  return occ_bytes(tw, th) + (size_t)16 * C + (size_t)((C + 15) & ~15) + 32 * 8 + kHashSlots * 4 + kListCap * 8 + 16 +
          32 * kLaneBuf * 4 + class_map_bytes(tw, th) + seg_bytes(tw, th) + row_table_bytes(tw);  // 16-byte
                                                                        // multiple: warps' uint4 cells stay aligned
 }
@@ -122,6 +130,7 @@ struct WarpSmem {
   unsigned long long* xtab;  // [kExtSlots] (predecessor << 5 | task index) pairs from before the window
                             // (in the lane-parallel path's buffer)
   int* xcount;              // its entries
+  uint32_t* occ;            // [class cell] window candidates that cover it (lane-parallel path; null: larger tiles)
 };
 
 // in place: a[i] <- a[0] + ... + a[i] over a[0..L) (one warp, convergent)
@@ -414,38 +423,58 @@ __device__ bool stage_lanes(Ctx& x, const WarpSmem& w, const SweepOut& o, unsign
   // position of this candidate's task (its group's first candidate)
   const unsigned upto = lane == 31 ? starts : (starts & ((2u << lane) - 1u));
   const int gpos = x.pos + (upto ? 31 - __clz((int)upto) : 0);
-  int level = 0;
-  bool bad = false;
-  for (int j = 0; j < end; ++j) {
-    const int x0 = __shfl_sync(kFull, b.x0, j), x1 = __shfl_sync(kFull, b.x1, j);
-    const int y0 = __shfl_sync(kFull, b.y0, j), y1 = __shfl_sync(kFull, b.y1, j);
-    const int tj = __shfl_sync(kFull, b.task, j), lj = __shfl_sync(kFull, level, j);
-    if (mine && lane > j && b.x0 <= x1 && x0 <= b.x1 && b.y0 <= y1 && y0 <= b.y1) {
-      if (tj == b.task) bad = true;
-      else if (lj + 1 > level) level = lj + 1;
+  // the earlier candidates this one overlaps: from the masks of its cells (every
+  // lane marks its own; comparing the 32 boxes by shuffles took a good part of the
+  // window: 328 -> 238 us of sweep on the random 1024 x 1000 Task Bench graph at
+  // 32 x 4 tiles), on large tiles by comparing the boxes
+  unsigned conf = 0u;
+  if (w.occ) {
+    const int y1 = mine ? b.y1 : -1;
+    for (int cy = b.y0; cy <= y1; ++cy)
+      for (int cx = b.x0; cx <= b.x1; ++cx) atomicOr(w.occ + cy * x.tw + cx, 1u << lane);
+    __syncwarp();
+    for (int cy = b.y0; cy <= y1; ++cy)
+      for (int cx = b.x0; cx <= b.x1; ++cx) conf |= w.occ[cy * x.tw + cx];
+    __syncwarp();
+    for (int cy = b.y0; cy <= y1; ++cy)
+      for (int cx = b.x0; cx <= b.x1; ++cx) w.occ[cy * x.tw + cx] = 0u;
+    conf &= lanemask_lt();
+    __syncwarp();
+  } else {
+    for (int j = 0; j < end; ++j) {
+      const int x0 = __shfl_sync(kFull, b.x0, j), x1 = __shfl_sync(kFull, b.x1, j);
+      const int y0 = __shfl_sync(kFull, b.y0, j), y1 = __shfl_sync(kFull, b.y1, j);
+      if (mine && lane > j && b.x0 <= x1 && x0 <= b.x1 && b.y0 <= y1 && y0 <= b.y1) conf |= 1u << j;
     }
   }
-  if (__any_sync(kFull, bad)) return false;
-  int maxl = level;
-#pragma unroll
-  for (int o2 = 16; o2 >= 1; o2 >>= 1) maxl = max(maxl, __shfl_xor_sync(kFull, maxl, o2));
-  if (maxl >= kMaxRounds) return false;  // nothing applied yet: the warp-wide path takes the window
+  const unsigned own = ~((1u << (gpos - x.pos)) - 1u);  // this task's candidates (and later ones)
+  if (__any_sync(kFull, mine && (conf & own))) return false;
+  // levels, round by round: a candidate runs once all it overlaps have
+  int level = 0, maxl = 0;
+  const unsigned all = __ballot_sync(kFull, mine);
+  for (unsigned done = 0u;; ++maxl) {
+    const unsigned now = __ballot_sync(kFull, mine && !((done >> lane) & 1u) && !(conf & ~done));
+    if ((now >> lane) & 1u) level = maxl;
+    done |= now;
+    if (done == all) break;
+    if (maxl + 1 >= kMaxRounds) return false;  // nothing applied yet: the warp-wide path takes the window
+  }
   // each lane runs in one round (its level) and buffers its candidate's
   // predecessors; the buffers are written out once, after the last round
   int nb = 0;
   for (int r = 0; r <= maxl; ++r) {
     if (mine && level == r) {
-      const int bw = b.x1 - b.x0 + 1;
-      for (int i = 0; i < cells; ++i) {
-        const int cx = b.x0 + i % bw, cy = b.y0 + i / bw;
-        uint32_t rs, rl, rc;
-        apply_cell(w, cy * x.tw + cx, gpos, b.priv, rs, rl, rc);
-        if (rc >= 1u) lane_add(w, o, lane, nb, (int)(uint32_t)entry_at(x, w, (int)rs), b.task);
-        if (rc >= 2u) lane_add(w, o, lane, nb, (int)(uint32_t)entry_at(x, w, (int)rl), b.task);
-        if (rc == 3u) {
-          for (uint32_t q = rs + 1; q < rl; ++q) {
-            Box e = unpack_c(x, w, entry_at(x, w, (int)q));
-            if (e.x0 <= cx && cx <= e.x1 && e.y0 <= cy && cy <= e.y1) lane_add(w, o, lane, nb, e.task, b.task);
+      for (int cy = b.y0; cy <= b.y1; ++cy) {
+        for (int cx = b.x0; cx <= b.x1; ++cx) {
+          uint32_t rs, rl, rc;
+          apply_cell(w, cy * x.tw + cx, gpos, b.priv, rs, rl, rc);
+          if (rc >= 1u) lane_add(w, o, lane, nb, (int)(uint32_t)entry_at(x, w, (int)rs), b.task);
+          if (rc >= 2u) lane_add(w, o, lane, nb, (int)(uint32_t)entry_at(x, w, (int)rl), b.task);
+          if (rc == 3u) {
+            for (uint32_t q = rs + 1; q < rl; ++q) {
+              Box e = unpack_c(x, w, entry_at(x, w, (int)q));
+              if (e.x0 <= cx && cx <= e.x1 && e.y0 <= cy && cy <= e.y1) lane_add(w, o, lane, nb, e.task, b.task);
+            }
           }
         }
       }
@@ -470,8 +499,8 @@ __device__ bool stage_lanes(Ctx& x, const WarpSmem& w, const SweepOut& o, unsign
   }
   const int total = __shfl_sync(kFull, incl, 31);
   // the tile's count bounds a rerun, which writes every pair: count them all
-  const int all = __reduce_add_sync(kFull, (unsigned)nb);
-  if (lane == 0 && all) atomicAdd(w.npairs, all);
+  const int found = (int)__reduce_add_sync(kFull, (unsigned)nb);
+  if (lane == 0 && found) atomicAdd(w.npairs, found);
   if (total > 0) {
     const PairDst pd = reserve_pairs(x, o, (uint32_t)total);
     int pos = incl - nf;
@@ -1026,6 +1055,9 @@ __global__ void __launch_bounds__(256, 3) k_sweep(const uint64_t* __restrict__ p
   w.rpred = w.rbox + 32;
   w.rlo = w.rpred + 32;
   w.rhi = w.rlo + d.tw;
+  w.occ = occ_bytes(d.tw, d.th) ? reinterpret_cast<uint32_t*>(base + per_warp_bytes(d.tw, d.th) - occ_bytes(d.tw, d.th)) : nullptr;
+  if (w.occ)
+    for (int i = lane; i < C; i += 32) w.occ[i] = 0u;
   static_assert(kExtSlots * 8 <= 32 * kLaneBuf * 4, "the set fits the lane-parallel path's buffer");
   w.xtab = reinterpret_cast<unsigned long long*>(w.lbuf);
   w.dropped = w.hcount + 1;
