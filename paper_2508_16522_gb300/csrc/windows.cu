@@ -27,12 +27,12 @@
 // candidates spread over many warps and the last tile holds up no one.
 //
 // Bound by instruction issue (71% of the active cycles on 60k launches of the
-// 4096 x 4096 trace, 1280 warp instructions per 16 candidates; DRAM 2%): about a
-// seventh is spent on pairs, a seventh on walks, the rest on classes and cells.
-// 32 warps an SM. The 1M-launch trace at 16 x 32 tiles sweeps in 35 ms where the
-// tile sweep takes 192, 43 captured requests in 2.1 ms where it takes 3.4. A
-// shorter look back or fewer new candidates a window (8, with 24, 16 or 12
-// before them) were slower: 36 to 45 ms, more cells need walks.
+// 4096 x 4096 trace; DRAM 2%), spent on class columns and rows, cells, pairs and
+// walks in about that order. 32 warps an SM. The 1M-launch trace at 16 x 32 tiles
+// sweeps in 29 ms where the tile sweep takes 192, 43 captured requests in 1.6 ms
+// where it takes 3.4. (When the sweep stood at 33 ms, 10 candidates before a
+// window made it 43, and 8 new ones with 24, 16 or 12 before them 36 to 45: more
+// cells need walks.)
 //
 // A tile this does not suit is flagged and left to sweep.cu, which keeps state
 // and so never looks back: one with a task of more than kNew candidates, with
@@ -376,8 +376,11 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
       // (class j in lane j of colm / colx, class 32 + j in lane j of colm2 / colx2)
       unsigned colm = 0u, rowm = 0u, colm2 = 0u, rowm2 = 0u;
       int cols = 0, rows = 0, colx = 0, rowy = 0, colx2 = 0, rowy2 = 0;
+      // a box left out covers nothing
+      const unsigned bx0 = act ? (unsigned)e.x0 : 0x10000u, bxw = act ? (unsigned)(e.x1 - e.x0) : 0u;
+      const unsigned by0 = act ? (unsigned)e.y0 : 0x10000u, byw = act ? (unsigned)(e.y1 - e.y0) : 0u;
       auto column = [&](int c) {
-        const unsigned b = __ballot_sync(kFullW, act && e.x0 <= c && c <= e.x1);
+        const unsigned b = __ballot_sync(kFullW, (unsigned)c - bx0 <= bxw);
         if (!(b & newbits)) return;
         if (lane == (cols & 31)) {
           if (!WIDE || cols < 32) {
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
         ++cols;
       };
       auto row = [&](int c) {
-        const unsigned b = __ballot_sync(kFullW, act && e.y0 <= c && c <= e.y1);
+        const unsigned b = __ballot_sync(kFullW, (unsigned)c - by0 <= byw);
         if (!(b & newbits)) return;
         if (lane == (rows & 31)) {
           if (!WIDE || rows < 32) {
@@ -444,7 +447,21 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
       const unsigned S = (rp & me) ? rp : ((dp & me) ? dp : 0u);
       const unsigned gts = gt & ~S;
       // ---- every class cell, PARTS rows at a time ------------------------------
-      for (int i = 0; i < rows && !drop; i += PARTS) {
+      // every run is decided here, no task has two candidates: 97% of the 1M-launch
+      // trace's windows (their own loop: 35 -> 29 ms)
+      const bool plain = !more && !nonst;
+      for (int i = 0; plain && i < rows && !drop; i += PARTS) {
+        unsigned rm = pick(rowm, rowm2, i + part);
+        if (i + part >= rows) rm = 0u;
+        for (int j = 0; j < cols; ++j) {
+          const unsigned m = rm & pick(colm, colm2, j);
+          bool open;
+          unsigned lo;
+          const unsigned run = pred_run(m, rp, dp, gt, gts, open, lo);
+          if (m & me) acc |= run;
+        }
+      }
+      for (int i = 0; !plain && i < rows && !drop; i += PARTS) {
         unsigned rm = pick(rowm, rowm2, i + part);
         if (i + part >= rows) rm = 0u;
         for (int j = 0; j < cols && !drop; ++j) {
