@@ -126,6 +126,43 @@ __global__ void k_widen_bounds(const int32_t* lo32, const int32_t* hi32, int64_t
   }
 }
 
+// A batch's rectangles into the graph's own arrays, widened and checked in one
+// pass (a copy each and a checking kernel read the bounds twice: 55 us more for
+// 6.1M rectangles). priv_in may be priv. Two bounds go as one load and store
+// where the caller's arrays allow it (wide).
+template <class T, bool WIDE>
+__global__ void __launch_bounds__(256) k_ingest_rects(const T* lo_in, const T* hi_in, const uint8_t* priv_in, int64_t R,
+                                                      AnalysisDims d, int64_t* lo, int64_t* hi, uint8_t* priv,
+                                                      uint32_t* err) {
+  struct alignas(2 * sizeof(T)) Pair {
+    T x, y;
+  };
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= R) return;
+  uint32_t e = 0;
+  int64_t a[2] = {0, 0}, b[2] = {0, 0};
+  if (WIDE) {
+    const Pair p = reinterpret_cast<const Pair*>(lo_in)[r], q = reinterpret_cast<const Pair*>(hi_in)[r];
+    a[0] = p.x;
+    a[1] = p.y;
+    b[0] = q.x;
+    b[1] = q.y;
+    reinterpret_cast<longlong2*>(lo)[r] = make_longlong2(a[0], a[1]);
+    reinterpret_cast<longlong2*>(hi)[r] = make_longlong2(b[0], b[1]);
+  } else {
+    for (int k = 0; k < d.ndim; ++k) {
+      lo[r * d.ndim + k] = a[k] = lo_in[r * d.ndim + k];
+      hi[r * d.ndim + k] = b[k] = hi_in[r * d.ndim + k];
+    }
+  }
+  for (int k = 0; k < d.ndim; ++k)
+    if (a[k] > b[k] || a[k] < d.dom_lo[k] || b[k] > d.dom_lo[k] + d.ext[k] - 1) e |= kErrRect;
+  const uint8_t p = priv_in[r];
+  if (p > 2) e |= kErrPriv;
+  priv[r] = p;
+  if (e) atomicOr(err, e);
+}
+
 // tile range of one rectangle (coordinates relative to the domain origin)
 struct TileRange {
   int64_t lx, hx, ly, hy;  // relative inclusive bounds
@@ -149,28 +186,37 @@ __device__ __forceinline__ TileRange tile_range(const int64_t* lo, const int64_t
     t.ly = 0;
     t.hy = 0;
   }
-  t.tx0 = (int32_t)(t.lx / d.tw);
-  t.ty0 = (int32_t)(t.ly / d.th);
-  t.ntx = (int32_t)(t.hx / d.tw) - t.tx0 + 1;
-  t.nty = (int32_t)(t.hy / d.th) - t.ty0 + 1;
+  // a 64-bit division takes about a hundred instructions, and there are four
+  if (d.shx >= 0) {
+    t.tx0 = (int32_t)(t.lx >> d.shx);
+    t.ty0 = (int32_t)(t.ly >> d.shy);
+    t.ntx = (int32_t)(t.hx >> d.shx) - t.tx0 + 1;
+    t.nty = (int32_t)(t.hy >> d.shy) - t.ty0 + 1;
+  } else {
+    t.tx0 = (int32_t)(t.lx / d.tw);
+    t.ty0 = (int32_t)(t.ly / d.th);
+    t.ntx = (int32_t)(t.hx / d.tw) - t.tx0 + 1;
+    t.nty = (int32_t)(t.hy / d.th) - t.ty0 + 1;
+  }
   return t;
 }
 
 // Each rectangle's tiles, and its task. A warp takes the rectangles of 32
 // consecutive tasks, one per lane at a time, so that the corners' loads coalesce
 // (a thread per task, each walking its own rectangles: 81 us for 6.1M rectangles
-// of 1M tasks). Also adds up the cells of all rectangles (*area, zeroed by the
-// caller): with the entry count it says how much of their tiles the entries
-// cover; and clears zero[0..n), the pair counts per source of the CSR stage.
+// of 1M tasks). Also adds up the cells of all rectangles (area[0], zeroed by the
+// caller) and their tiles (area[1], in 64 bits: the counts themselves are only
+// scanned once the sum is known to fit), which together say how much of their
+// tiles the entries cover; and clears zero[0..n), the pair counts per source of the CSR stage.
 __global__ void __launch_bounds__(256) k_bin_count(const int32_t* __restrict__ req_off, int32_t n, int64_t R,
                                                    const int64_t* __restrict__ lo, const int64_t* __restrict__ hi,
                                                    AnalysisDims d, int32_t* __restrict__ rect_task,
-                                                   uint64_t* __restrict__ cnt, unsigned long long* area,
+                                                   uint32_t* __restrict__ cnt, unsigned long long* area,
                                                    uint32_t* __restrict__ zero) {
-  __shared__ unsigned long long part[8];
+  __shared__ unsigned long long part[8][2];
   const int lane = threadIdx.x & 31;
   const int32_t t = blockIdx.x * blockDim.x + threadIdx.x, t0 = t - lane;
-  unsigned long long sum = 0;
+  unsigned long long sum = 0, tiles = 0;
   if (t < n) zero[t] = 0u;
   // lane l holds the first rectangle of task t0 + l
   const int32_t first = req_off[t < n ? t : n];
@@ -186,76 +232,99 @@ __global__ void __launch_bounds__(256) k_bin_count(const int32_t* __restrict__ r
     if (r < end) {
       rect_task[r] = t0 + own;
       const TileRange tr = tile_range(lo, hi, r, d);
-      cnt[r] = (uint64_t)tr.ntx * (uint64_t)tr.nty;
+      cnt[r] = (uint32_t)tr.ntx * (uint32_t)tr.nty;  // at most the domain's 2^26 tiles
+      tiles += (unsigned long long)tr.ntx * (unsigned long long)tr.nty;
       sum += (unsigned long long)(tr.hx - tr.lx + 1) * (unsigned long long)(tr.hy - tr.ly + 1);
     }
   }
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (lane == 0) part[threadIdx.x >> 5] = sum;
+  for (int o = 16; o >= 1; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    tiles += __shfl_xor_sync(0xffffffffu, tiles, o);
+  }
+  if (lane == 0) {
+    part[threadIdx.x >> 5][0] = sum;
+    part[threadIdx.x >> 5][1] = tiles;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 2) {
+    sum = 0;
 #pragma unroll
-    for (int w = 1; w < 8; ++w) sum += part[w];
-    if (sum) red_add_u64(area, sum);
+    for (int w = 0; w < 8; ++w) sum += part[w][threadIdx.x];
+    if (sum) red_add_u64(area + threadIdx.x, sum);
   }
 }
 
 // One thread per rectangle: a rectangle over a few tiles writes its own
 // entries; the entries of a larger one are written by its whole warp
-// (lane-strided), so that large rectangles do not serialise on one lane.
-constexpr uint64_t kOwnTiles = 4;
+// (lane-strided), so that large rectangles do not serialise on one lane. Only a
+// rectangle's first and last tile column (row) cut it, so an entry's box is four
+// selections of 32-bit offsets.
+constexpr uint32_t kOwnTiles = 4;
 
-__global__ void k_bin_expand(const int32_t* rect_task, const int64_t* lo, const int64_t* hi,
-                             const uint8_t* priv, int64_t R, const uint64_t* off, AnalysisDims d,
-                             uint32_t* keys, uint64_t* payload) {
+__global__ void __launch_bounds__(256) k_bin_expand(const int32_t* __restrict__ rect_task,
+                                                    const int64_t* __restrict__ lo, const int64_t* __restrict__ hi,
+                                                    const uint8_t* __restrict__ priv, int64_t R,
+                                                    const uint32_t* __restrict__ off, AnalysisDims d,
+                                                    uint32_t* __restrict__ keys, uint64_t* __restrict__ payload) {
   const int lane = threadIdx.x & 31;
-  int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-  bool valid = r < R;
-  TileRange tr{};
-  uint64_t base = 0, cnt = 0;
-  uint32_t task = 0, pv = 0;
+  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  const bool valid = r < R;
+  uint32_t base = 0, cnt = 0, task = 0, pv = 0, tile0 = 0;
+  int ntx = 1, nty = 1, fx = 0, lx = 0, fy = 0, ly = 0;  // first and last column (row) inside their tiles
   if (valid) {
-    tr = tile_range(lo, hi, r, d);
+    const TileRange tr = tile_range(lo, hi, r, d);
     base = off[r];
     cnt = off[r + 1] - base;
     task = (uint32_t)rect_task[r];
     pv = priv[r];
+    ntx = tr.ntx;
+    nty = tr.nty;
+    fx = (int)(tr.lx - (int64_t)tr.tx0 * d.tw);
+    fy = (int)(tr.ly - (int64_t)tr.ty0 * d.th);
+    lx = (int)(tr.hx - (int64_t)(tr.tx0 + ntx - 1) * d.tw);
+    ly = (int)(tr.hy - (int64_t)(tr.ty0 + nty - 1) * d.th);
+    tile0 = (uint32_t)tr.ty0 * (uint32_t)d.ntx + (uint32_t)tr.tx0;
   }
+  auto put = [&](uint32_t at, uint32_t tile, int i, int j, int nx, int ny, int x0, int x1, int y0, int y1, uint32_t tk,
+                 uint32_t p) {
+    keys[at] = tile + (uint32_t)j * (uint32_t)d.ntx + (uint32_t)i;
+    payload[at] = pack_entry(tk, p, d.ndim, (uint32_t)(i == 0 ? x0 : 0), (uint32_t)(i == nx - 1 ? x1 : d.tw - 1),
+                             (uint32_t)(j == 0 ? y0 : 0), (uint32_t)(j == ny - 1 ? y1 : d.th - 1));
+  };
   // A rectangle over at most kOwnTiles tiles (the usual case: one) is written
   // by its own lane; consecutive rectangles then write consecutive entries, so
   // the stores coalesce. Larger ones are written by the whole warp below.
-  const bool own = valid && cnt <= (uint64_t)kOwnTiles;
+  const bool own = valid && cnt <= kOwnTiles;
   if (own) {
-    for (uint64_t k = 0; k < cnt; ++k) {
-      const int32_t tx = tr.tx0 + (int32_t)(k % (uint64_t)tr.ntx);
-      const int32_t ty = tr.ty0 + (int32_t)(k / (uint64_t)tr.ntx);
-      const int64_t ox = (int64_t)tx * d.tw, oy = (int64_t)ty * d.th;
-      const int64_t x0 = (tr.lx > ox ? tr.lx : ox) - ox, x1 = (tr.hx < ox + d.tw - 1 ? tr.hx : ox + d.tw - 1) - ox;
-      const int64_t y0 = (tr.ly > oy ? tr.ly : oy) - oy, y1 = (tr.hy < oy + d.th - 1 ? tr.hy : oy + d.th - 1) - oy;
-      keys[base + k] = (uint32_t)ty * (uint32_t)d.ntx + (uint32_t)tx;
-      payload[base + k] = pack_entry(task, pv, d.ndim, (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
+    for (uint32_t k = 0, i = 0, j = 0; k < cnt; ++k) {
+      put(base + k, tile0, (int)i, (int)j, ntx, nty, fx, lx, fy, ly, task, pv);
+      if (++i == (uint32_t)ntx) {
+        i = 0;
+        ++j;
+      }
     }
   }
-  unsigned shared = __ballot_sync(0xffffffffu, valid && !own && cnt > 0);
+  unsigned shared = __ballot_sync(0xffffffffu, valid && !own);
   while (shared) {
-    const int i = __ffs((int)shared) - 1;
+    const int s = __ffs((int)shared) - 1;
     shared &= shared - 1;
-    uint64_t c = __shfl_sync(0xffffffffu, cnt, i);
-    uint64_t b = __shfl_sync(0xffffffffu, base, i);
-    int64_t lx = __shfl_sync(0xffffffffu, tr.lx, i), hx = __shfl_sync(0xffffffffu, tr.hx, i);
-    int64_t ly = __shfl_sync(0xffffffffu, tr.ly, i), hy = __shfl_sync(0xffffffffu, tr.hy, i);
-    int32_t tx0 = __shfl_sync(0xffffffffu, tr.tx0, i), ty0 = __shfl_sync(0xffffffffu, tr.ty0, i);
-    int32_t ntx = __shfl_sync(0xffffffffu, tr.ntx, i);
-    uint32_t tk = __shfl_sync(0xffffffffu, task, i), p = __shfl_sync(0xffffffffu, pv, i);
-    for (uint64_t k = lane; k < c; k += 32) {
-      int32_t tx = tx0 + (int32_t)(k % (uint64_t)ntx);
-      int32_t ty = ty0 + (int32_t)(k / (uint64_t)ntx);
-      int64_t ox = (int64_t)tx * d.tw, oy = (int64_t)ty * d.th;
-      int64_t x0 = (lx > ox ? lx : ox) - ox, x1 = (hx < ox + d.tw - 1 ? hx : ox + d.tw - 1) - ox;
-      int64_t y0 = (ly > oy ? ly : oy) - oy, y1 = (hy < oy + d.th - 1 ? hy : oy + d.th - 1) - oy;
-      keys[b + k] = (uint32_t)ty * (uint32_t)d.ntx + (uint32_t)tx;
-      payload[b + k] = pack_entry(tk, p, d.ndim, (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
+    const uint32_t c = __shfl_sync(0xffffffffu, cnt, s), b = __shfl_sync(0xffffffffu, base, s);
+    const uint32_t t0 = __shfl_sync(0xffffffffu, tile0, s);
+    const int nx = __shfl_sync(0xffffffffu, ntx, s), ny = __shfl_sync(0xffffffffu, nty, s);
+    const int x0 = __shfl_sync(0xffffffffu, fx, s), x1 = __shfl_sync(0xffffffffu, lx, s);
+    const int y0 = __shfl_sync(0xffffffffu, fy, s), y1 = __shfl_sync(0xffffffffu, ly, s);
+    const uint32_t tk = __shfl_sync(0xffffffffu, task, s), p = __shfl_sync(0xffffffffu, pv, s);
+    const int dj = 32 / nx, di = 32 - dj * nx;  // 32 entries further
+    int j = lane / nx, i = lane - j * nx;
+    for (uint32_t k = (uint32_t)lane; k < c; k += 32) {
+      put(b + k, t0, i, j, nx, ny, x0, x1, y0, y1, tk, p);
+      i += di;
+      j += dj;
+      if (i >= nx) {
+        i -= nx;
+        ++j;
+      }
     }
   }
 }
@@ -614,7 +683,7 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 void launch_validate(const int32_t* req_off, int32_t n, int64_t r_first, const int64_t* lo,
-                     const int64_t* hi, const uint8_t* priv, int64_t R, const int32_t* pred_off,
+                     const int64_t* hi, const uint8_t* priv, int64_t R, bool rects_checked, const int32_t* pred_off,
                      const int32_t* pred, int64_t p_first, int64_t p_end, int32_t task_base,
                      const int32_t* body_arg, int64_t body_limit, AnalysisDims d, uint32_t* err,
                      cudaStream_t s) {
@@ -622,7 +691,7 @@ void launch_validate(const int32_t* req_off, int32_t n, int64_t r_first, const i
   k_validate_tasks<<<nblk((int64_t)n + 1, 256), 256, 0, s>>>(req_off, n, r_first, r_first + R, pred_off,
                                                            pred, p_first, p_end, task_base, body_arg,
                                                            body_limit, err);
-  if (R > 0) {
+  if (R > 0 && !rects_checked) {
     count_launch();
     k_validate_rects<<<nblk(R, 256), 256, 0, s>>>(lo, hi, priv, R, d, err);
   }
@@ -646,6 +715,23 @@ void launch_widen_bounds(const int32_t* lo32, const int32_t* hi32, int64_t m, in
   k_widen_bounds<<<blocks, 256, 0, s>>>(lo32, hi32, m, lo, hi);
 }
 
+template <class T>
+void launch_ingest_rects(const T* lo_in, const T* hi_in, const uint8_t* priv_in, int64_t R, AnalysisDims d, int64_t* lo,
+                         int64_t* hi, uint8_t* priv, uint32_t* err, cudaStream_t s) {
+  if (R <= 0) return;
+  count_launch();
+  const uintptr_t at = reinterpret_cast<uintptr_t>(lo_in) | reinterpret_cast<uintptr_t>(hi_in);
+  const uintptr_t to = reinterpret_cast<uintptr_t>(lo) | reinterpret_cast<uintptr_t>(hi);
+  if (d.ndim == 2 && at % (2 * sizeof(T)) == 0 && to % 16 == 0)
+    k_ingest_rects<T, true><<<nblk(R, 256), 256, 0, s>>>(lo_in, hi_in, priv_in, R, d, lo, hi, priv, err);
+  else
+    k_ingest_rects<T, false><<<nblk(R, 256), 256, 0, s>>>(lo_in, hi_in, priv_in, R, d, lo, hi, priv, err);
+}
+template void launch_ingest_rects<int32_t>(const int32_t*, const int32_t*, const uint8_t*, int64_t, AnalysisDims,
+                                           int64_t*, int64_t*, uint8_t*, uint32_t*, cudaStream_t);
+template void launch_ingest_rects<int64_t>(const int64_t*, const int64_t*, const uint8_t*, int64_t, AnalysisDims,
+                                           int64_t*, int64_t*, uint8_t*, uint32_t*, cudaStream_t);
+
 void launch_add_offset(int32_t* a, int64_t n, int32_t add, cudaStream_t s) {
   if (n > 0 && add != 0) {
     count_launch();
@@ -654,7 +740,7 @@ void launch_add_offset(int32_t* a, int64_t n, int32_t add, cudaStream_t s) {
 }
 
 void launch_bin_count(const int32_t* req_off, int32_t n, int64_t R, const int64_t* lo, const int64_t* hi,
-                      AnalysisDims d, int32_t* rect_task, uint64_t* cnt, unsigned long long* area,
+                      AnalysisDims d, int32_t* rect_task, uint32_t* cnt, unsigned long long* area,
                       uint32_t* zero, cudaStream_t s) {
   if (n > 0) {
     count_launch();
@@ -663,7 +749,7 @@ void launch_bin_count(const int32_t* req_off, int32_t n, int64_t R, const int64_
 }
 
 void launch_bin_expand(const int32_t* rect_task, const int64_t* lo, const int64_t* hi,
-                       const uint8_t* priv, int64_t R, const uint64_t* off, AnalysisDims d,
+                       const uint8_t* priv, int64_t R, const uint32_t* off, AnalysisDims d,
                        uint32_t* keys, uint64_t* payload, cudaStream_t s) {
   if (R > 0) {
     count_launch();
@@ -772,6 +858,10 @@ void preload_analysis() {
   cudaFuncGetAttributes(&a, k_report);
   cudaFuncGetAttributes(&a, k_band_place);
   cudaFuncGetAttributes(&a, k_widen_bounds);
+  cudaFuncGetAttributes(&a, k_ingest_rects<int32_t, false>);
+  cudaFuncGetAttributes(&a, k_ingest_rects<int32_t, true>);
+  cudaFuncGetAttributes(&a, k_ingest_rects<int64_t, false>);
+  cudaFuncGetAttributes(&a, k_ingest_rects<int64_t, true>);
   cudaFuncGetAttributes(&a, k_bucket_count);
   cudaFuncGetAttributes(&a, k_bucket_maxrow);
   cudaFuncGetAttributes(&a, k_bucket_scatter);

@@ -314,6 +314,11 @@ rt_status check_desc(const rt_graph_desc* d, AnalysisDims* out, int64_t* ncells)
   if (ntx * nty > (1ll << 26)) return fail(RT_ERR_INVALID, "domain has more than 2^26 tiles; use a larger tile");
   a.ntx = (int)ntx;
   a.nty = (int)nty;
+  a.shx = a.shy = -1;
+  if ((a.tw & (a.tw - 1)) == 0 && (a.th & (a.th - 1)) == 0) {
+    a.shx = bits_for((uint64_t)(a.tw - 1));
+    a.shy = bits_for((uint64_t)(a.th - 1));
+  }
   int64_t cells = a.ext[0] * a.ext[1];
   if (d->body == RT_BODY_CHECK) {
     if (!d->state || d->state_elems < cells)
@@ -476,6 +481,18 @@ bool kernel_reads(const void* p) {
   return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
+// The word that a batch's device checks report to: word 0 gathers the deferred
+// checks' findings until the analysis, word 1 is one call's own.
+rt_status ready_err(rt_graph* g, bool now, uint32_t** err) {
+  if (!g->err.p) {
+    CKR(g->err.reserve(256, g->s));
+    CK(cudaMemsetAsync(g->err.p, 0, 4, g->s));
+  }
+  *err = g->err.as<uint32_t>() + (now ? 1 : 0);
+  if (now) CK(cudaMemsetAsync(*err, 0, 4, g->s));
+  return RT_OK;
+}
+
 rt_status ensure_pinned(rt_graph* g) {
   if (g->hpin) return RT_OK;
   CK(cudaMallocHost(&g->hpin, 1024));
@@ -586,6 +603,8 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
   const int32_t n0 = g->n;
   const int64_t R0 = g->R, P0 = g->P;
   const bool had_pred = g->has_pred, had_body_arg = g->has_body_arg;
+  uint32_t* err = nullptr;     // where this batch's device checks report
+  bool rects_checked = false;  // ... its rectangles already have
   // offsets: position 0 of the batch is the previous end, so copy [1..n] (a
   // first batch's own 0 with them)
   CKR(g->req_off.reserve((size_t)(n0 + n + 1) * 4, s, (size_t)(n0 + 1) * 4));
@@ -596,18 +615,42 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     CKR(g->lo.reserve((size_t)(R0 + R) * D * 8, s, (size_t)R0 * D * 8));
     CKR(g->hi.reserve((size_t)(R0 + R) * D * 8, s, (size_t)R0 * D * 8));
     CKR(g->priv.reserve((size_t)(R0 + R), s, (size_t)R0));
-    if (c32) {
-      // the int32 bounds through a staging buffer, widened into the graph's arrays
+    int64_t* const dlo = g->lo.as<int64_t>() + R0 * D;
+    int64_t* const dhi = g->hi.as<int64_t>() + R0 * D;
+    uint8_t* const dpriv = g->priv.as<uint8_t>() + R0;
+    // read where they are, when a kernel may
+    const bool direct = dev && kernel_reads(lo) && kernel_reads(hi) && kernel_reads(priv);
+    const bool check = (on_device_check || check_now) && !bp;  // a placed batch is checked after its placement
+    if (check) CKR(ready_err(g, check_now, &err));
+    const void *from_lo = lo, *from_hi = hi;
+    const uint8_t* from_priv = priv;
+    if (c32 && !direct) {  // the int32 bounds through a staging buffer
       CKR(g->stage32.reserve((size_t)R * D * 8, s));
       int32_t* st = g->stage32.as<int32_t>();
       CKR(copy_in(st, lo, (size_t)R * D * 4, s));
       CKR(copy_in(st + R * D, hi, (size_t)R * D * 4, s));
-      launch_widen_bounds(st, st + R * D, R * D, g->lo.as<int64_t>() + R0 * D, g->hi.as<int64_t>() + R0 * D, s);
-    } else {
-      CKR(copy_in(g->lo.as<int64_t>() + R0 * D, lo, (size_t)R * D * 8, s));
-      CKR(copy_in(g->hi.as<int64_t>() + R0 * D, hi, (size_t)R * D * 8, s));
+      CKR(copy_in(dpriv, priv, (size_t)R, s));
+      from_lo = st;
+      from_hi = st + R * D;
+      from_priv = dpriv;
     }
-    CKR(copy_in(g->priv.as<uint8_t>() + R0, priv, (size_t)R, s));
+    if (check && (c32 || direct)) {
+      if (c32)
+        launch_ingest_rects(static_cast<const int32_t*>(from_lo), static_cast<const int32_t*>(from_hi), from_priv, R,
+                            g->dims, dlo, dhi, dpriv, err, s);
+      else
+        launch_ingest_rects(static_cast<const int64_t*>(from_lo), static_cast<const int64_t*>(from_hi), from_priv, R,
+                            g->dims, dlo, dhi, dpriv, err, s);
+      rects_checked = true;
+    } else {
+      if (c32) {
+        launch_widen_bounds(static_cast<const int32_t*>(from_lo), static_cast<const int32_t*>(from_hi), R * D, dlo, dhi, s);
+      } else {
+        CKR(copy_in(dlo, lo, (size_t)R * D * 8, s));
+        CKR(copy_in(dhi, hi, (size_t)R * D * 8, s));
+      }
+      if (from_priv == priv) CKR(copy_in(dpriv, priv, (size_t)R, s));
+    }
   }
   if (pred_off || g->has_pred) {
     CKR(g->pred_off.reserve((size_t)(n0 + n + 1) * 4, s, g->has_pred ? (size_t)(n0 + 1) * 4 : 0));
@@ -636,20 +679,13 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     g->has_body_arg = true;
   }
   if (on_device_check || check_now) {
-    if (!g->err.p) {
-      CKR(g->err.reserve(256, s));
-      CK(cudaMemsetAsync(g->err.p, 0, 4, s));
-    }
-    // word 0 gathers the deferred checks' findings until the analysis, word 1 is
-    // this call's own
-    uint32_t* err = g->err.as<uint32_t>() + (check_now ? 1 : 0);
-    if (check_now) CK(cudaMemsetAsync(err, 0, 4, s));
+    if (!err) CKR(ready_err(g, check_now, &err));
     if (bp)  // each rectangle checked against its own graph's domain, then moved into its band
       launch_band_place(g->req_off.as<int32_t>() + n0, n, bp->task_first, bp->G, bp->box, D,
-                        g->lo.as<int64_t>() + R0 * D, g->hi.as<int64_t>() + R0 * D, R, g->err.as<uint32_t>(), s);
+                        g->lo.as<int64_t>() + R0 * D, g->hi.as<int64_t>() + R0 * D, R, err, s);
     const int64_t limit = g->desc.body == RT_BODY_COUNTER ? g->desc.state_elems : -1;
     launch_validate(g->req_off.as<int32_t>() + n0, n, R0, g->lo.as<int64_t>() + R0 * D,
-                    g->hi.as<int64_t>() + R0 * D, g->priv.as<uint8_t>() + R0, R,
+                    g->hi.as<int64_t>() + R0 * D, g->priv.as<uint8_t>() + R0, R, rects_checked,
                     g->has_pred ? g->pred_off.as<int32_t>() + n0 : nullptr, g->pred.as<int32_t>(), P0,
                     P0 + Pb, n0, body_arg ? g->body_arg.as<int32_t>() + n0 : nullptr, limit, g->dims,
                     err, s);
@@ -710,7 +746,8 @@ rt_status run_analysis(rt_graph* g) {
   uint32_t* tile_counter = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 64);
   // control words, zeroed above: 0 the pair cursor, 64 and 68 tile counters, 96
   // tiles left by the sweep by windows, 100 the longest row, 104 long rows, 128
-  // pairs of the tiles to sweep again, 160 the rectangles' cells, 192
+  // pairs of the tiles to sweep again, 160 and 168 the rectangles' cells
+  // and tiles, 192
   // the largest out-degree, the longest edge and the last root
   uint32_t* nbail = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 96);
   uint32_t* bmax = reinterpret_cast<uint32_t*>(g->misc.as<char>() + 100);
@@ -737,16 +774,16 @@ rt_status run_analysis(rt_graph* g) {
   uint8_t *flags1 = nullptr, *flags2 = nullptr;
   if (R > 0) {
     CKR(g->rect_task.reserve((size_t)R * 4, s));
-    CKR(g->cnt.reserve((size_t)(R + 1) * 8, s));
-    CKR(reserve_ws(g, scan_ws_elems<uint64_t>(R) * 8));
+    CKR(g->cnt.reserve((size_t)(R + 1) * 4, s));
+    CKR(reserve_ws(g, scan_ws_elems<uint32_t>(R) * 4));
     launch_bin_count(g->req_off.as<int32_t>(), n, R, g->lo.as<int64_t>(), g->hi.as<int64_t>(), d,
-                     g->rect_task.as<int32_t>(), g->cnt.as<uint64_t>(), area, bcnt, s);
-    scan_exclusive<uint64_t>(g->cnt.as<uint64_t>(), g->cnt.as<uint64_t>(), R, g->ws.as<uint64_t>(), s);
+                     g->rect_task.as<int32_t>(), g->cnt.as<uint32_t>(), area, bcnt, s);
+    scan_exclusive<uint32_t>(g->cnt.as<uint32_t>(), g->cnt.as<uint32_t>(), R, g->ws.as<uint32_t>(), s);
   }
   h64[1] = 0;
   ReportArgs ra1;
   if (R > 0) {
-    ra1.add((void*)&h64[0], g->cnt.as<uint64_t>() + R, true);
+    ra1.add((void*)&h64[0], area + 1, true);
     ra1.add((void*)&h64[4], area, true);
   }
   if (g->pending_validate) ra1.add((void*)&h64[1], g->err.p);
@@ -773,7 +810,7 @@ rt_status run_analysis(rt_graph* g) {
     CKR(reserve_ws(g, radix_ws_bytes(M)));
     trace("analyze: entry buffers reserved");
     launch_bin_expand(g->rect_task.as<int32_t>(), g->lo.as<int64_t>(), g->hi.as<int64_t>(),
-                      g->priv.as<uint8_t>(), R, g->cnt.as<uint64_t>(), d, g->keys.as<uint32_t>(),
+                      g->priv.as<uint8_t>(), R, g->cnt.as<uint32_t>(), d, g->keys.as<uint32_t>(),
                       g->pay.as<uint64_t>(), s);
     if (prof) CK(cudaEventRecord(g->ev[EV_BIN], s));
     const int tbits = std::max(bits_for((uint64_t)(ntiles - 1)), 1);

@@ -303,10 +303,11 @@ struct AnalysisDims {
   int64_t ext[2];
   int tw, th;
   int ntx, nty;
+  int shx, shy;  // log2 of tw and th where both are powers of two, else -1
 };
 
 void launch_validate(const int32_t* req_off, int32_t n, int64_t r_first, const int64_t* lo,
-                     const int64_t* hi, const uint8_t* priv, int64_t R, const int32_t* pred_off,
+                     const int64_t* hi, const uint8_t* priv, int64_t R, bool rects_checked, const int32_t* pred_off,
                      const int32_t* pred, int64_t p_first, int64_t p_end, int32_t task_base,
                      const int32_t* body_arg, int64_t body_limit, AnalysisDims d, uint32_t* err,
                      cudaStream_t s);
@@ -314,15 +315,19 @@ void launch_add_offset(int32_t* a, int64_t n, int32_t add, cudaStream_t s);
 // lo[i] = lo32[i], hi[i] = hi32[i] for i < m
 void launch_widen_bounds(const int32_t* lo32, const int32_t* hi32, int64_t m, int64_t* lo, int64_t* hi,
                          cudaStream_t s);
+// a batch's rectangles into the graph's arrays, widened and checked in one pass
+template <class T>
+void launch_ingest_rects(const T* lo_in, const T* hi_in, const uint8_t* priv_in, int64_t R, AnalysisDims d, int64_t* lo,
+                         int64_t* hi, uint8_t* priv, uint32_t* err, cudaStream_t s);
 // rt_batch_capture: checks every rectangle against its graph's own domain and
 // moves it into the graph's band (box: int64 [G][3][ndim] = lo, hi, shift)
 void launch_band_place(const int32_t* req_off, int32_t n, const int32_t* task_first, int32_t G, const int64_t* box,
                        int D, int64_t* lo, int64_t* hi, int64_t R, uint32_t* err, cudaStream_t s);
 void launch_bin_count(const int32_t* req_off, int32_t n, int64_t R, const int64_t* lo, const int64_t* hi,
-                      AnalysisDims d, int32_t* rect_task, uint64_t* cnt, unsigned long long* area,
+                      AnalysisDims d, int32_t* rect_task, uint32_t* cnt, unsigned long long* area,
                       uint32_t* zero, cudaStream_t s);
 void launch_bin_expand(const int32_t* rect_task, const int64_t* lo, const int64_t* hi,
-                       const uint8_t* priv, int64_t R, const uint64_t* off, AnalysisDims d,
+                       const uint8_t* priv, int64_t R, const uint32_t* off, AnalysisDims d,
                        uint32_t* keys, uint64_t* payload, cudaStream_t s);
 void launch_segments(const uint32_t* keys, int64_t M, int64_t ntiles, uint32_t* seg_begin, uint32_t* seg_end,
                      cudaStream_t s);

@@ -238,9 +238,7 @@ void scan_zeros(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* ws, cuda
 }
 
 template size_t scan_ws_elems<uint32_t>(int64_t);
-template size_t scan_ws_elems<uint64_t>(int64_t);
 template void scan_exclusive<uint32_t>(const uint32_t*, uint32_t*, int64_t, uint32_t*, cudaStream_t);
-template void scan_exclusive<uint64_t>(const uint64_t*, uint64_t*, int64_t, uint64_t*, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // radix sort
@@ -458,13 +456,10 @@ void preload_primitives() {
   cudaFuncAttributes a;
   cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t, false>);
   cudaFuncGetAttributes(&a, k_scan_reduce<uint32_t, true>);
-  cudaFuncGetAttributes(&a, k_scan_reduce<uint64_t, false>);
   cudaFuncGetAttributes(&a, k_scan_down<uint32_t, false>);
   cudaFuncGetAttributes(&a, k_scan_down<uint32_t, true>);
-  cudaFuncGetAttributes(&a, k_scan_down<uint64_t, false>);
   cudaFuncGetAttributes(&a, k_scan_one<uint32_t, false>);
   cudaFuncGetAttributes(&a, k_scan_one<uint32_t, true>);
-  cudaFuncGetAttributes(&a, k_scan_one<uint64_t, false>);
   cudaFuncGetAttributes(&a, k_radix_hist<uint32_t>);
   cudaFuncGetAttributes(&a, k_radix_hist<uint64_t>);
   cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, true>);
