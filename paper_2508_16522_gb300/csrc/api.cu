@@ -722,6 +722,8 @@ namespace {
 // (without the pair filter) least mean entries per tile
 constexpr double kWindowCover = 0.2;
 constexpr int kWindowTileEntries = 64;
+// the tile sweep: mean cells an entry up to which it keeps every cell
+constexpr double kPlainCells = 4.0;
 
 rt_status reserve_ws(rt_graph* g, size_t bytes) { return g->ws.reserve(bytes + 1024, g->s); }
 
@@ -869,6 +871,10 @@ rt_status run_analysis(rt_graph* g) {
   const double cover = M > 0 ? (double)h64[4] / ((double)M * d.tw * d.th) : 0.0;
   const bool by_windows = M > 0 && cover >= kWindowCover && (fbits > 0 || M >= (int64_t)kWindowTileEntries * ntiles);
   if (by_windows && !fbits) guess *= 2;
+  // entries of a few cells each need no classes (at most one in 64 can then cover
+  // a 256-cell tile), unless the tiles hold so few that clearing all cells costs more
+  const bool plain = M > 0 && (double)h64[4] <= kPlainCells * (double)M && d.tw * d.th <= kMaxClassCells &&
+                     8 * M >= ntiles * (int64_t)(d.tw * d.th);
   int wblocks = 0, wspan = 16;
   uint32_t wchunk = 1;
   if (by_windows) {
@@ -926,7 +932,7 @@ rt_status run_analysis(rt_graph* g) {
       }
       if (fbits) CK(cudaMemsetAsync(g->pfilt.p, 0xFF, ((size_t)n << fslots) * 4, s));
       SweepOut o{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, nullptr, flags1, rerun,
-                 fbits ? g->pfilt.as<uint32_t>() : nullptr, fslots};
+                 fbits ? g->pfilt.as<uint32_t>() : nullptr, fslots, plain};
       if (prof) CK(cudaEventRecord(g->ev[EV_SW0], s));
       if (win) {
         SweepOut ow = o;
@@ -964,7 +970,7 @@ rt_status run_analysis(rt_graph* g) {
       CK(cudaMemsetAsync(tile_counter, 0, 4, s));
       // the rerun writes every pair its tiles find: no filter (a pair whose
       // first write fell past the buffer's end may already sit in it)
-      SweepOut o2{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, flags1, flags2, rerun, nullptr, 0};
+      SweepOut o2{g->pairs.as<uint64_t>(), cap, cursor, tile_counter, B, chunk, flags1, flags2, rerun, nullptr, 0, plain};
       launch_sweep(spay, seg_b, seg_e, d, o2, sweep_blocks, s);
       if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
       CK(cudaGetLastError());

@@ -346,6 +346,10 @@ struct SweepOut {
   // they find
   uint32_t* filt;
   int filt_bits;
+  // rectangles of a few cells (and a tile whose cells fit the state): no classes,
+  // which would cost two passes over every tile's entries to find (random 1024 x
+  // 1000 Task Bench graph: sweep 0.233 -> 0.215 ms)
+  bool plain_cells;
 };
 int sweep_warps_per_block(int tw, int th);
 size_t sweep_smem_bytes(int tw, int th, int warps);

@@ -1066,6 +1066,10 @@ __global__ void __launch_bounds__(256, 3) k_sweep(const uint64_t* __restrict__ p
   // row mode runs in 2-D segment tiles, whose class columns the tables cover
   const bool rowmode = d.ndim == 2 && row_table_bytes(d.tw) > 0;
   for (int i = lane; i < kHashSlots; i += 32) w.htab[i] = -1;
+  if (o.plain_cells) {  // every cell its own class
+    for (int i = lane; i < d.tw; i += 32) w.cmx[i] = (uint16_t)i;
+    for (int i = lane; i < d.th; i += 32) w.cmy[i] = (uint16_t)i;
+  }
   if (lane == 0) {
     *w.hcount = 0;
     *w.dropped = 0;
@@ -1091,32 +1095,37 @@ __global__ void __launch_bounds__(256, 3) k_sweep(const uint64_t* __restrict__ p
     if (o.only && !o.only[t]) continue;  // a rerun sweeps the tiles that dropped pairs
     x.L = payload + sb;
     x.n = (int)(se - sb);
-    // class maps of this tile: mark every rectangle boundary inside it, then
-    // number the classes by a prefix sum
-    for (int i = lane; i < d.tw; i += 32) w.cmx[i] = 0;
-    for (int i = lane; i < d.th; i += 32) w.cmy[i] = 0;
-    __syncwarp();
-    for (int k = lane; k < x.n; k += 32) {
-      const Box b = unpack_entry(x.L[k], x.ndim);
-      if (b.x0 > 0) w.cmx[b.x0] = 1;
-      if (b.x1 + 1 < d.tw) w.cmx[b.x1 + 1] = 1;
-      if (b.y0 > 0) w.cmy[b.y0] = 1;
-      if (b.y1 + 1 < d.th) w.cmy[b.y1 + 1] = 1;
-    }
-    __syncwarp();
-    scan_flags(w.cmx, d.tw, lane);
-    scan_flags(w.cmy, d.th, lane);
-    const int cw = w.cmx[d.tw - 1] + 1, ch = w.cmy[d.th - 1] + 1;
-    x.tw = cw;  // row stride of the class grid
-    // segment mode when the candidates cover many classes each
-    unsigned long long area = 0;
-    for (int k = lane; k < x.n; k += 32) {
-      const Box b = unpack_entry(x.L[k], x.ndim);
-      area += (unsigned long long)(w.cmx[b.x1] - w.cmx[b.x0] + 1) * (unsigned long long)(w.cmy[b.y1] - w.cmy[b.y0] + 1);
-    }
+    int cw = d.tw, ch = d.th;
+    x.segmode = false;
+    if (!o.plain_cells) {
+      // class maps of this tile: mark every rectangle boundary inside it, then
+      // number the classes by a prefix sum
+      for (int i = lane; i < d.tw; i += 32) w.cmx[i] = 0;
+      for (int i = lane; i < d.th; i += 32) w.cmy[i] = 0;
+      __syncwarp();
+      for (int k = lane; k < x.n; k += 32) {
+        const Box b = unpack_entry(x.L[k], x.ndim);
+        if (b.x0 > 0) w.cmx[b.x0] = 1;
+        if (b.x1 + 1 < d.tw) w.cmx[b.x1 + 1] = 1;
+        if (b.y0 > 0) w.cmy[b.y0] = 1;
+        if (b.y1 + 1 < d.th) w.cmy[b.y1 + 1] = 1;
+      }
+      __syncwarp();
+      scan_flags(w.cmx, d.tw, lane);
+      scan_flags(w.cmy, d.th, lane);
+      cw = w.cmx[d.tw - 1] + 1;
+      ch = w.cmy[d.th - 1] + 1;
+      // segment mode when the candidates cover many classes each
+      unsigned long long area = 0;
+      for (int k = lane; k < x.n; k += 32) {
+        const Box b = unpack_entry(x.L[k], x.ndim);
+        area += (unsigned long long)(w.cmx[b.x1] - w.cmx[b.x0] + 1) * (unsigned long long)(w.cmy[b.y1] - w.cmy[b.y0] + 1);
+      }
 #pragma unroll
-    for (int o2 = 16; o2 >= 1; o2 >>= 1) area += __shfl_xor_sync(kFull, area, o2);
-    x.segmode = area >= (unsigned long long)kSegMinArea * (unsigned long long)x.n;
+      for (int o2 = 16; o2 >= 1; o2 >>= 1) area += __shfl_xor_sync(kFull, area, o2);
+      x.segmode = area >= (unsigned long long)kSegMinArea * (unsigned long long)x.n;
+    }
+    x.tw = cw;  // row stride of the class grid
     // a class grid larger than the cell state is swept in strips of class
     // rows, each pass over every candidate (those outside see empty boxes)
     const int cap = class_cap(d.tw, d.th);

@@ -1,5 +1,6 @@
-"""The sweep by windows (dense inputs): the CSR equals the oracle's where the
-windows can go wrong -- tile shapes on both sides of 32 columns and rows, 1-D
+"""The sweep by windows (dense inputs), and the tile sweep without classes
+(rectangles of a few cells): the CSR equals the oracle's where they can go
+wrong -- tile shapes on both sides of 32 columns and rows, 1-D
 tiles, windows cut inside a task of many rectangles, tasks of more candidates
 than a window takes, runs of readers longer than a walk, thinly covered domain
 borders, and more distinct pairs than the buffer's first guess."""
@@ -53,7 +54,23 @@ def long_runs(readers, seed):
     return _boxes(2, (24, 24), np.ones(len(priv), np.int64), boxes, priv, f"runs{readers}")
 
 
+def few_large(seed):
+    """Boxes of one or two cells, one in a thousand the whole domain: the tile
+    sweep that keeps every cell its own class."""
+    rng = np.random.default_rng(seed)
+    boxes, priv = [], []
+    for k in range(4000):
+        x, y = rng.integers(0, 45, 2)
+        boxes.append([[0, 0], [47, 39]] if k % 1000 == 7 else [[x, min(y, 39)], [min(x + rng.integers(0, 2), 47), min(y, 39)]])
+        priv.append(rng.choice(3, p=(0.6, 0.3, 0.1)))
+    counts = rng.integers(1, 4, 4000)
+    counts = counts[:int(np.searchsorted(np.cumsum(counts), 4000))]
+    counts = np.append(counts, 4000 - counts.sum())
+    return _boxes(2, (48, 40), counts, boxes, priv, f"few_large{seed}")
+
+
 CASES = [
+    ("few_large", lambda: few_large(6), [(16, 16), (8, 8), (32, 4), (48, 20), (7, 9)]),
     ("tiles", lambda: dense((200, 168), 700, (4, 90), 3), [(16, 16), (16, 32), (32, 32), (32, 4), (33, 31), (64, 64), (128, 16)]),
     ("thin", lambda: dense((256, 256), 1500, (20, 120), 5, probs=(0.9, 0.02, 0.08)), [(16, 16), (32, 32), (64, 32)]),
     ("ragged", lambda: dense((97, 1), 400, (1, 60), 7), [(16, 16), (32, 1), (97, 1)]),
