@@ -15,6 +15,7 @@
 
 #include <mutex>
 #include <set>
+#include <type_traits>
 
 #include "grt_internal.cuh"
 
@@ -246,26 +247,31 @@ template void scan_exclusive<uint32_t>(const uint32_t*, uint32_t*, int64_t, uint
 namespace {
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / 32;
-constexpr int kRadixIpt = 16;                                 // keys per thread
-constexpr int kRadixTile = kRadixThreads * kRadixIpt;         // 4096 keys per block
-constexpr int kRadixWarpKeys = kRadixTile / kRadixWarps;      // 512 keys per warp
+// Keys per thread: 16 (4096 a block), or 4 for small sorts, whose few blocks are
+// a chain of ranking rounds each (6200 keys: 13.9 us a pass with 16).
+constexpr int kRadixIpt = 16, kRadixIptSmall = 4;
+constexpr int64_t kRadixSmall = 96 * kRadixThreads * kRadixIptSmall;  // its digit counts still fit one scan block
+inline int64_t radix_blocks(int64_t n) {
+  const int64_t tile = kRadixThreads * (n <= kRadixSmall ? kRadixIptSmall : kRadixIpt);
+  return (n + tile - 1) / tile;
+}
 
-template <typename K>
+template <typename K, int IPT>
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const K* keys, int64_t n, int shift,
                                                              uint32_t mask, uint32_t* hist,
                                                              int64_t nblocks) {
   __shared__ uint32_t h[256];
   h[threadIdx.x] = 0;
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-  K kv[kRadixIpt];
+  const int64_t base = (int64_t)blockIdx.x * (kRadixThreads * IPT);
+  K kv[IPT];
 #pragma unroll
-  for (int j = 0; j < kRadixIpt; ++j) {
+  for (int j = 0; j < IPT; ++j) {
     const int64_t k = base + j * kRadixThreads + threadIdx.x;
     kv[j] = k < n ? keys[k] : K(0);
   }
 #pragma unroll
-  for (int j = 0; j < kRadixIpt; ++j)
+  for (int j = 0; j < IPT; ++j)
     if (base + j * kRadixThreads + threadIdx.x < n) atomicAdd(&h[(uint32_t)(kv[j] >> shift) & mask], 1u);
   __syncthreads();
   hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
@@ -273,17 +279,17 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const K* keys, int
 
 // dynamic shared memory of one scatter block: its keys (and values) in
 // block-sorted order
-template <typename K, bool HAS_V>
+template <typename K, bool HAS_V, int IPT>
 constexpr size_t scatter_smem_bytes() {
-  return (size_t)kRadixTile * (sizeof(K) + (HAS_V ? sizeof(uint64_t) : 0));
+  return (size_t)(kRadixThreads * IPT) * (sizeof(K) + (HAS_V ? sizeof(uint64_t) : 0));
 }
 
-// One pass of the LSD radix sort over a block of kRadixTile keys: every key is
+// One pass of the LSD radix sort over a block of (kRadixThreads * IPT) keys: every key is
 // ranked within its warp and digit (match_any), the ranks become positions in
 // the block's digit-sorted order, the keys are reordered in shared memory, and
 // consecutive threads then write consecutive keys of each digit run to the
 // run's global offset, so the global writes are coalesced. Stable.
-template <typename K, bool HAS_V>
+template <typename K, bool HAS_V, int IPT>
 __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     const K* __restrict__ keys, const uint64_t* __restrict__ vals, K* __restrict__ keys_out,
     uint64_t* __restrict__ vals_out, int64_t n, int shift, uint32_t mask,
@@ -294,27 +300,27 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   __shared__ uint32_t wsum[kRadixWarps];
   extern __shared__ __align__(16) unsigned char rsmem[];
   K* sk = reinterpret_cast<K*>(rsmem);
-  uint64_t* sv = reinterpret_cast<uint64_t*>(rsmem + (size_t)kRadixTile * sizeof(K));
+  uint64_t* sv = reinterpret_cast<uint64_t*>(rsmem + (size_t)(kRadixThreads * IPT) * sizeof(K));
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int w = 0; w < kRadixWarps; ++w) wcnt[w][threadIdx.x] = 0;
   boff[threadIdx.x] = offs[(int64_t)threadIdx.x * nblocks + blockIdx.x];
   __syncthreads();
-  const int64_t wbase = (int64_t)blockIdx.x * kRadixTile + (int64_t)warp * kRadixWarpKeys;
-  K kv[kRadixIpt];
-  uint64_t vv[HAS_V ? kRadixIpt : 1];
-  uint32_t rk[kRadixIpt];
+  const int64_t wbase = (int64_t)blockIdx.x * (kRadixThreads * IPT) + (int64_t)warp * (32 * IPT);
+  K kv[IPT];
+  uint64_t vv[HAS_V ? IPT : 1];
+  uint32_t rk[IPT];
   const unsigned lt = lanemask_lt();
   // every key's load in flight before the ranking, whose warp barriers would hold
   // each round's loads back until the round before it is done (two passes over the
   // 343M entries of the 1M-launch trace: 9.9 -> 7.1 ms)
 #pragma unroll
-  for (int r = 0; r < kRadixIpt; ++r) {
+  for (int r = 0; r < IPT; ++r) {
     const int64_t idx = wbase + r * 32 + lane;
     kv[r] = idx < n ? keys[idx] : K(0);
   }
 #pragma unroll
-  for (int r = 0; r < kRadixIpt; ++r) {
+  for (int r = 0; r < IPT; ++r) {
     int64_t idx = wbase + r * 32 + lane;
     bool valid = idx < n;
     const K k = kv[r];
@@ -352,14 +358,14 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   if (threadIdx.x == kRadixThreads - 1) bstart[256] = wpre + incl;
   if (HAS_V) {
 #pragma unroll
-    for (int r = 0; r < kRadixIpt; ++r) {
+    for (int r = 0; r < IPT; ++r) {
       const int64_t idx = wbase + r * 32 + lane;
       vv[HAS_V ? r : 0] = idx < n ? vals[idx] : 0ull;
     }
   }
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < kRadixIpt; ++r) {
+  for (int r = 0; r < IPT; ++r) {
     int64_t idx = wbase + r * 32 + lane;
     if (idx < n) {
       const uint32_t d = (uint32_t)(kv[r] >> shift) & mask;
@@ -379,7 +385,7 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   }
 }
 
-template <typename K, bool HAS_V>
+template <typename K, bool HAS_V, int IPT>
 void launch_scatter(const K* kin, const uint64_t* vin, K* kout, uint64_t* vout, int64_t n, int shift, uint32_t mask,
                     const uint32_t* offs, int64_t nb, cudaStream_t s) {
   // above the default 48 KB of dynamic shared memory for some instantiations:
@@ -391,19 +397,19 @@ void launch_scatter(const K* kin, const uint64_t* vin, K* kout, uint64_t* vout, 
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!done.count(dev)) {
-      cudaFuncSetAttribute(k_radix_scatter<K, HAS_V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)scatter_smem_bytes<K, HAS_V>());
+      cudaFuncSetAttribute(k_radix_scatter<K, HAS_V, IPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)scatter_smem_bytes<K, HAS_V, IPT>());
       done.insert(dev);
     }
   }
   count_launch();
-  k_radix_scatter<K, HAS_V><<<(unsigned)nb, kRadixThreads, scatter_smem_bytes<K, HAS_V>(), s>>>(
+  k_radix_scatter<K, HAS_V, IPT><<<(unsigned)nb, kRadixThreads, scatter_smem_bytes<K, HAS_V, IPT>(), s>>>(
       kin, vin, kout, vout, n, shift, mask, offs, nb);
 }
 }  // namespace
 
 size_t radix_ws_bytes(int64_t n) {
-  int64_t nb = (n + kRadixTile - 1) / kRadixTile;
+  const int64_t nb = radix_blocks(n);
   int64_t h = 256 * (nb > 0 ? nb : 1);
   return (size_t)(2 * h + 1 + scan_ws_elems<uint32_t>(h)) * sizeof(uint32_t) + 256;
 }
@@ -412,7 +418,8 @@ template <typename K>
 int radix_sort(K* keys, K* keys_alt, uint64_t* vals, uint64_t* vals_alt, int64_t n, int nbits,
                void* ws, cudaStream_t s) {
   if (n <= 1 || nbits <= 0) return 0;
-  int64_t nb = (n + kRadixTile - 1) / kRadixTile;
+  const int64_t nb = radix_blocks(n);
+  const bool small = n <= kRadixSmall;
   int64_t h = 256 * nb;
   uint32_t* hist = (uint32_t*)ws;
   uint32_t* offs = hist + h;
@@ -425,14 +432,16 @@ int radix_sort(K* keys, K* keys_alt, uint64_t* vals, uint64_t* vals_alt, int64_t
   for (int shift = 0; shift < nbits; shift += 8) {
     int bits = nbits - shift < 8 ? nbits - shift : 8;
     uint32_t mask = (1u << bits) - 1u;
-    count_launch();
-    k_radix_hist<K><<<(unsigned)nb, kRadixThreads, 0, s>>>(kin, n, shift, mask, hist, nb);
-    scan_exclusive<uint32_t>(hist, offs, h, sws, s);
-    if (vals) {
-      launch_scatter<K, true>(kin, vin, kout, vout, n, shift, mask, offs, nb, s);
-    } else {
-      launch_scatter<K, false>(kin, nullptr, kout, nullptr, n, shift, mask, offs, nb, s);
-    }
+    auto pass = [&](auto ipt) {
+      constexpr int IPT = decltype(ipt)::value;
+      count_launch();
+      k_radix_hist<K, IPT><<<(unsigned)nb, kRadixThreads, 0, s>>>(kin, n, shift, mask, hist, nb);
+      scan_exclusive<uint32_t>(hist, offs, h, sws, s);
+      if (vals) launch_scatter<K, true, IPT>(kin, vin, kout, vout, n, shift, mask, offs, nb, s);
+      else launch_scatter<K, false, IPT>(kin, nullptr, kout, nullptr, n, shift, mask, offs, nb, s);
+    };
+    if (small) pass(std::integral_constant<int, kRadixIptSmall>());
+    else pass(std::integral_constant<int, kRadixIpt>());
     K* t = kin;
     kin = kout;
     kout = t;
@@ -460,12 +469,18 @@ void preload_primitives() {
   cudaFuncGetAttributes(&a, k_scan_down<uint32_t, true>);
   cudaFuncGetAttributes(&a, k_scan_one<uint32_t, false>);
   cudaFuncGetAttributes(&a, k_scan_one<uint32_t, true>);
-  cudaFuncGetAttributes(&a, k_radix_hist<uint32_t>);
-  cudaFuncGetAttributes(&a, k_radix_hist<uint64_t>);
-  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, true>);
-  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, false>);
-  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, true>);
-  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, false>);
+  cudaFuncGetAttributes(&a, k_radix_hist<uint32_t, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_hist<uint64_t, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_hist<uint32_t, kRadixIptSmall>);
+  cudaFuncGetAttributes(&a, k_radix_hist<uint64_t, kRadixIptSmall>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, true, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, false, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, true, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, false, kRadixIpt>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, true, kRadixIptSmall>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint32_t, false, kRadixIptSmall>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, true, kRadixIptSmall>);
+  cudaFuncGetAttributes(&a, k_radix_scatter<uint64_t, false, kRadixIptSmall>);
 }
 
 void preload_all() {
