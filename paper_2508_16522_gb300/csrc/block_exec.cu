@@ -371,7 +371,14 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
 // slot of a successor c was last used by c - S, which has run. So the graph may
 // have any number of tasks. The first unfinished task is always in a chunk its
 // owner holds (or may take), with its predecessors done: no warp waits forever.
-template <int WARPS, bool FENCE>
+//
+// WIDE: some task has successors past its trigger record (p.adjx). A graph without
+// loads half the bytes a chunk, sets up 5 successor slots instead of 13 and keeps
+// half the registers: 300 steps of a 600-wide stencil 285 -> 205 us, 32 wide with
+// 256 FMA 1000 steps 850 -> 818. The wide kernel still tests adjx itself, although
+// it is set: with those tests compiled out its schedule was worse (batch of 40
+// random graphs of 60k tasks, 20 replays: 3.95 ms instead of 3.75).
+template <int WARPS, bool FENCE, bool WIDE>
 __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_exec_window(ExecParams p, BlockArgs a,
                                                                                           int S) {
   extern __shared__ __align__(16) unsigned char wsmem[];
@@ -383,6 +390,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
   constexpr int T = WARPS * 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t mask = (uint32_t)S - 1u;
+  constexpr int NQ = WIDE ? 4 : 2, NS = WIDE ? kAdjWide : kAdjInline;  // a record's int4s and successors
   for (int i = tid; i < S + 32; i += T) count[i] = 0u;
   if (tid == 0) {
     s_status = 0u;
@@ -405,18 +413,18 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
     int32_t* const state = G.state;
     const int32_t* const body_arg = FENCE ? G.body_arg : nullptr;
     const int4* const adj = p.adj + 2 * (int64_t)base;
-    const int4* const adjx = p.adjx ? p.adjx + 2 * (int64_t)base : nullptr;
+    const int4* const adjx = WIDE && p.adjx ? p.adjx + 2 * (int64_t)base : nullptr;
     const int room = S - (a.order ? a.spans[gi] : a.span);
     for (int r = 0; r < p.replays; ++r) {
       if (lane == 0) held[warp] = warp * 32 < n ? (uint32_t)(warp * 32) : 0xFFFFFFFFu;
       if (tid == 0) s_done = 0u;
       __syncthreads();
       uint32_t oldest = 0;  // no task before it is unfinished
-      int4 nq[4];           // the next chunk's records
+      int4 nq[NQ];          // the next chunk's records
       int narg = 0;         // ... and counters
       auto fetch = [&](int v) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < NQ; ++k) {
           nq[k] = make_int4(0, 0, 0, -1);
           if (k > 0) nq[k].x = nq[k].y = nq[k].z = -1;
           if (v < n && (k < 2 || adjx)) nq[k] = __ldg(k < 2 ? adj + 2 * (int64_t)v + k : adjx + 2 * (int64_t)v + (k - 2));
@@ -438,9 +446,9 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
         // the lane's own spare word past the window, so that the additions below
         // need no branches (a divergent one a successor took 30 cycles each)
         const uint32_t spare = (uint32_t)S + (uint32_t)lane;
-        uint32_t succ[kAdjWide];
+        uint32_t succ[NS];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < NQ; ++k) {
           auto slot = [&](int t) -> uint32_t { return t >= 0 ? (uint32_t)(t - base) & mask : spare; };
           if (k > 0) {
             succ[4 * k - 3] = slot(nq[k].x);
@@ -504,7 +512,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
           if (FENCE) __threadfence_block();  // release: bodies before the counters
           // COMPLETED_EDGE
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
+          for (int k = 0; k < NQ; ++k) {
             if (4 * k - 3 < dmax && (k < 2 || adjx)) {  // uniform
 #pragma unroll
               for (int j = k > 0 ? 4 * k - 3 : 0; j <= 4 * k; ++j) atomicAdd(count + (ready ? succ[j] : spare), 1u);
@@ -598,8 +606,8 @@ void launch_block(const ExecParams& p, const BlockArgs& a, int32_t max_n, int bl
   else k_exec_block<WARPS, false><<<blocks, WARPS * 32, bytes, s>>>(p, a);
 }
 
-template <int WARPS>
-void launch_window_warps(const ExecParams& p, const BlockArgs& a, int S, int blocks, cudaStream_t s) {
+template <int WARPS, bool FENCE, bool WIDE>
+void launch_window_kernel(const ExecParams& p, const BlockArgs& a, int S, int blocks, cudaStream_t s) {
   static std::mutex mu;
   static std::set<int> done;
   int dev = 0;
@@ -607,16 +615,24 @@ void launch_window_warps(const ExecParams& p, const BlockArgs& a, int S, int blo
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!done.count(dev)) {
-      cudaFuncSetAttribute(k_exec_window<WARPS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (kWindowSlots + 32) * 4);
-      cudaFuncSetAttribute(k_exec_window<WARPS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(k_exec_window<WARPS, FENCE, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (kWindowSlots + 32) * 4);
       done.insert(dev);
     }
   }
   count_launch();
-  if (p.need_fence) k_exec_window<WARPS, true><<<blocks, WARPS * 32, ((size_t)S + 32) * 4, s>>>(p, a, S);
-  else k_exec_window<WARPS, false><<<blocks, WARPS * 32, ((size_t)S + 32) * 4, s>>>(p, a, S);
+  k_exec_window<WARPS, FENCE, WIDE><<<blocks, WARPS * 32, ((size_t)S + 32) * 4, s>>>(p, a, S);
+}
+
+template <int WARPS>
+void launch_window_warps(const ExecParams& p, const BlockArgs& a, int S, int blocks, cudaStream_t s) {
+  if (p.need_fence) {
+    if (p.adjx) launch_window_kernel<WARPS, true, true>(p, a, S, blocks, s);
+    else launch_window_kernel<WARPS, true, false>(p, a, S, blocks, s);
+  } else {
+    if (p.adjx) launch_window_kernel<WARPS, false, true>(p, a, S, blocks, s);
+    else launch_window_kernel<WARPS, false, false>(p, a, S, blocks, s);
+  }
 }
 }  // namespace
 
@@ -660,10 +676,14 @@ void launch_exec_block(ExecParams p, const BlockArgs& a, int32_t max_n, int bloc
 void preload_block_exec() {
   cudaFuncAttributes a;
   cudaFuncGetAttributes(&a, k_batch_shape);
-  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, false>);
-  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, true>);
-  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, false>);
-  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, true>);
+  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, false, false>);
+  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, false, true>);
+  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, true, false>);
+  cudaFuncGetAttributes(&a, k_exec_window<kBlockWarps, true, true>);
+  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, false, false>);
+  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, false, true>);
+  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, true, false>);
+  cudaFuncGetAttributes(&a, k_exec_window<kSmallWarps, true, true>);
   cudaFuncGetAttributes(&a, k_exec_block<kBlockWarps, false>);
   cudaFuncGetAttributes(&a, k_exec_block<kBlockWarps, true>);
   cudaFuncGetAttributes(&a, k_exec_block<kSmallWarps, false>);

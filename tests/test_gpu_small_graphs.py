@@ -61,6 +61,28 @@ def test_counter_chains_in_every_executor(n, counters, reach, extra):
     g.close()
 
 
+@pytest.mark.parametrize("body", [grt.RT_BODY_COUNTER, grt.RT_BODY_SPIN])
+@pytest.mark.parametrize("n,counters,reach,extra", [(3001, 60, 0, 0), (3001, 500, 0, 0), (3001, 50, 60, 40), (3001, 500, 600, 40)],
+                         ids=["small", "large", "small-wide", "large-wide"])
+def test_window_records(n, counters, reach, extra, body):
+    """Windows of both sizes, with and without successors past the trigger record."""
+    ensure_built()
+    tr = chains(n, counters, reach, seed=counters, extra=extra)
+    if body == grt.RT_BODY_SPIN:
+        g = gpu_graph(tr, body=body, spin_iters=9)
+        g.analyze()
+        g.replay(2)
+        g.sync()
+        assert np.array_equal(g.out.cpu().numpy()[:n], oracle.run_bodies(tr, body, spin_iters=9)[1])
+    else:
+        g = gpu_graph(tr, body=body, state_elems=counters)
+        g.analyze()
+        g.replay(5)
+        g.sync()
+        assert np.array_equal(g.state.cpu().numpy(), want(tr, counters, 5))
+    g.close()
+
+
 @pytest.mark.parametrize("body", [grt.RT_BODY_SPIN, grt.RT_BODY_FMA])
 def test_bodies_of_wide_and_deep_graphs(body):
     ensure_built()
