@@ -247,9 +247,11 @@ template void scan_exclusive<uint32_t>(const uint32_t*, uint32_t*, int64_t, uint
 namespace {
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / 32;
-// Keys per thread: 16 (4096 a block), or 4 for small sorts, whose few blocks are
-// a chain of ranking rounds each (6200 keys: 13.9 us a pass with 16).
-constexpr int kRadixIpt = 16, kRadixIptSmall = 4;
+// Keys per thread: 12 (3072 a block: 53 KB of shared memory, four blocks an SM;
+// with 16 three, 6.6 ms for the two passes over 343M entries instead of 6.0, and
+// with 8 five but more digit counts, 6.2), or 4 for small sorts, whose few blocks
+// are a chain of ranking rounds each (6200 keys: 13.9 us a pass with 16).
+constexpr int kRadixIpt = 12, kRadixIptSmall = 4;
 constexpr int64_t kRadixSmall = 96 * kRadixThreads * kRadixIptSmall;  // its digit counts still fit one scan block
 inline int64_t radix_blocks(int64_t n) {
   const int64_t tile = kRadixThreads * (n <= kRadixSmall ? kRadixIptSmall : kRadixIpt);
@@ -281,14 +283,24 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const K* keys, int
 // block-sorted order
 template <typename K, bool HAS_V, int IPT>
 constexpr size_t scatter_smem_bytes() {
-  return (size_t)(kRadixThreads * IPT) * (sizeof(K) + (HAS_V ? sizeof(uint64_t) : 0));
+  return (size_t)(kRadixThreads * IPT) * (sizeof(K) + (HAS_V ? sizeof(uint64_t) + sizeof(uint16_t) : 0));
+}
+
+__device__ __forceinline__ void copy8_async(void* to, const void* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from)
+               : "memory");
 }
 
 // One pass of the LSD radix sort over a block of (kRadixThreads * IPT) keys: every key is
 // ranked within its warp and digit (match_any), the ranks become positions in
 // the block's digit-sorted order, the keys are reordered in shared memory, and
 // consecutive threads then write consecutive keys of each digit run to the
-// run's global offset, so the global writes are coalesced. Stable.
+// run's global offset, so the global writes are coalesced. Stable. The values go
+// to shared memory as they lie, by asynchronous copies under the ranking, and
+// are picked by a 16-bit index when they are written: held in registers over the
+// ranking they cost a third of the resident warps and their own load latency
+// (two passes over 343M entries of 12 bytes: 7.06 -> 6.0 ms, with the write
+// loop unrolled and 12 keys a thread; copy rate allows 2.9).
 template <typename K, bool HAS_V, int IPT>
 __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     const K* __restrict__ keys, const uint64_t* __restrict__ vals, K* __restrict__ keys_out,
@@ -301,6 +313,7 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   extern __shared__ __align__(16) unsigned char rsmem[];
   K* sk = reinterpret_cast<K*>(rsmem);
   uint64_t* sv = reinterpret_cast<uint64_t*>(rsmem + (size_t)(kRadixThreads * IPT) * sizeof(K));
+  uint16_t* from = reinterpret_cast<uint16_t*>(sv + kRadixThreads * IPT);  // the value of a sorted position
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int w = 0; w < kRadixWarps; ++w) wcnt[w][threadIdx.x] = 0;
@@ -308,7 +321,6 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   __syncthreads();
   const int64_t wbase = (int64_t)blockIdx.x * (kRadixThreads * IPT) + (int64_t)warp * (32 * IPT);
   K kv[IPT];
-  uint64_t vv[HAS_V ? IPT : 1];
   uint32_t rk[IPT];
   const unsigned lt = lanemask_lt();
   // every key's load in flight before the ranking, whose warp barriers would hold
@@ -318,6 +330,14 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
   for (int r = 0; r < IPT; ++r) {
     const int64_t idx = wbase + r * 32 + lane;
     kv[r] = idx < n ? keys[idx] : K(0);
+  }
+  // the values go to shared memory as they lie, while the keys are ranked
+  if (HAS_V) {
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+      const int64_t idx = wbase + r * 32 + lane;
+      if (idx < n) copy8_async(sv + (warp * (32 * IPT) + r * 32 + lane), vals + idx);
+    }
   }
 #pragma unroll
   for (int r = 0; r < IPT; ++r) {
@@ -355,14 +375,8 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
 #pragma unroll
   for (int w = 0; w < kRadixWarps; ++w) wpre += w < warp ? wsum[w] : 0u;
   bstart[threadIdx.x] = wpre + incl - tot;
+  boff[threadIdx.x] -= wpre + incl - tot;  // read back after the next barriers: where position 0 would go
   if (threadIdx.x == kRadixThreads - 1) bstart[256] = wpre + incl;
-  if (HAS_V) {
-#pragma unroll
-    for (int r = 0; r < IPT; ++r) {
-      const int64_t idx = wbase + r * 32 + lane;
-      vv[HAS_V ? r : 0] = idx < n ? vals[idx] : 0ull;
-    }
-  }
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < IPT; ++r) {
@@ -371,17 +385,21 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
       const uint32_t d = (uint32_t)(kv[r] >> shift) & mask;
       const uint32_t lp = bstart[d] + wcnt[warp][d] + rk[r];
       sk[lp] = kv[r];
-      if (HAS_V) sv[lp] = vv[HAS_V ? r : 0];
+      if (HAS_V) from[lp] = (uint16_t)(warp * (32 * IPT) + r * 32 + lane);
     }
   }
+  if (HAS_V) asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const uint32_t nvalid = bstart[256];
-  for (uint32_t i = threadIdx.x; i < nvalid; i += kRadixThreads) {
-    const K k = sk[i];
-    const uint32_t d = (uint32_t)(k >> shift) & mask;
-    const uint32_t dst = boff[d] + (i - bstart[d]);
-    keys_out[dst] = k;
-    if (HAS_V) vals_out[dst] = sv[i];
+#pragma unroll
+  for (int r = 0; r < IPT; ++r) {
+    const uint32_t i = r * kRadixThreads + threadIdx.x;
+    if (i < nvalid) {
+      const K k = sk[i];
+      const uint32_t dst = boff[(uint32_t)(k >> shift) & mask] + i;
+      keys_out[dst] = k;
+      if (HAS_V) vals_out[dst] = sv[from[i]];
+    }
   }
 }
 
