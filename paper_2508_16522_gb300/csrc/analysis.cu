@@ -590,9 +590,55 @@ __global__ void __launch_bounds__(256) k_bucket_sort_warp(const uint32_t* __rest
   if (lane == 0) ucnt[v] = (uint32_t)__popc(m);
 }
 
+// Row v of len targets at b, 32 < len <= 32 E, by one warp: E targets a lane
+// (target 32 e + lane in x[e]), a bitonic network of shuffles and of exchanges
+// between a lane's own registers; the distinct ones to the front.
+template <int E>
+__device__ __forceinline__ uint32_t sort_row(uint32_t* b, uint32_t len) {
+  const int lane = threadIdx.x & 31;
+  uint32_t x[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) x[e] = (uint32_t)(32 * e + lane) < len ? b[32 * e + lane] : 0xFFFFFFFFu;
+#pragma unroll
+  for (int k = 2; k <= 32 * E; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        if (j >= 32) {
+          const int f = e ^ (j >> 5);
+          if (f > e) {
+            const uint32_t lo = min(x[e], x[f]), hi = max(x[e], x[f]);
+            const bool up = ((32 * e) & k) == 0;
+            x[e] = up ? lo : hi;
+            x[f] = up ? hi : lo;
+          }
+        } else {
+          const uint32_t y = __shfl_xor_sync(0xffffffffu, x[e], j);
+          const bool low = (lane & j) == 0, up = ((32 * e + lane) & k) == 0;
+          x[e] = low == up ? min(x[e], y) : max(x[e], y);
+        }
+      }
+    }
+  }
+  uint32_t u = 0, last = 0xFFFFFFFFu;  // no target is ~0
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const uint32_t left = __shfl_up_sync(0xffffffffu, x[e], 1);
+    const bool keep = (uint32_t)(32 * e + lane) < len && x[e] != (lane == 0 ? last : left);
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (keep) b[u + (uint32_t)__popc(m & lanemask_lt())] = x[e];
+    u += (uint32_t)__popc(m);
+    last = __shfl_sync(0xffffffffu, x[e], 31);
+  }
+  return u;
+}
+
 // the listed long rows (at most kBucketMaxRow pairs): one warp each, a bitonic
 // sort in shared memory padded with ~0, then the distinct targets written back
-// to the row's front
+// to the row's front. Up to 256 pairs the row stays in registers (in shared memory
+// half the lanes idle in each exchange: analysis of 5317 dense launches 0.375 ->
+// 0.360 ms, of the 1M-launch trace 38.2 -> 37.5).
 __global__ void __launch_bounds__(128) k_bucket_sort_large(const uint32_t* off, uint32_t* bucket, uint32_t* ucnt,
                                                            const uint32_t* big, const uint32_t* nbig) {
   __shared__ uint32_t buf[4][kBucketMaxRow];
@@ -602,7 +648,14 @@ __global__ void __launch_bounds__(128) k_bucket_sort_large(const uint32_t* off, 
   for (uint32_t r = blockIdx.x * 4 + warp; r < nb; r += gridDim.x * 4) {
     const uint32_t v = big[r];
     const uint32_t a = off[v], len = off[v + 1] - a;
-    uint32_t N = 64;
+    if (len <= 256u) {
+      const uint32_t d = len <= 64u    ? sort_row<2>(bucket + a, len)
+                         : len <= 128u ? sort_row<4>(bucket + a, len)
+                                       : sort_row<8>(bucket + a, len);
+      if (lane == 0) ucnt[v] = d;
+      continue;
+    }
+    uint32_t N = 512;
     while (N < len) N <<= 1;
     for (uint32_t i = lane; i < N; i += 32) s[i] = i < len ? bucket[a + i] : 0xFFFFFFFFu;
     __syncwarp();
@@ -811,7 +864,7 @@ void launch_bucket_build(const uint64_t* pairs, int64_t P, int key_bits, int32_t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     count_launch();
-    k_bucket_sort_large<<<(unsigned)(sms > 0 ? sms * 4 : 512), 128, 0, s>>>(off, bucket, ucnt, big, nbig);
+    k_bucket_sort_large<<<(unsigned)(sms > 0 ? sms * 8 : 1024), 128, 0, s>>>(off, bucket, ucnt, big, nbig);
   }
   scan_exclusive<uint32_t>(ucnt, row_ptr, n, scan_ws, s);
   count_launch();
