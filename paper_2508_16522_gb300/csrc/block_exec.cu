@@ -50,7 +50,7 @@ struct BlockCtl {
   uint32_t done, status;
   int32_t graph;
   uint32_t pad;
-  uint32_t cnt[kCntCount + 1];
+  uint32_t cnt[kCntCount];
 };
 
 size_t block_smem_bytes(int32_t n, int warps) {
@@ -77,13 +77,13 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
   uint32_t cnt[kCntCount];
 #pragma unroll
   for (int k = 0; k < kCntCount; ++k) cnt[k] = 0;
-  if (tid <= kCntCount) ctl->cnt[tid] = 0;
+  if (tid < kCntCount) ctl->cnt[tid] = 0;
   if (tid == 0) ctl->status = 0;
 
-  for (;;) {
+  for (uint32_t turn = 0;; ++turn) {
     // the next graph: graph 0, or the batch's, largest first
     if (tid == 0) {
-      const uint32_t i = a.order ? atomicAdd(a.next, 1u) : ctl->cnt[kCntCount]++;
+      const uint32_t i = a.order ? atomicAdd(a.next, 1u) : turn;
       ctl->graph = i < (uint32_t)a.n_order ? (a.order ? a.order[i] : 0) : -1;
     }
     __syncthreads();
@@ -136,25 +136,29 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
             if (lane == 0) atomicAdd(&ctl->done, pend);
             pend = 0;
           }
-          const unsigned long long v0 = *(volatile unsigned long long*)&ctl->ht;
+          // one lane's look for the whole warp: lanes that read for themselves could
+          // see different words, and part over the shuffles below
+          unsigned long long v0 = 0;
+          if (lane == 0) v0 = *(volatile unsigned long long*)&ctl->ht;
+          v0 = __shfl_sync(kFullB, v0, 0);
           if ((uint32_t)v0 >= (uint32_t)(v0 >> 32)) {
-            const uint32_t d = *(volatile uint32_t*)&ctl->done;
-            if (d >= (uint32_t)n || *(volatile uint32_t*)&ctl->status) break;
-            if ((++polls & 63u) == 0u) {
-              int late = 0;
-              if (lane == 0) {
+            ++polls;
+            int over = 0;
+            if (lane == 0) {
+              const uint32_t d = *(volatile uint32_t*)&ctl->done;
+              over = d >= (uint32_t)n || *(volatile uint32_t*)&ctl->status != 0u;
+              if (!over && (polls & 63u) == 0u) {
                 const uint64_t now = globaltimer_ns();
                 if (idle_since == 0 || d != seen) {
                   idle_since = now;
                   seen = d;
                 } else if (now - idle_since > (uint64_t)p.timeout_ns) {
-                  late = 1;
+                  over = 1;
                   *(volatile uint32_t*)&ctl->status = (uint32_t)RT_ERR_TIMEOUT;
                 }
               }
-              if (__shfl_sync(kFullB, late, 0)) break;
             }
-            __syncwarp();
+            if (__shfl_sync(kFullB, over, 0)) break;
             __nanosleep(kBlockSleep);
             continue;
           }

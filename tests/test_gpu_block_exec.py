@@ -1,0 +1,43 @@
+"""The executor that runs a graph inside one block from a queue of ready tasks:
+graphs of up to 65534 tasks whose edges are too long for a window of program
+order."""
+import numpy as np
+import pytest
+
+from paper_2508_16522_gb300 import grt
+from paper_2508_16522_gb300 import tracegen as tg
+
+from gpu_helpers import ensure_built, gpu_graph
+
+pytestmark = pytest.mark.gpu
+
+
+def explicit(n, preds, counters=1):
+    """A trace of n tasks without rectangles; preds: (task, predecessor) rows, task v adds to counter v % counters."""
+    preds = np.unique(np.asarray(preds, np.int64).reshape(-1, 2), axis=0)
+    return tg._finish(1, [0], [0], np.zeros(n, np.int64), np.zeros(0, np.int64), np.zeros(0, np.int64),
+                      np.zeros(0, np.uint8), pred_counts=np.bincount(preds[:, 0], minlength=n), pred=preds[:, 1],
+                      body_arg=np.arange(n) % counters, name=f"explicit{n}_{len(preds)}")
+
+
+def chain(n, *more):
+    """One chain of n tasks and an edge from the first to the last, longer than any window."""
+    v = np.arange(1, n)
+    return explicit(n, np.concatenate([np.stack([v, v - 1], 1), [[n - 1, 0]], *[np.asarray(m).reshape(-1, 2) for m in more]]))
+
+
+@pytest.mark.parametrize("n", [800, 5000, 20000])
+def test_every_run_runs_every_task(n):
+    """Each launch runs all of its tasks, whichever warp finds the queue empty first."""
+    ensure_built()
+    tr = chain(n, [(v, v - 700) for v in range(701, n, 3)])
+    g = gpu_graph(tr, body=grt.RT_BODY_COUNTER, state_elems=1)
+    g.analyze()
+    for k in range(60):
+        g.execute()
+        g.sync()
+        st = g.stats()
+        assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
+        assert st["exec_counters"]["tasks"] == n
+    assert int(g.state.cpu()[0]) == 60 * n
+    g.close()
