@@ -183,9 +183,18 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
           cnt[kCntClaims] += 1;
           h = __shfl_sync(kFullB, h, 0) + (uint32_t)lane;
           if ((uint32_t)lane < take) {
-            // a slot is written just after its place was taken
-            do id = h < (uint32_t)Q ? queue[h] : spill[h];
-            while (id == kNoId && !*(volatile uint32_t*)&ctl->status);
+            // a slot is written just after its place was taken; the clock bounds the
+            // wait here too (an idle warp's may not run: all of them can be here)
+            uint64_t from = 0;
+            for (uint32_t tries = 1;; ++tries) {
+              id = h < (uint32_t)Q ? queue[h] : spill[h];
+              if (id != kNoId || *(volatile uint32_t*)&ctl->status) break;
+              if ((tries & 1023u) == 0u) {
+                const uint64_t now = globaltimer_ns();
+                if (from == 0) from = now;
+                else if (now - from > (uint64_t)p.timeout_ns) *(volatile uint32_t*)&ctl->status = (uint32_t)RT_ERR_TIMEOUT;
+              }
+            }
           }
           __syncwarp();
           idle_since = 0;

@@ -41,3 +41,22 @@ def test_every_run_runs_every_task(n):
         assert st["exec_counters"]["tasks"] == n
     assert int(g.state.cpu()[0]) == 60 * n
     g.close()
+
+
+def test_a_run_past_its_limit_reports_and_recovers():
+    """Bodies of many times the limit: the launch ends with RT_ERR_TIMEOUT, the graph stays usable."""
+    ensure_built()
+    tr = explicit(2, [(1, 0)])
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=1 << 20, timeout_ns=200_000)
+    g.analyze()
+    with pytest.raises(grt.GrtError) as e:
+        g.execute()
+        g.sync()
+    assert e.value.status == grt.RT_ERR_TIMEOUT
+    g.close()
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=1 << 20)
+    g.analyze()
+    g.execute()
+    g.sync()
+    assert g.stats()["exec_counters"]["tasks"] == 2
+    g.close()
