@@ -28,7 +28,9 @@
 //
 // The bodies' effects need only reach the block's own warps: fences are block
 // scope, and COUNTER's state may stay in L1. Every wait is bounded by
-// timeout_ns without a finished task.
+// timeout_ns without reported progress: a warp reports what it ran when it finds
+// nothing kept and at the latest after kBlockReport tasks, k_exec_window's after
+// four chunks of 32.
 #include <mutex>
 #include <set>
 
@@ -44,6 +46,7 @@ constexpr int kSmallWarps = 4;    // a batch's graphs of at most kBlockSmall tas
 constexpr int kBlockKeep = 64;  // kept ids per warp
 constexpr unsigned kBlockSleep = 40;  // ns between an idle warp's polls
 constexpr uint32_t kNoId = 0xFFFFu;
+constexpr uint32_t kBlockReport = 1024;  // tasks a warp runs at most, and a batch, before it counts them
 
 struct BlockCtl {
   unsigned long long ht;  // queue: head in the low 32 bits, tail in the high ones
@@ -125,6 +128,13 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
           const int m = nl < 32 ? nl : 32;
           if (lane < m) id = keepq[nl - m + lane];
           nl -= m;
+          // a warp that always keeps something still reports: the others' limit
+          // counts from the last finished task they know of
+          if (pend >= kBlockReport) {
+            cnt[kCntTasks] += pend;
+            if (lane == 0) atomicAdd(&ctl->done, pend);
+            pend = 0;
+          }
           __syncwarp();
         } else {
           // count what ran since the last look, then up to `claim` queued ids. An

@@ -60,3 +60,19 @@ def test_a_run_past_its_limit_reports_and_recovers():
     g.sync()
     assert g.stats()["exec_counters"]["tasks"] == 2
     g.close()
+
+
+def test_a_warp_that_never_waits_reports_its_progress():
+    """A chain runs in one warp, which always keeps its next task: 60000 tasks take several times the limit, the 4096
+    between two reports a small part of it."""
+    ensure_built()
+    n = 60000
+    tr = chain(n)
+    g = gpu_graph(tr, body=grt.RT_BODY_COUNTER, state_elems=1, timeout_ns=15_000_000)
+    g.analyze()
+    g.execute()
+    g.sync()
+    st = g.stats()
+    assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
+    assert int(g.state.cpu()[0]) == n
+    g.close()
