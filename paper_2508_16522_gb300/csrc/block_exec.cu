@@ -53,7 +53,7 @@ struct BlockCtl {
   uint32_t done, status;
   int32_t graph;
   uint32_t pad;
-  uint32_t cnt[kCntCount];
+  unsigned long long cnt[kCntCount];  // the block's totals: one block may run a whole graph many times
 };
 
 size_t block_smem_bytes(int32_t n, int warps) {
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
   uint16_t* const keepq = reinterpret_cast<uint16_t*>(bsmem + sizeof(BlockCtl)) + warp * kBlockKeep;
   uint32_t* const cntw = reinterpret_cast<uint32_t*>(bsmem + sizeof(BlockCtl) + WARPS * kBlockKeep * 2);
   const unsigned lt = lanemask_lt();
-  uint32_t edges = 0;  // out-edges of the tasks this lane ran
+  uint32_t edges = 0;  // out-edges of the tasks this lane ran in this run
   uint32_t cnt[kCntCount];
 #pragma unroll
   for (int k = 0; k < kCntCount; ++k) cnt[k] = 0;
@@ -355,6 +355,9 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
         __syncwarp();
       }
       if (FENCE) __threadfence_block();
+      const uint32_t e = __reduce_add_sync(kFullB, edges);  // one run has fewer than 2^31
+      if (lane == 0) atomicAdd(&ctl->cnt[kCntEdges], (unsigned long long)e);
+      edges = 0;
       __syncthreads();  // the run is over (or timed out)
       if (ctl->status) break;
       dirty = (uint32_t)(ctl->ht >> 32);
@@ -362,15 +365,14 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
     }
     __syncthreads();
   }
-  cnt[kCntEdges] = __reduce_add_sync(kFullB, edges);
   if (lane == 0) {
 #pragma unroll
     for (int k = 0; k < kCntCount; ++k)
-      if (cnt[k]) atomicAdd(&ctl->cnt[k], cnt[k]);
+      if (k != kCntEdges && cnt[k]) atomicAdd(&ctl->cnt[k], (unsigned long long)cnt[k]);
   }
   __syncthreads();
   if (a.order) {
-    if (tid < kCntCount && ctl->cnt[tid]) atomicAdd(&p.ctrl->counters[tid], (unsigned long long)ctl->cnt[tid]);
+    if (tid < kCntCount && ctl->cnt[tid]) atomicAdd(&p.ctrl->counters[tid], ctl->cnt[tid]);
     if (tid == 0 && ctl->status) atomicCAS(&p.ctrl->status, 0u, ctl->status);
   } else {
     // pinned host memory: the host reads it after the stream's synchronisation
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
   __shared__ uint32_t held[WARPS];  // first task of the chunk each warp holds (past the end: ~0)
   __shared__ uint32_t s_done, s_status;
   __shared__ int32_t s_graph;
-  __shared__ uint32_t s_cnt[2];
+  __shared__ unsigned long long s_cnt[2];
   uint32_t* const count = reinterpret_cast<uint32_t*>(wsmem);
   constexpr int T = WARPS * 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
   if (tid == 0) {
     s_status = 0u;
     s_graph = -1;
-    s_cnt[0] = s_cnt[1] = 0u;
+    s_cnt[0] = s_cnt[1] = 0ull;
   }
   uint32_t edges = 0, ran = 0, batches = 0;
   __syncthreads();
@@ -561,16 +563,15 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 4) k_ex
         ran += (uint32_t)(n - c0 < 32 ? n - c0 : 32);
       }
       if (FENCE) __threadfence_block();
+      const uint32_t e = __reduce_add_sync(kFullB, edges);  // one run has fewer than 2^31
+      if (lane == 0) atomicAdd(&s_cnt[1], (unsigned long long)e);
+      edges = 0;
       __syncthreads();
       if (s_status) break;
     }
     __syncthreads();
   }
-  edges = __reduce_add_sync(kFullB, edges);
-  if (lane == 0) {
-    atomicAdd(&s_cnt[0], ran);
-    atomicAdd(&s_cnt[1], edges);
-  }
+  if (lane == 0) atomicAdd(&s_cnt[0], (unsigned long long)ran);
   __syncthreads();
   if (tid == 0) {
     const unsigned long long cnt[3] = {batches, s_cnt[0], s_cnt[1]};  // batches: one warp's

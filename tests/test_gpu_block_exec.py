@@ -76,3 +76,25 @@ def test_a_warp_that_never_waits_reports_its_progress():
     assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
     assert int(g.state.cpu()[0]) == n
     g.close()
+
+
+@pytest.mark.parametrize("longest", [False, True], ids=["window", "queue"])
+def test_edges_of_many_replays_are_counted_in_64_bits(longest):
+    """255 layers of 256 tasks, each after all of the layer before it: 16.6M edges a run, over 2^32 in 264 runs."""
+    ensure_built()
+    w, t, runs = 256, 255, 264
+    v = np.repeat(np.arange(w, w * t), w)
+    preds = np.stack([v, (v // w - 1) * w + np.tile(np.arange(w), w * (t - 1))], 1)
+    if longest:
+        preds = np.concatenate([preds, [[w * t - 1, 0]]])
+    tr = explicit(w * t, preds, counters=w)
+    g = gpu_graph(tr, body=grt.RT_BODY_COUNTER, state_elems=w, timeout_ns=2_000_000_000)
+    g.analyze()
+    g.replay(runs)
+    g.sync()
+    st = g.stats()
+    assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
+    assert st["exec_counters"]["tasks"] == runs * tr.n
+    assert st["exec_counters"]["edges"] == runs * len(preds) > 1 << 32
+    assert np.array_equal(g.state.cpu().numpy(), np.full(w, t * runs))
+    g.close()
