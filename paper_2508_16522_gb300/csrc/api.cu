@@ -1214,7 +1214,7 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   p.claim = g->cfg_claim > 0 ? g->cfg_claim : (owned ? 1 : (block ? block_claim(g->n_edges, g->n) : 8));  // owned: chunks a warp holds at once
   p.keep = g->cfg_keep > 0 ? g->cfg_keep : (block ? block_keep(g->n_edges, g->n) : 16);
   p.block_n = block ? g->n : 0;
-  p.window = window;
+  p.window = !window ? 0 : (block_window_small(g->max_span, g->last_root) ? 2 : 1);
   p.span = g->max_span;
   if (block && !window) CKR(g->spill.reserve((size_t)g->n * 2, s));
   p.tickets = (g->desc.flags & RT_GRAPH_TICKETS) ? g->tickets.as<int32_t>() : nullptr;
@@ -1250,11 +1250,11 @@ rt_status enqueue_run(rt_graph* g, const ExecParams& p, int64_t ring_clear, cuda
     ba.status_out = g->hpin + kStatusWord;
     ba.counters_out = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(g->hpin) + kCountersByte);
     ba.span = p.span;
-    if (p.window) launch_exec_window(p, ba, 1, p.span <= kSmallSpan, s);
+    if (p.window) launch_exec_window(p, ba, 1, p.window == 2, s);
     else launch_exec_block(p, ba, p.block_n, 1, false, s);
     if (timed) CK(cudaEventRecord(g->ev[EV_XK1], s));
     g->exec_blocks = 1;
-    g->exec_warps = p.window && p.span <= kSmallSpan ? block_small_warps() : block_exec_warps();
+    g->exec_warps = p.window == 2 ? block_small_warps() : block_exec_warps();
     return RT_OK;
   }
   launch_seed(p, ring_clear, s);
@@ -1798,10 +1798,10 @@ rt_status finish_batch(rt_batch* b, const std::vector<ExecGraph>& table) {
   b->blocks_fit = true;
   for (const int32_t k : by_size) {
     const ExecGraph& X = table[(size_t)k];
-    const int32_t span = (int32_t)shape[3 * (size_t)k];
+    const int32_t span = (int32_t)shape[3 * (size_t)k], last_root = (int32_t)shape[3 * (size_t)k + 1];
     b->max_outdeg = std::max(b->max_outdeg, (int32_t)shape[3 * (size_t)k + 2]);
-    if (block_window_fits(span, (int32_t)shape[3 * (size_t)k + 1], X.body, X.spin_iters)) {
-      lists[span <= kSmallSpan ? 1 : 0].push_back(k);
+    if (block_window_fits(span, last_root, X.body, X.spin_iters)) {
+      lists[block_window_small(span, last_root) ? 1 : 0].push_back(k);
     } else if (block_exec_fits(X.n_tasks, X.n_roots, X.body, X.spin_iters)) {
       lists[X.n_tasks <= kBlockSmall ? 3 : 2].push_back(k);
       b->max_queue_n = std::max(b->max_queue_n, X.n_tasks);

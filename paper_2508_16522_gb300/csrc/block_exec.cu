@@ -660,12 +660,18 @@ void launch_window_warps(const ExecParams& p, const BlockArgs& a, int S, int blo
 }
 }  // namespace
 
+// how many tasks can be ready at once, on average over a run's steps: the tasks
+// of the first d steps end at most d spans after the last root
+static int32_t window_width(int32_t span, int32_t last_root) { return span > last_root ? span : last_root + 1; }
+
 bool block_window_fits(int32_t span, int32_t last_root, int32_t body, int32_t spin_iters) {
   if (span > kWindowSpan || last_root > kWindowSpan) return false;
   if (body == RT_BODY_CHECK) return false;
   const int64_t iters = body == RT_BODY_SPIN || body == RT_BODY_FMA ? spin_iters : 0;
-  return (int64_t)span * (iters + 20) <= kWindowWork;
+  return (int64_t)window_width(span, last_root) * (iters + 20) <= kWindowWork;
 }
+
+bool block_window_small(int32_t span, int32_t last_root) { return window_width(span, last_root) <= kSmallSpan; }
 
 void launch_exec_window(const ExecParams& p, const BlockArgs& a, int blocks, bool small, cudaStream_t s) {
   if (small) launch_window_warps<kSmallWarps>(p, a, kSmallSlots, blocks, s);
