@@ -1106,9 +1106,11 @@ int block_keep(int64_t edges, int64_t tasks) {
   return deg < 6 ? 32 : (int)std::max<int64_t>(1, 24 / deg);
 }
 
-// ... and takes from the queue at once: one task of many edges, whose row the
-// warp then shares
-int block_claim(int64_t edges, int64_t tasks) { return tasks > 0 && edges / tasks >= 6 ? 1 : 32; }
+// ... and whether it takes only its share of the queue at once: tasks of many
+// edges, each of which keeps a warp busy by itself while there are few. (One at
+// a time however many there are leaves 31 lanes of each warp idle: 60 steps of
+// 1000 tasks of degree 8 took 3.5 ms like that, 0.8 by shares.)
+bool block_share(int64_t edges, int64_t tasks) { return tasks > 0 && edges / tasks >= 6; }
 
 // the owned executors' extension records, if some task has more successors
 // than its trigger record holds
@@ -1211,7 +1213,7 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   p.replays = replays;
   p.graphs_target = 1;
   p.timeout_ns = g->desc.timeout_ns;
-  p.claim = g->cfg_claim > 0 ? g->cfg_claim : (owned ? 1 : (block ? block_claim(g->n_edges, g->n) : 8));  // owned: chunks a warp holds at once
+  p.claim = g->cfg_claim > 0 ? g->cfg_claim : (owned ? 1 : (block ? 32 : 8));  // owned: chunks a warp holds at once
   p.keep = g->cfg_keep > 0 ? g->cfg_keep : (block ? block_keep(g->n_edges, g->n) : 16);
   p.block_n = block ? g->n : 0;
   p.window = !window ? 0 : (block_window_small(g->max_span, g->last_root) ? 2 : 1);
@@ -1250,6 +1252,7 @@ rt_status enqueue_run(rt_graph* g, const ExecParams& p, int64_t ring_clear, cuda
     ba.status_out = g->hpin + kStatusWord;
     ba.counters_out = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(g->hpin) + kCountersByte);
     ba.span = p.span;
+    ba.share = g->cfg_claim == 0 && block_share(g->n_edges, g->n);
     if (p.window) launch_exec_window(p, ba, 1, p.window == 2, s);
     else launch_exec_block(p, ba, p.block_n, 1, false, s);
     if (timed) CK(cudaEventRecord(g->ev[EV_XK1], s));
@@ -2081,7 +2084,7 @@ rt_status prepare_batch_blocks(rt_batch* b) {
   return RT_OK;
 }
 
-rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, cudaStream_t s) {
+rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, bool share, cudaStream_t s) {
   CK(cudaMemsetAsync(p.ctrl, 0, sizeof(ExecCtrl), s));  // status, counters and the launches' next graphs
   p.adjx = b->adjx.as<int4>();
   uint32_t* const next[4] = {&p.ctrl->head, &p.ctrl->tail, &p.ctrl->ticket,
@@ -2103,6 +2106,7 @@ rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, cudaStream_t s) {
     a.order = list;
     a.n_order = n[l];
     a.next = next[l];
+    a.share = share;
     const bool small = l & 1;
     const int blocks = std::min(n[l], g_dev.num_sms * (small ? 8 : 2));
     cudaStream_t on = small ? side : s;
@@ -2297,16 +2301,17 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
   p.replays = replays;
   p.graphs_target = b->G_nonempty;
   p.timeout_ns = 2000000000ll;
-  p.claim = claim > 0 ? claim : (in_blocks ? block_claim(b->E, b->T) : 32);
+  p.claim = claim > 0 ? claim : 32;
   p.keep = keep > 0 ? keep : (in_blocks ? block_keep(b->E, b->T) : 32);
   p.tickets = nullptr;
   p.total_roots = (int32_t)b->Rtot;
   p.need_fence = b->need_fence;
+  const bool share = claim <= 0 && block_share(b->E, b->T);
   CK(cudaEventRecord(b->e0, s));
   if (in_blocks && !b->graph_next) {
     // the first launch direct: a batch run once does not pay for a CUDA graph
     b->graph_next = true;
-    CKR(enqueue_batch_blocks(b, p, s));
+    CKR(enqueue_batch_blocks(b, p, share, s));
   } else if (clear) {
     // a new or dirty ring is cleared whole: a direct launch
     CKR(enqueue_batch(b, p, (int64_t)(b->ring.cap / 8), blocks, warps, s));
@@ -2315,7 +2320,7 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
     const int64_t key[7] = {replays,
                             in_blocks ? 0 : blocks,
                             in_blocks ? 0 : warps,
-                            p.claim,
+                            in_blocks && share ? -p.claim : p.claim,
                             p.keep,
                             in_blocks ? -2 : (int64_t)(uintptr_t)p.ring,
                             (int64_t)p.ring_cap};
@@ -2323,7 +2328,7 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
       drop_batch_graph(b);
       if (!b->cap_stream) CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
       CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-      rt_status st = in_blocks ? enqueue_batch_blocks(b, p, b->cap_stream)
+      rt_status st = in_blocks ? enqueue_batch_blocks(b, p, share, b->cap_stream)
                                : enqueue_batch(b, p, 0, blocks, warps, b->cap_stream);
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamEndCapture(b->cap_stream, &graph);

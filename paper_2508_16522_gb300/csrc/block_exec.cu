@@ -178,7 +178,9 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kBlockWarps ? 2 : 8) k_ex
             for (;;) {
               const uint32_t hd = (uint32_t)v, tl = (uint32_t)(v >> 32);
               if (hd >= tl) break;
-              const uint32_t k = tl - hd < (uint32_t)p.claim ? tl - hd : (uint32_t)p.claim;
+              uint32_t k = tl - hd;
+              if (a.share) k = k < 2 * WARPS ? 1u : k / WARPS;
+              k = k < (uint32_t)p.claim ? k : (uint32_t)p.claim;
               const unsigned long long w = atomicCAS(&ctl->ht, v, v + k);
               if (w == v) {
                 h = hd;

@@ -447,6 +447,7 @@ struct BlockArgs {
   const int32_t* order;   // a batch: the graphs to run, largest first (null: one graph)
   int32_t n_order;        // how many (1 for one graph)
   uint32_t* next;         // ... and the counter that hands them out, zeroed by the caller
+  int32_t share;          // k_exec_block: a warp takes its share of the queue, not all up to the claim width
   uint32_t* status_out;   // one graph: status and diagnostic counters, in pinned host memory
   unsigned long long* counters_out;
 };

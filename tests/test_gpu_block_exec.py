@@ -4,6 +4,7 @@ order."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2508_16522_gb300 import grt
 from paper_2508_16522_gb300 import tracegen as tg
 
@@ -97,4 +98,30 @@ def test_edges_of_many_replays_are_counted_in_64_bits(longest):
     assert st["exec_counters"]["tasks"] == runs * tr.n
     assert st["exec_counters"]["edges"] == runs * len(preds) > 1 << 32
     assert np.array_equal(g.state.cpu().numpy(), np.full(w, t * runs))
+    g.close()
+
+
+def layered(w, t, d):
+    """t steps of w tasks, each after d tasks of the step before it."""
+    v = np.arange(w, w * t)
+    p = (v // w - 1)[:, None] * w + ((v % w)[:, None] * 7 + np.arange(d)[None, :] * (w // d)) % w
+    return explicit(w * t, np.stack([np.repeat(v, d), p.reshape(-1)], 1))
+
+
+def test_a_full_queue_is_shared_out_in_batches():
+    """Steps of 1000 ready tasks of degree 8: the warps take batches, not a task each."""
+    ensure_built()
+    tr = layered(1000, 30, 8)
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=9)
+    g.analyze()
+    b = grt.Batch([g])
+    for _ in range(2):
+        g.out.zero_()
+        b.execute(replays=2)
+        b.sync()
+        assert np.array_equal(g.out.cpu().numpy(), oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=9)[1])
+        c = b.counters()
+        assert c["tasks"] == 2 * tr.n and c["edges"] == 2 * g.stats()["n_edges"]
+        assert 4 * c["claims"] < c["tasks"]
+    b.close()
     g.close()
