@@ -2043,7 +2043,9 @@ namespace {
 // the persistent executor and the status read-back.
 rt_status enqueue_batch(rt_batch* b, const ExecParams& p, int64_t ring_clear, int blocks, int warps,
                         cudaStream_t s) {
-  CK(cudaMemsetAsync(b->count.p, 0, (size_t)b->T * 4, s));
+  // (a batch of one graph takes the single-graph kernel, whose counters count down)
+  if (p.n_graphs == 1) launch_reset_counts(b->count.as<int32_t>(), b->indeg.as<int32_t>(), b->T, -1, 0, s);
+  else CK(cudaMemsetAsync(b->count.p, 0, (size_t)b->T * 4, s));
   launch_seed(p, ring_clear, s);
   launch_exec(p, blocks, warps, s);
   report_exec(p, b->hpin, b->hpin, s);
