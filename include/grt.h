@@ -279,11 +279,12 @@ rt_status rt_execute_kernels(rt_graph_t g, int32_t mode, int32_t iters, int32_t 
  * warp keeps for its own next batch instead of publishing them (0..64). These
  * are the autotuner's knobs; results do not depend on them. With neither blocks
  * nor warps given, the library also picks the executor under RT_EXEC_RING: a
- * graph of up to 65534 tasks, or one of any size whose edges span few tasks of
- * program order, runs inside one block (rt_graph_stats then reports 1 block),
- * and a larger one whose edges and roots stay within 16384 tasks of program
- * order over owned chunks; runs with tickets, a held task or the CHECK body
- * keep the ring. rt_execute_stitched picks owned chunks by the same rule. The
+ * graph of any size whose edges and roots reach at most 700 tasks of program
+ * order (and whose bodies are short enough for one SM's lanes) runs inside one
+ * block (rt_graph_stats then reports 1 block); one whose edges and roots stay
+ * within 16384 tasks runs over owned chunks; of the others, one of up to 65534
+ * tasks and few roots runs inside one block too, from a queue. Runs with tickets,
+ * a held task or the CHECK body keep the ring. rt_execute_stitched picks owned chunks by the same rule. The
  * event-based executor (rt_execute_events) takes the same claim width. */
 rt_status rt_graph_exec_config(rt_graph_t g, int32_t blocks, int32_t warps, int32_t claim, int32_t keep);
 

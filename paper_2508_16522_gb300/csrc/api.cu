@@ -1143,17 +1143,17 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   bool owned = g->cfg_policy == RT_EXEC_OWNED;  // no ring: every warp polls the countdowns it owns
   const uint64_t cap = (uint64_t)g->n * (uint64_t)replays + 64;
   if (cap >= 0xFFFFFFF0ull) return fail(RT_ERR_INVALID, "tasks x replays must stay below 2^32 per launch");
-  // a small graph whose launch shape is left to the library runs inside one
+  // a graph whose launch shape is left to the library: a narrow one runs inside one
   // block (not a run that records tickets, holds a task or must reset counters)
   const bool free_shape = !owned && g->cfg_blocks == 0 && g->cfg_warps == 0 && !(g->desc.flags & RT_GRAPH_TICKETS) &&
                           !g->dirty && g->hold_task < 0;
   const bool window = free_shape && block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters);
-  const bool block =
-      window || (free_shape && block_exec_fits(g->n, g->n_roots, g->desc.body, g->desc.spin_iters));
   // a larger one whose program order follows its dependences closely runs over
   // owned chunks; a CHECK body's time is its rectangles' cells, which the ring
   // spreads better
   const int own_warps = owned_warps_for(g->max_span, g->last_root);
+  const bool block = window || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
+                                                               g->desc.spin_iters, own_warps > 0));
   const bool auto_owned = free_shape && !block && own_warps > 0 && g->desc.body != RT_BODY_CHECK;
   if (auto_owned) owned = true;
   const bool grow = !owned && !block && (cap * 8 > g->ring.cap || !g->ring.p);

@@ -694,6 +694,13 @@ bool block_exec_fits(int32_t n, int64_t n_roots, int32_t body, int32_t spin_iter
   return iters * n <= kBlockWork;
 }
 
+bool block_exec_alone(int32_t n, int64_t n_roots, int64_t n_edges, int32_t body, int32_t spin_iters, bool owned) {
+  if (n <= 0 || !block_exec_fits(n, n_roots, body, spin_iters)) return false;
+  const int64_t iters = body == RT_BODY_SPIN || body == RT_BODY_FMA ? spin_iters : 0;
+  if (owned) return n <= kBlockTiny && iters * n <= kBlockTinyWork;
+  return n_roots <= (n_edges / n >= 6 ? kBlockAloneRootsDense : kBlockAloneRoots);
+}
+
 int block_exec_warps() { return kBlockWarps; }
 int block_small_warps() { return kSmallWarps; }
 

@@ -424,6 +424,19 @@ constexpr int32_t kBlockSmall = 4096;
 constexpr int64_t kBlockRoots = 1024;
 constexpr int64_t kBlockWork = 1ll << 24;
 bool block_exec_fits(int32_t n, int64_t n_roots, int32_t body, int32_t spin_iters);
+// the same for a graph that has the device to itself. Where owned chunks suit it
+// (owned) they are better as soon as steps are wide, and little worse where they
+// are narrow: 60 steps of 1024 random fan-in tasks 88 us against 380 in the block
+// (400 of 8 predecessors: 79 and 730), a captured request of 5317 launches 800
+// against 750; only a handful of tasks is quicker in the block (200 launches 29
+// and 19, at 1000 iterations 89 and 103). Where they do not, the ring is the other
+// choice, better from some width on (1024 wide 250 against 390, 512: 234 and 213;
+// of 8 predecessors 150 wide 396 and 790, 60 wide 644 and 362), which the roots
+// stand for
+constexpr int32_t kBlockTiny = 256;
+constexpr int64_t kBlockTinyWork = 1ll << 16;
+constexpr int64_t kBlockAloneRoots = 512, kBlockAloneRootsDense = 64;
+bool block_exec_alone(int32_t n, int64_t n_roots, int64_t n_edges, int32_t body, int32_t spin_iters, bool owned);
 int block_exec_warps();
 int block_small_warps();
 // the same with counters for a window of program order only: graphs whose edges

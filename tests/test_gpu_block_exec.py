@@ -27,7 +27,7 @@ def chain(n, *more):
     return explicit(n, np.concatenate([np.stack([v, v - 1], 1), [[n - 1, 0]], *[np.asarray(m).reshape(-1, 2) for m in more]]))
 
 
-@pytest.mark.parametrize("n", [800, 5000, 20000])
+@pytest.mark.parametrize("n", [17000, 20000, 65534])
 def test_every_run_runs_every_task(n):
     """Each launch runs all of its tasks, whichever warp finds the queue empty first."""
     ensure_built()
@@ -45,21 +45,22 @@ def test_every_run_runs_every_task(n):
 
 
 def test_a_run_past_its_limit_reports_and_recovers():
-    """Bodies of many times the limit: the launch ends with RT_ERR_TIMEOUT, the graph stays usable."""
+    """A limit far below the time between two reports: the launch ends with RT_ERR_TIMEOUT, the graph stays usable."""
     ensure_built()
-    tr = explicit(2, [(1, 0)])
-    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=1 << 20, timeout_ns=200_000)
+    tr = chain(17000)
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=900, timeout_ns=100_000)
     g.analyze()
     with pytest.raises(grt.GrtError) as e:
         g.execute()
         g.sync()
     assert e.value.status == grt.RT_ERR_TIMEOUT
     g.close()
-    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=1 << 20)
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=900)
     g.analyze()
     g.execute()
     g.sync()
-    assert g.stats()["exec_counters"]["tasks"] == 2
+    st = g.stats()
+    assert (st["exec_blocks"], st["exec_threads"], st["exec_counters"]["tasks"]) == (1, 512, tr.n)
     g.close()
 
 
@@ -91,21 +92,30 @@ def test_edges_of_many_replays_are_counted_in_64_bits(longest):
     tr = explicit(w * t, preds, counters=w)
     g = gpu_graph(tr, body=grt.RT_BODY_COUNTER, state_elems=w, timeout_ns=2_000_000_000)
     g.analyze()
-    g.replay(runs)
-    g.sync()
-    st = g.stats()
-    assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
-    assert st["exec_counters"]["tasks"] == runs * tr.n
-    assert st["exec_counters"]["edges"] == runs * len(preds) > 1 << 32
+    if longest:  # a batch of one
+        b = grt.Batch([g])
+        b.execute(replays=runs)
+        b.sync()
+        c = b.counters()
+        b.close()
+    else:
+        g.replay(runs)
+        g.sync()
+        st = g.stats()
+        assert (st["exec_blocks"], st["exec_threads"]) == (1, 512)
+        c = st["exec_counters"]
+    assert c["tasks"] == runs * tr.n
+    assert c["edges"] == runs * len(preds) > 1 << 32
     assert np.array_equal(g.state.cpu().numpy(), np.full(w, t * runs))
     g.close()
 
 
-def layered(w, t, d):
-    """t steps of w tasks, each after d tasks of the step before it."""
+def layered(w, t, d, longest=False):
+    """t steps of w tasks, each after d tasks of the step before it; longest: and an edge from the first to the last."""
     v = np.arange(w, w * t)
     p = (v // w - 1)[:, None] * w + ((v % w)[:, None] * 7 + np.arange(d)[None, :] * (w // d)) % w
-    return explicit(w * t, np.stack([np.repeat(v, d), p.reshape(-1)], 1))
+    rows = np.stack([np.repeat(v, d), p.reshape(-1)], 1)
+    return explicit(w * t, np.concatenate([rows, [[w * t - 1, 0]]]) if longest else rows)
 
 
 def test_a_full_queue_is_shared_out_in_batches():

@@ -10,7 +10,7 @@ from paper_2508_16522_gb300 import grt
 from paper_2508_16522_gb300 import tracegen as tg
 
 from gpu_helpers import ensure_built, gpu_graph
-from test_gpu_block_exec import explicit
+from test_gpu_block_exec import explicit, layered
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +45,23 @@ def test_many_roots_of_long_bodies_leave_the_block():
     assert shape_of(roots_then_chain(200, 900), 8) == (1, 512)
     assert shape_of(roots_then_chain(70, 900), 8) == (1, 128)
     assert shape_of(explicit(60, np.zeros((0, 2))), 1000) == (1, 128)
+
+
+def random_steps(w, t, seed, longest=False):
+    """w x t tasks of random fan-in 5; longest: and an edge from the first to the last."""
+    tr = tg.taskbench(w, t, "random", seed=seed, encode="explicit")
+    rows = np.stack([np.repeat(np.arange(tr.n), np.diff(tr.pred_off)), tr.pred], 1)
+    return explicit(tr.n, np.concatenate([rows, [[tr.n - 1, 0]]]) if longest else rows)
+
+
+def test_wide_small_graphs_are_not_put_in_one_block():
+    """Steps of a thousand tasks want more than one SM's lanes, however few tasks there are in all."""
+    assert shape_of(random_steps(1024, 20, 3), 8) == (32, 32)
+    assert shape_of(layered(1000, 20, 8), 64) == (32, 32)
+    assert shape_of(random_steps(600, 90, 4, longest=True), 8)[0] > 32  # the ring
+    assert shape_of(layered(100, 300, 8, longest=True), 8)[0] > 32
+    # a few hundred wide, or dense and narrow, with edges too long for owned chunks: the queue in a block
+    assert shape_of(random_steps(300, 90, 4, longest=True), 8) == (1, 512)
+    assert shape_of(layered(40, 600, 8, longest=True), 8) == (1, 512)
+    # a handful of tasks
+    assert shape_of(explicit(200, [(v, 0) for v in range(1, 200)] + [(199, v) for v in range(1, 199)]), 8) == (1, 512)
