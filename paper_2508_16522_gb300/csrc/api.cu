@@ -1806,7 +1806,7 @@ rt_status finish_batch(rt_batch* b, const std::vector<ExecGraph>& table) {
     if (block_window_fits(span, last_root, X.body, X.spin_iters)) {
       lists[block_window_small(span, last_root) ? 1 : 0].push_back(k);
     } else if (block_exec_fits(X.n_tasks, X.n_roots, X.body, X.spin_iters)) {
-      lists[X.n_tasks <= kBlockSmall ? 3 : 2].push_back(k);
+      lists[block_exec_small(X.n_tasks, X.body, X.spin_iters) ? 3 : 2].push_back(k);
       b->max_queue_n = std::max(b->max_queue_n, X.n_tasks);
     } else {
       b->blocks_fit = false;

@@ -691,7 +691,12 @@ bool block_exec_fits(int32_t n, int64_t n_roots, int32_t body, int32_t spin_iter
   if (n > kBlockTasks || n_roots > kBlockRoots) return false;
   if (body == RT_BODY_CHECK) return false;  // its time depends on its rectangles' cells
   const int64_t iters = body == RT_BODY_SPIN || body == RT_BODY_FMA ? spin_iters : 0;
-  return iters * n <= kBlockWork;
+  return iters * n <= kBlockWork && iters * n_roots <= kBlockStep;
+}
+
+bool block_exec_small(int32_t n, int32_t body, int32_t spin_iters) {
+  const int64_t iters = body == RT_BODY_SPIN || body == RT_BODY_FMA ? spin_iters : 0;
+  return n <= kBlockSmall && iters * n <= kBlockSmallWork;
 }
 
 bool block_exec_alone(int32_t n, int64_t n_roots, int64_t n_edges, int32_t body, int32_t spin_iters, bool owned) {

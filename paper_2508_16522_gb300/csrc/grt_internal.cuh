@@ -416,14 +416,21 @@ int exec_max_blocks_per_sm(int warps);
 // small graphs inside one block each (block_exec.cu). The bounds: task ids of 16
 // bits; 2 bytes of shared memory a task for its countdown and 2 for the first
 // kBlockQueue places of the ready queue, 164 KB in all (a resident server's
-// blocks leave that on every SM); at most kBlockRoots tasks ready at the start
-// and kBlockWork body iterations in all, so that one SM's lanes suffice
+// blocks leave that on every SM); at most kBlockRoots tasks ready at the start,
+// kBlockStep iterations of their bodies and kBlockWork of all bodies, so that one
+// SM's lanes suffice. A batch's graph takes a block of 4 warps, an eighth of an
+// SM, up to kBlockSmall tasks and kBlockSmallWork iterations. (128 graphs of 1000
+// independent tasks of 16000 iterations: 329 us in blocks of 4 warps, 157 by the
+// ring; 2 of them 328 and 92.)
 constexpr int32_t kBlockTasks = 65534;
 constexpr int32_t kBlockQueue = 16384;
 constexpr int32_t kBlockSmall = 4096;
 constexpr int64_t kBlockRoots = 1024;
 constexpr int64_t kBlockWork = 1ll << 24;
+constexpr int64_t kBlockStep = 1ll << 19;
+constexpr int64_t kBlockSmallWork = 1ll << 20;
 bool block_exec_fits(int32_t n, int64_t n_roots, int32_t body, int32_t spin_iters);
+bool block_exec_small(int32_t n, int32_t body, int32_t spin_iters);
 // the same for a graph that has the device to itself. Where owned chunks suit it
 // (owned) they are better as soon as steps are wide, and little worse where they
 // are narrow: 60 steps of 1024 random fan-in tasks 88 us against 380 in the block

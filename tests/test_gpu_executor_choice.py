@@ -65,3 +65,28 @@ def test_wide_small_graphs_are_not_put_in_one_block():
     assert shape_of(layered(40, 600, 8, longest=True), 8) == (1, 512)
     # a handful of tasks
     assert shape_of(explicit(200, [(v, 0) for v in range(1, 200)] + [(199, v) for v in range(1, 199)]), 8) == (1, 512)
+
+
+@pytest.mark.parametrize("n,iters,in_blocks", [(1000, 16000, False), (1000, 500, True), (300, 3000, False),
+                                               (4000, 8, False), (64, 8000, True)])
+def test_batches_of_long_independent_bodies(n, iters, in_blocks):
+    """Graphs whose roots alone outweigh one SM's lanes run on the grid; the block executors never count idle polls."""
+    ensure_built()
+    tr = explicit(n, np.concatenate([[[n - 1, 0]], [[n - 2, 0]]]))
+    want = oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=iters)[1]
+    graphs = [gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=iters) for _ in range(3)]
+    for g in graphs:
+        g.analyze()
+    b = grt.Batch(graphs)
+    for _ in range(2):
+        for g in graphs:
+            g.out.zero_()
+        b.execute(replays=2)
+        b.sync()
+        c = b.counters()
+        assert c["tasks"] == 6 * n and (c["idle"] == 0) == in_blocks
+        for g in graphs:
+            assert np.array_equal(g.out.cpu().numpy(), want)
+    b.close()
+    for g in graphs:
+        g.close()
