@@ -1126,16 +1126,30 @@ rt_status ensure_adjx(rt_graph* g) {
 // longest edge spans `span` tasks of program order and whose last task without
 // predecessors is `last_root`; 0: not suited. W warps hold a window of 32 W
 // consecutive tasks, so a chain that starts late in program order waits for
-// what comes before it: with every edge and every start inside the window the
-// front of ready tasks is inside it too. A level-ordered graph of width w has
-// edges of w to 2 w. (Random fan-in, 1024 x 300: 0.38 ms, by the ring 1.26 at its
-// default shape and 0.81 at its best; 20 stitched replays of a 1024 x 100
-// stencil 0.23 ms, 1.85 and 0.58. More than one step's warps gained nothing.)
+// what comes before it: with every edge and every start inside two windows the
+// front of ready tasks is inside them too. A level-ordered graph of width w has
+// edges of w to 2 w, and its roots are its first step: for a whole step at once
+// (alone) each of them has its lane. (Random fan-in, 1024 x 300: 0.38 ms, by the
+// ring 1.26 at its default shape and 0.81 at its best; 20 stitched replays of a
+// 1024 x 100 stencil 0.23 ms, 1.85 and 0.58. A stencil of 2000 x 200 with 32 warps
+// and with 64: 289 and 176 us, at 1000 iterations 1204 and 890, by the ring 1001.
+// With a lane for every step of the longest edge a butterfly of 1024 took 109 us
+// instead of 99.)
 constexpr int kOwnedMin = 32, kOwnedMax = 256;
-int owned_warps_for(int32_t span, int32_t last_root) {
+int owned_warps_for(int32_t span, int32_t last_root, bool alone) {
   int w = kOwnedMin;
-  while (w < kOwnedMax && 64 * w < span) w *= 2;
+  while (w < kOwnedMax && (64 * w < span || (alone && 32 * w <= last_root))) w *= 2;
   return span <= 64 * w && last_root < 64 * w ? w : 0;
+}
+
+// The longest bodies for which owned chunks are better than the ring: the tasks
+// of a chunk that become ready at different polls run their bodies one after
+// another, the ring's claims are whole batches. (100 steps of a 1024 wide stencil
+// at 1000, 2000 and 5000 iterations: 433, 781 and 1839 us, by the ring 501, 777
+// and 1602; of random fan-in 568, 1001 and 2303, and 789, 1166 and 2341.)
+constexpr int32_t kOwnedIters = 2000;
+int32_t body_iters(const rt_graph* g) {
+  return g->desc.body == RT_BODY_SPIN || g->desc.body == RT_BODY_FMA ? g->desc.spin_iters : 0;
 }
 
 rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ring_clear) {
@@ -1151,10 +1165,11 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   // a larger one whose program order follows its dependences closely runs over
   // owned chunks; a CHECK body's time is its rectangles' cells, which the ring
   // spreads better
-  const int own_warps = owned_warps_for(g->max_span, g->last_root);
+  const int own_warps = owned_warps_for(g->max_span, g->last_root, true);
   const bool block = window || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
                                                                g->desc.spin_iters, own_warps > 0));
-  const bool auto_owned = free_shape && !block && own_warps > 0 && g->desc.body != RT_BODY_CHECK;
+  const bool auto_owned = free_shape && !block && own_warps > 0 && g->desc.body != RT_BODY_CHECK &&
+                          body_iters(g) <= kOwnedIters;
   if (auto_owned) owned = true;
   const bool grow = !owned && !block && (cap * 8 > g->ring.cap || !g->ring.p);
   if (grow) {
@@ -1586,8 +1601,15 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   if (g->hpin[kStatusWord] & 2u)
     return fail(RT_ERR_INVALID, "the graph's two halves have different internal edges");
   const bool tickets = (g->desc.flags & RT_GRAPH_TICKETS) != 0;
-  const int wr = owned_warps_for((int32_t)g->hpin[kStatusWord + 1], (int32_t)g->hpin[kStatusWord + 2]);
-  const bool owned = wr > 0 && !tickets && body != RT_BODY_CHECK && g->cfg_blocks == 0 && g->cfg_warps == 0;
+  const int32_t last_root = (int32_t)g->hpin[kStatusWord + 2];
+  const int wr = owned_warps_for((int32_t)g->hpin[kStatusWord + 1], last_root, false);
+  // long bodies: unless all replays' steps are more than the ring's default shape has
+  // lanes for (5000 iterations, a 1024 wide stencil of 50 steps, 2 replays: 1022 us
+  // over owned chunks, 867 by the ring; 20 replays: 1962 and 4909)
+  const bool long_bodies =
+      body_iters(g) > kOwnedIters && ((int64_t)last_root + 1) * replays <= (int64_t)g_dev.num_sms * 64;
+  const bool owned =
+      wr > 0 && !tickets && body != RT_BODY_CHECK && g->cfg_blocks == 0 && g->cfg_warps == 0 && !long_bodies;
   CKR(g->st_count.reserve((size_t)total * 4, s));
   if (!owned) CKR(g->st_ring.reserve((size_t)total * 8, s));
   CKR(g->st_ctrl.reserve(sizeof(ExecCtrl), s));

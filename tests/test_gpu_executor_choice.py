@@ -90,3 +90,12 @@ def test_batches_of_long_independent_bodies(n, iters, in_blocks):
     b.close()
     for g in graphs:
         g.close()
+
+
+def test_owned_chunks_hold_a_whole_step_and_no_long_bodies():
+    ensure_built()
+    assert shape_of(tg.taskbench(1024, 70, "stencil"), 8) == (32, 32)
+    assert shape_of(tg.taskbench(2000, 40, "stencil"), 8) == (64, 32)
+    assert shape_of(tg.taskbench(3000, 30, "stencil"), 1000) == (128, 32)
+    assert shape_of(tg.taskbench(1024, 40, "random", seed=2), 1000) == (32, 32)
+    assert shape_of(tg.taskbench(2000, 10, "stencil"), 2500)[1] == 64  # two warps a block: the ring
