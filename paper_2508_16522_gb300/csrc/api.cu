@@ -1148,6 +1148,13 @@ int owned_warps_for(int32_t span, int32_t last_root, bool alone) {
 // at 1000, 2000 and 5000 iterations: 433, 781 and 1839 us, by the ring 501, 777
 // and 1602; of random fan-in 568, 1001 and 2303, and 789, 1166 and 2341.)
 constexpr int32_t kOwnedIters = 2000;
+// ... and for which a block of 16 warps is better than them: its warps share the
+// SM's four schedulers, and rounds that owned chunks run on an SM each take turns.
+// (300 steps of a 100 wide stencil at 100, 600 and 1200 iterations: 250, 1063 and
+// 2044 us in a block, 333, 762 and 1310 over owned chunks, 805, 1162 and 1559 by the
+// ring; of 100 wide random fan-in at 300 and 600: 586 and 1022, 651 and 983. Up to
+// 70 wide, in a block of 4 warps, the block stays better: 1233 and 1277 at 1200.)
+constexpr int32_t kWindowIters = 512;
 int32_t body_iters(const rt_graph* g) {
   return g->desc.body == RT_BODY_SPIN || g->desc.body == RT_BODY_FMA ? g->desc.spin_iters : 0;
 }
@@ -1161,7 +1168,8 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   // block (not a run that records tickets, holds a task or must reset counters)
   const bool free_shape = !owned && g->cfg_blocks == 0 && g->cfg_warps == 0 && !(g->desc.flags & RT_GRAPH_TICKETS) &&
                           !g->dirty && g->hold_task < 0;
-  const bool window = free_shape && block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters);
+  const bool window = free_shape && block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters) &&
+                      (body_iters(g) <= kWindowIters || block_window_small(g->max_span, g->last_root));
   // a larger one whose program order follows its dependences closely runs over
   // owned chunks; a CHECK body's time is its rectangles' cells, which the ring
   // spreads better

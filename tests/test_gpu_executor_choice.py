@@ -99,3 +99,10 @@ def test_owned_chunks_hold_a_whole_step_and_no_long_bodies():
     assert shape_of(tg.taskbench(3000, 30, "stencil"), 1000) == (128, 32)
     assert shape_of(tg.taskbench(1024, 40, "random", seed=2), 1000) == (32, 32)
     assert shape_of(tg.taskbench(2000, 10, "stencil"), 2500)[1] == 64  # two warps a block: the ring
+
+
+def test_window_of_sixteen_warps_and_long_bodies():
+    ensure_built()
+    assert shape_of(tg.taskbench(100, 60, "stencil"), 500) == (1, 512)
+    assert shape_of(tg.taskbench(100, 60, "stencil"), 1200) == (32, 32)
+    assert shape_of(tg.taskbench(60, 60, "stencil"), 1200) == (1, 128)
