@@ -1145,8 +1145,8 @@ int owned_warps_for(int32_t span, int32_t last_root, bool alone) {
 // The longest bodies for which owned chunks are better than the ring: the tasks
 // of a chunk that become ready at different polls run their bodies one after
 // another, the ring's claims are whole batches. (100 steps of a 1024 wide stencil
-// at 1000, 2000 and 5000 iterations: 433, 781 and 1839 us, by the ring 501, 777
-// and 1602; of random fan-in 568, 1001 and 2303, and 789, 1166 and 2341.)
+// at 1000, 2000 and 5000 iterations: 433, 781 and 1839 us, by the ring 471, 720
+// and 1460; of random fan-in 568, 1001 and 2303, and 737, 1084 and 2145.)
 constexpr int32_t kOwnedIters = 2000;
 // ... and for which a block of 16 warps is better than them: its warps share the
 // SM's four schedulers, and rounds that owned chunks run on an SM each take turns.

@@ -13,10 +13,14 @@ namespace {
 // compiler cannot fold the recurrence (it would in some kernels and not in
 // others): the body costs the same `iters` dependent operations in every
 // executor, which is what its granularity stands for.
-// Eight to a loop step and the remainder by its bits: a rolled loop's branch
-// and counter stood beside each step, and its remainder loop took a branch a
-// step (a stencil of 1024 x 1000 over owned chunks: 0.91 -> 0.76 ms at 8 steps a
-// task, 1.38 -> 1.28 at 128, with the later poll of k_exec_owned).
+// The taken branch of a loop's turn costs 7 cycles, each step 4, so the loop takes
+// several steps a turn and the remainder by its bits. Eight a turn where a hop
+// takes a microsecond or less (owned chunks, inside a block); LONG: 32 a turn
+// before them, in the executors that long bodies are left to (the ring, events,
+// serving). Cycles a step of a body of 8, 64, 256, 1000 and 5000 steps: 9.8, 5.6,
+// 5.1, 5.0, 4.9, and LONG 12.6, 5.3, 4.6, 4.4, 4.4; by the compiler's own
+// unrolling, with a branch a step in the remainder, 23.7, 6.8, 5.0, 4.6, 4.5. (LONG
+// everywhere: 640 mixed graphs x 20 replays of 8 to 15 steps 3.97 -> 4.69 ms.)
 __device__ __forceinline__ void spin_step(uint32_t& x) {
   asm volatile("mad.lo.u32 %0, %0, 1664525, 1013904223;" : "+r"(x));
 }
@@ -25,9 +29,14 @@ __device__ __forceinline__ void spin_steps(uint32_t& x) {
 #pragma unroll
   for (int k = 0; k < N; ++k) spin_step(x);
 }
+template <bool LONG = false>
 __device__ __forceinline__ uint32_t spin_body(uint32_t x, int iters) {
+  if (LONG) {
 #pragma unroll 1
-  for (int k = iters >> 3; k > 0; --k) spin_steps<8>(x);
+    for (int k = iters >> 5; k > 0; --k) spin_steps<32>(x);
+  }
+#pragma unroll 1
+  for (int k = LONG ? (iters >> 3) & 3 : iters >> 3; k > 0; --k) spin_steps<8>(x);
   if (iters & 4) spin_steps<4>(x);
   if (iters & 2) spin_steps<2>(x);
   if (iters & 1) spin_steps<1>(x);
@@ -44,10 +53,15 @@ __device__ __forceinline__ void fma_steps(float& x) {
 #pragma unroll
   for (int k = 0; k < N; ++k) asm volatile("fma.rn.f32 %0, %0, %1, %2;" : "+f"(x) : "f"(0.999f), "f"(0.25f));
 }
+template <bool LONG = false>
 __device__ __forceinline__ int32_t fma_body(uint32_t task, int iters) {
   float x = (float)task;
+  if (LONG) {
 #pragma unroll 1
-  for (int k = iters >> 3; k > 0; --k) fma_steps<8>(x);
+    for (int k = iters >> 5; k > 0; --k) fma_steps<32>(x);
+  }
+#pragma unroll 1
+  for (int k = LONG ? (iters >> 3) & 3 : iters >> 3; k > 0; --k) fma_steps<8>(x);
   if (iters & 4) fma_steps<4>(x);
   if (iters & 2) fma_steps<2>(x);
   if (iters & 1) fma_steps<1>(x);
@@ -106,23 +120,23 @@ __device__ __forceinline__ void check_body(const ExecGraph& G, int j) { G.out[j]
 
 // FENCE = false: the launch only has bodies that read nothing written by
 // other tasks (EMPTY, SPIN, FMA), so the order-sensitive bodies are compiled out.
-template <bool FENCE>
+template <bool FENCE, bool LONG = false>
 __device__ __forceinline__ void run_body(const ExecGraph& G, int j) {
   if (!FENCE) {
     if (G.body == RT_BODY_SPIN) {
-      G.out[j] = (int32_t)spin_body((uint32_t)j, G.spin_iters);
+      G.out[j] = (int32_t)spin_body<LONG>((uint32_t)j, G.spin_iters);
     } else if (G.body == RT_BODY_FMA) {
-      G.out[j] = fma_body((uint32_t)j, G.spin_iters);
+      G.out[j] = fma_body<LONG>((uint32_t)j, G.spin_iters);
     }
     return;
   }
   switch (G.body) {
     case RT_BODY_SPIN: {
-      G.out[j] = (int32_t)spin_body((uint32_t)j, G.spin_iters);
+      G.out[j] = (int32_t)spin_body<LONG>((uint32_t)j, G.spin_iters);
       break;
     }
     case RT_BODY_FMA:
-      G.out[j] = fma_body((uint32_t)j, G.spin_iters);
+      G.out[j] = fma_body<LONG>((uint32_t)j, G.spin_iters);
       break;
     case RT_BODY_COUNTER: {
       const int k = G.body_arg[j];

@@ -157,9 +157,9 @@ __global__ void __launch_bounds__(256) k_events(EvParams p) {
     if (item != kFree) {
       fence_acq_rel_gpu();  // the predecessors' effects before the body
       if (p.G.body == RT_BODY_SPIN) {
-        p.G.out[item] = (int32_t)spin_body(item, p.G.spin_iters);
+        p.G.out[item] = (int32_t)spin_body<true>(item, p.G.spin_iters);
       } else {
-        run_body<true>(p.G, (int)item);
+        run_body<true, true>(p.G, (int)item);
       }
       fence_acq_rel_gpu();  // the body's effects before the trigger
       // TASK_DONE: trigger the event and notify its waiters

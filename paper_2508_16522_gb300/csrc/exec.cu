@@ -250,13 +250,13 @@ __global__ void __launch_bounds__(256, 1) k_exec(ExecParams p) {
       if (TICKETS) p.tickets[2 * (int64_t)v] = (int32_t)atomicAdd(&ctrl->ticket, 1u);
       if (SINGLE && !FENCE) {
         if (body0 == RT_BODY_SPIN) {  // the one graph's fields live in registers
-          out0[v] = (int32_t)spin_body((uint32_t)v, spin0);
+          out0[v] = (int32_t)spin_body<true>((uint32_t)v, spin0);
         } else if (body0 == RT_BODY_FMA) {
-          out0[v] = fma_body((uint32_t)v, spin0);
+          out0[v] = fma_body<true>((uint32_t)v, spin0);
         }
       } else {
         const ExecGraph& G = p.graphs[g];
-        run_body<FENCE>(G, v - G.task_base);
+        run_body<FENCE, true>(G, v - G.task_base);
       }
       if (TICKETS) p.tickets[2 * (int64_t)v + 1] = (int32_t)atomicAdd(&ctrl->ticket, 1u);
     }

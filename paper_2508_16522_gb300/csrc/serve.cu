@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256, 1) k_serve(ServeParams p) {
     if (has) {
       // (no counter re-arm: every served request is analysed afresh)
       if (S.body == RT_BODY_SPIN && S.out) {
-        S.out[v] = (int32_t)spin_body((uint32_t)(v - S.base), S.spin_iters);  // id within its request
+        S.out[v] = (int32_t)spin_body<true>((uint32_t)(v - S.base), S.spin_iters);  // id within its request
       } else if (S.body == RT_BODY_CHECK) {
         const ExecGraph G = check_view(p, slot);
         S.out[v] = (int32_t)check_apply(G, v, (uint32_t)(v - S.base));

@@ -229,14 +229,14 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
       if (TICKETS) p.tickets[2 * slot] = (int32_t)atomicAdd(&ctrl->ticket, 1u);
       const ExecGraph& G = p.G;
       if (G.body == RT_BODY_SPIN) {
-        G.out[slot] = (int32_t)spin_body((uint32_t)v, G.spin_iters);
+        G.out[slot] = (int32_t)spin_body<true>((uint32_t)v, G.spin_iters);
       } else if (G.body == RT_BODY_FMA) {
-        G.out[slot] = fma_body((uint32_t)v, G.spin_iters);
+        G.out[slot] = fma_body<true>((uint32_t)v, G.spin_iters);
       } else if (FENCE) {
         if (G.body == RT_BODY_CHECK) {
           G.out[slot] = (int32_t)check_apply(G, v, (uint32_t)v);
         } else if (G.body == RT_BODY_COUNTER) {
-          run_body<true>(G, v);
+          run_body<true, true>(G, v);
         }
       }
       if (TICKETS) p.tickets[2 * slot + 1] = (int32_t)atomicAdd(&ctrl->ticket, 1u);

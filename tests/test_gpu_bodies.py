@@ -1,0 +1,35 @@
+"""The SPIN and FMA bodies at iteration counts on both sides of their loops'
+turns (32 steps, 8 steps, single ones), in the executors that inline them."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2508_16522_gb300 import grt
+from paper_2508_16522_gb300 import tracegen as tg
+
+from gpu_helpers import ensure_built, gpu_graph
+
+pytestmark = pytest.mark.gpu
+
+TRACE = tg.taskbench(40, 9, "stencil")
+COUNTS = (0, 1, 7, 8, 9, 24, 31, 32, 33, 40, 63, 64, 65, 127, 300)
+
+
+@pytest.mark.parametrize("body", [grt.RT_BODY_SPIN, grt.RT_BODY_FMA])
+@pytest.mark.parametrize("config", [(0, 0, 0, 0), (8, 2, 0, 0)], ids=["default", "ring"])
+def test_iteration_counts(body, config):
+    ensure_built()
+    for iters in COUNTS:
+        g = gpu_graph(TRACE, body=body, spin_iters=iters)
+        g.analyze()
+        g.exec_config(*config)
+        g.execute()
+        g.sync()
+        want = oracle.run_bodies(TRACE, body, spin_iters=iters)[1]
+        assert np.array_equal(g.out.cpu().numpy(), want), iters
+        g.exec_policy(grt.RT_EXEC_OWNED)
+        g.out.zero_()
+        g.execute()
+        g.sync()
+        assert np.array_equal(g.out.cpu().numpy(), want), iters
+        g.close()
