@@ -382,7 +382,8 @@ rt_status rt_batch_capture(const rt_graph_desc* desc, int32_t n_graphs, const in
  * independently of the other graphs. exec_blocks/exec_warps/claim/keep (0 =
  * default) are the launch shape of rt_graph_exec_config; a batch whose graphs
  * all fit (as one graph does there) runs each of them inside one block, several
- * to an SM, whatever the number of blocks and warps given. The batch's counters
+ * to an SM; exec_blocks, where given, still bounds the blocks in flight, and with
+ * them the SMs the batch takes, while exec_warps does not apply. The batch's counters
  * are reset at the start of every launch. The launch {counter reset, seed,
  * executor, status read-back} is captured as a CUDA graph once per launch
  * shape and relaunched from it afterwards (the first launch of a new or

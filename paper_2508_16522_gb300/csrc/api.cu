@@ -2116,13 +2116,21 @@ rt_status prepare_batch_blocks(rt_batch* b) {
   return RT_OK;
 }
 
-rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, bool share, cudaStream_t s) {
+// at_most: the caller's bound on blocks in flight (0: none), split between the two
+// streams by their numbers of graphs; the lists of one stream follow each other.
+rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, bool share, int at_most, cudaStream_t s) {
   CK(cudaMemsetAsync(p.ctrl, 0, sizeof(ExecCtrl), s));  // status, counters and the launches' next graphs
   p.adjx = b->adjx.as<int4>();
   uint32_t* const next[4] = {&p.ctrl->head, &p.ctrl->tail, &p.ctrl->ticket,
                              reinterpret_cast<uint32_t*>(&p.ctrl->executed)};
   const int32_t* const n = b->n_list;
-  const bool both = n[0] + n[2] > 0 && n[1] + n[3] > 0;
+  const int n_large = n[0] + n[2], n_small = n[1] + n[3];
+  const bool both = n_large > 0 && n_small > 0 && at_most != 1;
+  int cap[2] = {at_most, at_most};  // of the large blocks, of the small ones
+  if (at_most > 0 && both) {
+    cap[0] = std::min(std::max((int)((int64_t)at_most * n_large / (n_large + n_small)), 1), at_most - 1);
+    cap[1] = at_most - cap[0];
+  }
   cudaStream_t side = both ? b->side : s;
   if (both) {
     CK(cudaEventRecord(b->fork, s));
@@ -2140,7 +2148,8 @@ rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, bool share, cudaStream
     a.next = next[l];
     a.share = share;
     const bool small = l & 1;
-    const int blocks = std::min(n[l], g_dev.num_sms * (small ? 8 : 2));
+    int blocks = std::min(n[l], g_dev.num_sms * (small ? 8 : 2));
+    if (at_most > 0) blocks = std::min(blocks, cap[small]);
     cudaStream_t on = small ? side : s;
     if (l < 2) launch_exec_window(p, a, blocks, small, on);
     else launch_exec_block(p, a, small ? std::min(b->max_queue_n, kBlockSmall) : b->max_queue_n, blocks, small, on);
@@ -2343,14 +2352,14 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
   if (in_blocks && !b->graph_next) {
     // the first launch direct: a batch run once does not pay for a CUDA graph
     b->graph_next = true;
-    CKR(enqueue_batch_blocks(b, p, share, s));
+    CKR(enqueue_batch_blocks(b, p, share, exec_blocks, s));
   } else if (clear) {
     // a new or dirty ring is cleared whole: a direct launch
     CKR(enqueue_batch(b, p, (int64_t)(b->ring.cap / 8), blocks, warps, s));
   } else {
     // the launch from a cached CUDA graph, captured once per launch shape
     const int64_t key[7] = {replays,
-                            in_blocks ? 0 : blocks,
+                            in_blocks ? exec_blocks : blocks,
                             in_blocks ? 0 : warps,
                             in_blocks && share ? -p.claim : p.claim,
                             p.keep,
@@ -2360,7 +2369,7 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
       drop_batch_graph(b);
       if (!b->cap_stream) CK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
       CK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-      rt_status st = in_blocks ? enqueue_batch_blocks(b, p, share, b->cap_stream)
+      rt_status st = in_blocks ? enqueue_batch_blocks(b, p, share, exec_blocks, b->cap_stream)
                                : enqueue_batch(b, p, 0, blocks, warps, b->cap_stream);
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamEndCapture(b->cap_stream, &graph);
