@@ -283,8 +283,10 @@ rt_status rt_execute_kernels(rt_graph_t g, int32_t mode, int32_t iters, int32_t 
  * order (and whose bodies are short enough for one SM's lanes) runs inside one
  * block (rt_graph_stats then reports 1 block); one whose edges and roots stay
  * within 16384 tasks runs over owned chunks; of the others, one of up to 65534
- * tasks and few roots runs inside one block too, from a queue. Runs with tickets,
- * a held task or the CHECK body keep the ring. rt_execute_stitched picks owned chunks by the same rule. The
+ * tasks and few roots runs inside one block too, from a queue. One block of 8
+ * warps, given, also lets a graph that fits run inside one block (of the library's
+ * own number of warps). Runs with tickets, a held task or the CHECK body keep the
+ * ring. rt_execute_stitched picks owned chunks by the same rule. The
  * event-based executor (rt_execute_events) takes the same claim width. */
 rt_status rt_graph_exec_config(rt_graph_t g, int32_t blocks, int32_t warps, int32_t claim, int32_t keep);
 
@@ -443,8 +445,8 @@ rt_status rt_tune_tile(const rt_graph_desc* desc, int32_t n, const int32_t* req_
 
 /* Runs an analysed graph under candidate launch shapes -- the ring policy by
  * coordinate descent (warps x blocks per SM, then claim, then keep; best of
- * two runs each), the owned policy over its grids and then lanes per task
- * (best of three) -- and
+ * two runs each), one block where the graph fits inside it, the owned policy over
+ * its grids and then lanes per task (best of three) -- and
  * configures it with the fastest policy and shape (rt_graph_exec_policy,
  * rt_graph_exec_config). The graph's bodies run once per trial: a
  * state-changing body sees those runs. Synchronous. */

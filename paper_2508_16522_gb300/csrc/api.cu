@@ -1159,25 +1159,47 @@ int32_t body_iters(const rt_graph* g) {
   return g->desc.body == RT_BODY_SPIN || g->desc.body == RT_BODY_FMA ? g->desc.spin_iters : 0;
 }
 
+// What a graph's runs may use besides the ring and the configured owned chunks,
+// under the ring policy and apart from launch shapes: counters for a window of
+// program order or a queue in one block, owned chunks over own_warps warps. Not for
+// a run that records tickets, holds a task or must reset counters; and a CHECK
+// body's time is its rectangles' cells, which the ring spreads best.
+struct ExecFits {
+  bool window = false, queue = false;
+  int own_warps = 0;
+};
+ExecFits exec_fits(const rt_graph* g) {
+  ExecFits f;
+  if (g->cfg_policy == RT_EXEC_OWNED || (g->desc.flags & RT_GRAPH_TICKETS) || g->dirty || g->hold_task >= 0) return f;
+  f.window = block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters);
+  f.queue = block_exec_fits(g->n, g->n_roots, g->desc.body, g->desc.spin_iters);
+  if (g->desc.body != RT_BODY_CHECK) f.own_warps = owned_warps_for(g->max_span, g->last_root, true);
+  return f;
+}
+
+// One block of the most warps a launch may have: the shape under which a graph
+// that fits runs inside one block, as the library may choose by itself.
+constexpr int kOneBlockWarps = 8;
+
 rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ring_clear) {
   cudaStream_t s = g->s;
   bool owned = g->cfg_policy == RT_EXEC_OWNED;  // no ring: every warp polls the countdowns it owns
   const uint64_t cap = (uint64_t)g->n * (uint64_t)replays + 64;
   if (cap >= 0xFFFFFFF0ull) return fail(RT_ERR_INVALID, "tasks x replays must stay below 2^32 per launch");
   // a graph whose launch shape is left to the library: a narrow one runs inside one
-  // block (not a run that records tickets, holds a task or must reset counters)
-  const bool free_shape = !owned && g->cfg_blocks == 0 && g->cfg_warps == 0 && !(g->desc.flags & RT_GRAPH_TICKETS) &&
-                          !g->dirty && g->hold_task < 0;
-  const bool window = free_shape && block_window_fits(g->max_span, g->last_root, g->desc.body, g->desc.spin_iters) &&
-                      (body_iters(g) <= kWindowIters || block_window_small(g->max_span, g->last_root));
-  // a larger one whose program order follows its dependences closely runs over
-  // owned chunks; a CHECK body's time is its rectangles' cells, which the ring
-  // spreads better
-  const int own_warps = owned_warps_for(g->max_span, g->last_root, true);
-  const bool block = window || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
-                                                               g->desc.spin_iters, own_warps > 0));
-  const bool auto_owned = free_shape && !block && own_warps > 0 && g->desc.body != RT_BODY_CHECK &&
-                          body_iters(g) <= kOwnedIters;
+  // block; a larger one whose program order follows its dependences closely runs
+  // over owned chunks; one whose shape is one block runs inside it if it fits
+  const ExecFits fits = exec_fits(g);
+  const bool free_shape = g->cfg_blocks == 0 && g->cfg_warps == 0;
+  const bool one_block = g->cfg_blocks == 1 && g->cfg_warps == kOneBlockWarps;
+  const bool short_bodies = body_iters(g) <= kWindowIters || block_window_small(g->max_span, g->last_root);
+  const bool window = fits.window && (one_block || (free_shape && short_bodies));
+  const bool queue = fits.queue && !window &&
+                     (one_block || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
+                                                                   g->desc.spin_iters, fits.own_warps > 0)));
+  const bool block = window || queue;
+  const bool auto_owned = free_shape && !block && fits.own_warps > 0 && body_iters(g) <= kOwnedIters;
+  const int own_warps = fits.own_warps;
   if (auto_owned) owned = true;
   const bool grow = !owned && !block && (cap * 8 > g->ring.cap || !g->ring.p);
   if (grow) {
@@ -1350,6 +1372,13 @@ rt_status start_run(rt_graph* g, int32_t replays) {
 }
 
 }  // namespace
+
+namespace grt {
+ExecChoice exec_choice(rt_graph_t g) {
+  const ExecFits f = g->analyzed && g->n > 0 ? exec_fits(g) : ExecFits{};
+  return ExecChoice{f.window || f.queue ? kOneBlockWarps : 0, f.own_warps};
+}
+}  // namespace grt
 
 extern "C" {
 

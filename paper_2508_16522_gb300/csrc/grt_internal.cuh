@@ -587,6 +587,13 @@ size_t graph_footprint(rt_graph_t g);
 void graph_set_mem_cap(rt_graph_t g, size_t cap);
 // releases every device buffer of the graph (stream-ordered) and clears it
 rt_status graph_trim(rt_graph_t g);
+// for the tuner: the warps to configure one block with (ring policy) for an
+// analysed graph to run inside it, and the owned chunks' warps that the library
+// would take for it (0: not so)
+struct ExecChoice {
+  int one_block_warps, own_warps;
+};
+ExecChoice exec_choice(rt_graph_t g);
 rt_status batch_shape(rt_batch_t b, int64_t* graphs, int64_t* tasks, int64_t* edges);
 int32_t static_max_tasks();
 rt_status static_execute(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int32_t n,

@@ -12,9 +12,10 @@
 //   rt_tune_batch  -- the same for a batch launch with its replay count.
 // The executor search is coordinate descent for the ring policy: (warps,
 // blocks per SM) jointly, then the claim width, then the keep width, then
-// (warps, blocks per SM) again; then a pass over the grids of the owned
-// policy, and its group sizes (lanes per task) on the best grid; each ring
-// trial the best of two runs, each owned trial the best of three.
+// (warps, blocks per SM) again; then one block, where the graph fits inside it;
+// then a pass over the grids of the owned policy, the library's own choice among
+// them, and its group sizes (lanes per task) on the best grid; each ring trial the
+// best of two runs, each other trial the best of three.
 // Results go to an optional plain-text cache, one line per workload key
 // (device, SM count, kind, sizes, an input hash), so a later call with the
 // same workload answers without running anything.
@@ -276,9 +277,9 @@ rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* bes
   if (s != RT_OK) return s;
   int sms = 0;
   if ((s = rt_device_info(&sms, nullptr)) != RT_OK) return s;
-  // "exec7": entries for the owned kernel whose decrements are reductions, with
-  // its grids and group sizes (entries of older kernels are never read)
-  const std::string key = "exec7/" + device_tag() + "/" + std::to_string(st.n_tasks) + "/" +
+  // "exec8": entries that also weigh one block and the library's own number of
+  // owned warps (entries of older searches are never read)
+  const std::string key = "exec8/" + device_tag() + "/" + std::to_string(st.n_tasks) + "/" +
                           std::to_string(st.n_edges) + "/" + std::to_string(st.n_roots);
   auto apply = [&](const rt_exec_config& c) -> rt_status {
     rt_status r = rt_graph_exec_policy(g, c.policy);
@@ -305,6 +306,29 @@ rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* bes
     return tfail(s, std::string("executor trial failed: ") + rt_last_error());
   }
   *best = rt_exec_config{sms * b.bps, b.warps, b.claim, b.keep, ms, trials, RT_EXEC_RING};
+  // inside one block, where the graph fits: what the library would do untuned, or
+  // better than what it would do (the widths matter to the queue only)
+  const ExecChoice choice = exec_choice(g);
+  if (choice.one_block_warps > 0) {
+    for (int claim : {32, 1}) {
+      for (int keep : {32, 2}) {
+        double t = 1e30;
+        for (int rep = 0; rep < 3; ++rep) {
+          rt_status r = rt_graph_exec_config(g, 1, choice.one_block_warps, claim, keep);
+          const auto t0 = std::chrono::steady_clock::now();
+          if (r == RT_OK) r = rt_execute(g);
+          if (r == RT_OK) r = rt_sync(g);
+          if (r != RT_OK) {
+            rt_graph_exec_config(g, 0, 0, 0, 0);
+            return tfail(r, std::string("executor trial failed: ") + rt_last_error());
+          }
+          t = std::min(t, std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count());
+        }
+        ++trials;
+        if (t < best->ms) *best = rt_exec_config{1, choice.one_block_warps, claim, keep, (float)t, trials, RT_EXEC_RING};
+      }
+    }
+  }
   rt_graph_exec_policy(g, RT_EXEC_OWNED);
   // the owned policy: grids from 32 warps (a Task Bench step's 32 chunks, each
   // warp always on the same column of chunks) up to several warps per SM, one
@@ -334,6 +358,8 @@ rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* bes
     if (blocks > sms * std::max(exec_max_blocks_per_sm(bw[1]), 1)) continue;
     owned_trial(blocks, bw[1], 1);
   }
+  if (choice.own_warps > 0 && choice.own_warps <= sms * std::max(exec_max_blocks_per_sm(1), 1))
+    owned_trial(choice.own_warps, 1, 1);
   if (!failed && best->policy == RT_EXEC_OWNED) {
     const int gb = best->blocks, gwp = best->warps;
     for (int group : {2, 4}) {

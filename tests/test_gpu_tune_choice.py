@@ -1,0 +1,71 @@
+"""The tuners' answers include what the library does untuned."""
+import time
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2508_16522_gb300 import grt
+from paper_2508_16522_gb300 import tracegen as tg
+
+from gpu_helpers import ensure_built, gpu_graph
+
+pytestmark = pytest.mark.gpu
+
+
+def run_ms(g):
+    """The quickest of 20 runs, host time."""
+    best = 1e9
+    for _ in range(20):
+        t0 = time.perf_counter()
+        g.execute()
+        g.sync()
+        best = min(best, (time.perf_counter() - t0) * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("width,steps,untuned", [(32, 400, (1, 128)), (256, 200, (1, 512)), (5000, 40, (256, 32))])
+def test_a_tuned_graph_is_no_slower_than_an_untuned_one(tmp_path, width, steps, untuned):
+    ensure_built()
+    cache = tmp_path / "tune.txt"
+    tr = tg.taskbench(width, steps, "stencil")
+    g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=8)
+    g.analyze()
+    before = run_ms(g)
+    st = g.stats()
+    assert (st["exec_blocks"], st["exec_threads"]) == untuned
+    c = g.tune(cache)
+    assert run_ms(g) < 1.3 * before
+    st = g.stats()
+    if untuned[0] == 1:
+        assert c["blocks"] == 1 and (st["exec_blocks"], st["exec_threads"]) == untuned
+    g.out.zero_()
+    g.execute()
+    g.sync()
+    want = oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=8)[1]
+    assert np.array_equal(g.out.cpu().numpy(), want)
+    g.exec_config()
+    again = g.tune(cache)  # answered from the cache
+    assert again["trials"] == 0 and all(again[k] == c[k] for k in ("blocks", "warps", "claim", "keep", "policy"))
+    g.out.zero_()
+    g.replay(3)
+    g.sync()
+    assert g.stats()["exec_blocks"] == st["exec_blocks"]
+    assert np.array_equal(g.out.cpu().numpy(), want)
+    g.close()
+
+
+def test_one_block_of_eight_warps_runs_what_does_not_fit_on_the_ring():
+    """The shape lets a graph run inside one block; one that does not fit keeps the ring in that shape."""
+    ensure_built()
+    for tr, iters, threads in ((tg.taskbench(300, 20, "stencil"), 8, 512), (tg.taskbench(2000, 5, "stencil"), 8, 256),
+                               (tg.taskbench(1, 50, "stencil"), 8, 128)):
+        g = gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=iters)
+        g.analyze()
+        g.exec_config(1, 8, 4, 8)
+        g.execute()
+        g.sync()
+        st = g.stats()
+        assert (st["exec_blocks"], st["exec_threads"]) == (1, threads)
+        assert np.array_equal(g.out.cpu().numpy(), oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=iters)[1])
+        g.close()
