@@ -453,7 +453,8 @@ rt_status rt_tune_tile(const rt_graph_desc* desc, int32_t n, const int32_t* req_
 rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* best);
 
 /* The same for a batch launch of `replays` replays: the ring policy by
- * coordinate descent, then one run of the owned policy and, only if that run
+ * coordinate descent (where every graph runs inside one block only the widths,
+ * and blocks and warps are returned as 0), then one run of the owned policy and, only if that run
  * comes within 1.5x of the ring, its grids (1-3 blocks of 4 or 8 warps per SM)
  * and 1, 2 or 4 lanes per task; sets the batch's policy
  * (rt_batch_exec_policy) to the faster one and returns the shape (with its

@@ -2191,6 +2191,9 @@ rt_status enqueue_batch_blocks(rt_batch* b, ExecParams p, bool share, int at_mos
   return RT_OK;
 }
 
+// the batch's launches under the ring policy run each graph inside one block
+bool in_blocks_of(const rt_batch* b) { return b->blocks_fit && b->G_nonempty > 0; }
+
 rt_status prepare_batch_owned(rt_batch* b) {
   if (b->owned_ready) return RT_OK;
   cudaStream_t s = b->s;
@@ -2347,7 +2350,7 @@ rt_status rt_batch_execute(rt_batch_t b, int32_t replays, int32_t exec_blocks, i
     CK(cudaGetLastError());
     return RT_OK;  // the ring was not touched: it stays as clean as the last ring launch left it
   }
-  const bool in_blocks = b->blocks_fit && b->G_nonempty > 0;
+  const bool in_blocks = in_blocks_of(b);
   if (in_blocks) CKR(prepare_batch_blocks(b));
   bool clear = !in_blocks && b->dirty;
   if (!in_blocks && cap * 8 > b->ring.cap) {
@@ -2564,11 +2567,12 @@ void trace(const char* what) {
   fflush(stderr);
 }
 
-rt_status batch_shape(rt_batch_t b, int64_t* graphs, int64_t* tasks, int64_t* edges) {
+rt_status batch_shape(rt_batch_t b, int64_t* graphs, int64_t* tasks, int64_t* edges, bool* in_blocks) {
   if (!b) return fail(RT_ERR_INVALID, "batch is NULL");
   *graphs = b->G;
   *tasks = b->T;
   *edges = b->E;
+  *in_blocks = in_blocks_of(b);
   return RT_OK;
 }
 

@@ -594,7 +594,8 @@ struct ExecChoice {
   int one_block_warps, own_warps;
 };
 ExecChoice exec_choice(rt_graph_t g);
-rt_status batch_shape(rt_batch_t b, int64_t* graphs, int64_t* tasks, int64_t* edges);
+// in_blocks: the ring policy runs each of the batch's graphs inside one block
+rt_status batch_shape(rt_batch_t b, int64_t* graphs, int64_t* tasks, int64_t* edges, bool* in_blocks);
 int32_t static_max_tasks();
 rt_status static_execute(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int32_t n,
                          int64_t n_edges, int32_t spin_iters, int32_t* out, int32_t* tickets, cudaStream_t s,

@@ -382,12 +382,14 @@ rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* bes
 rt_status rt_tune_batch(rt_batch_t b, int32_t replays, const char* cache_path, rt_exec_config* best) {
   if (!b || !best || replays < 1) return tfail(RT_ERR_INVALID, "bad arguments");
   int64_t G = 0, T = 0, E = 0;
-  rt_status s = batch_shape(b, &G, &T, &E);
+  bool in_blocks = false;
+  rt_status s = batch_shape(b, &G, &T, &E, &in_blocks);
   if (s != RT_OK) return s;
   int sms = 0;
   if ((s = rt_device_info(&sms, nullptr)) != RT_OK) return s;
-  // "batch2": entries that also weigh the owned policy (the batch as one DAG)
-  const std::string key = "batch2/" + device_tag() + "/" + std::to_string(G) + "/" + std::to_string(T) + "/" +
+  // "batch3": entries of batches that run in blocks where their graphs fit (older
+  // ones answer for a ring that such a batch no longer runs on)
+  const std::string key = "batch3/" + device_tag() + "/" + std::to_string(G) + "/" + std::to_string(T) + "/" +
                           std::to_string(E) + "/" + std::to_string(replays);
   std::vector<double> c;
   if (cache_get(cache_path, key, &c) && c.size() >= 6) {
@@ -405,10 +407,35 @@ rt_status rt_tune_batch(rt_batch_t b, int32_t replays, const char* cache_path, r
   float ms = 0;
   int trials = 0;
   rt_batch_exec_policy(b, RT_EXEC_RING);
-  const int bps4 = std::max(exec_max_blocks_per_sm(4), 1);
-  if ((s = search(sms, Shape{4, std::min(bps4, 3), 32, 32}, run, &sh, &ms, &trials)) != RT_OK)
-    return tfail(s, std::string("batch trial failed: ") + rt_last_error());
-  *best = rt_exec_config{sms * sh.bps, sh.warps, sh.claim, sh.keep, ms, trials, RT_EXEC_RING};
+  if (in_blocks) {
+    // each graph inside one block: there is no grid to choose, and the widths
+    // matter only to graphs with a queue; a trial has to gain 2 % to count
+    *best = rt_exec_config{0, 0, 0, 0, 1e30f, 0, RT_EXEC_RING};
+    auto trial = [&](int claim, int keep) -> rt_status {
+      float t = 1e30f;
+      for (int rep = 0; rep < 2; ++rep) {
+        float m = 0;
+        rt_status r = rt_batch_execute(b, replays, 0, 0, claim, keep);
+        if (r == RT_OK) r = rt_batch_sync(b, &m);
+        if (r != RT_OK) return r;
+        t = std::min(t, m);
+      }
+      if (++trials == 1 || t < 0.98f * best->ms) *best = rt_exec_config{0, 0, claim, keep, t, trials, RT_EXEC_RING};
+      return RT_OK;
+    };
+    s = trial(0, 0);
+    for (int c : {1, 2, 4, 8, 16, 32})
+      if (s == RT_OK) s = trial(c, 0);
+    const int claim = best->claim;
+    for (int k : {1, 2, 4, 8, 16, 32})
+      if (s == RT_OK) s = trial(claim, k);
+    if (s != RT_OK) return tfail(s, std::string("batch trial failed: ") + rt_last_error());
+  } else {
+    const int bps4 = std::max(exec_max_blocks_per_sm(4), 1);
+    if ((s = search(sms, Shape{4, std::min(bps4, 3), 32, 32}, run, &sh, &ms, &trials)) != RT_OK)
+      return tfail(s, std::string("batch trial failed: ") + rt_last_error());
+    *best = rt_exec_config{sms * sh.bps, sh.warps, sh.claim, sh.keep, ms, trials, RT_EXEC_RING};
+  }
   // the owned policy: one probe at two blocks of 8 warps per SM (one run: on
   // a batch of unrelated graphs a warp's chunks lie in many graphs and one
   // graph's progress waits for the others', so it can be many times slower);

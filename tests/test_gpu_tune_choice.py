@@ -69,3 +69,32 @@ def test_one_block_of_eight_warps_runs_what_does_not_fit_on_the_ring():
         assert (st["exec_blocks"], st["exec_threads"]) == (1, threads)
         assert np.array_equal(g.out.cpu().numpy(), oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=iters)[1])
         g.close()
+
+
+def test_a_batch_in_blocks_is_tuned_without_a_grid(tmp_path):
+    """No bound on the blocks, and the time reported is that of the launch as it runs."""
+    ensure_built()
+    cache = tmp_path / "tune.txt"
+    traces = [tg.taskbench(40 + 13 * k, 60, tg.PATTERNS[k % 3] if k % 3 != 1 else "stencil", seed=k) for k in range(24)]
+    graphs = [gpu_graph(tr, body=grt.RT_BODY_SPIN, spin_iters=7) for tr in traces]
+    for g in graphs:
+        g.analyze()
+    b = grt.Batch(graphs)
+    b.execute(replays=4)
+    b.sync()
+    c = b.tune(replays=4, cache_path=cache)
+    assert c["trials"] >= 10
+    if c["policy"] == grt.RT_EXEC_RING:
+        assert (c["blocks"], c["warps"]) == (0, 0)
+    assert cache.read_text().startswith("batch3/")
+    best = 1e9
+    for _ in range(5):
+        b.execute(replays=4, blocks=c["blocks"], warps=c["warps"], claim=c["claim"], keep=c["keep"])
+        best = min(best, b.sync())
+    assert best < 1.3 * c["ms"]
+    for tr, g in zip(traces, graphs):
+        assert np.array_equal(g.out.cpu().numpy(), oracle.run_bodies(tr, oracle.oracle.BODY_SPIN, spin_iters=7)[1])
+    assert b.tune(replays=4, cache_path=cache)["trials"] == 0
+    b.close()
+    for g in graphs:
+        g.close()
