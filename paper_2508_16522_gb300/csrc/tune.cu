@@ -200,9 +200,9 @@ rt_status rt_tune_tile(const rt_graph_desc* desc, int32_t n, const int32_t* req_
   }
   char hb[32];
   snprintf(hb, sizeof hb, "%016llx", (unsigned long long)h);
-  // "tile3": entries of the sweep with its row mode for segment tiles, and of
-  // the candidate list below (older entries are never read)
-  const std::string key = "tile3/" + device_tag() + "/" + std::to_string(D) + "/" +
+  // "tile4": entries of the sweeps by windows and by plain cells, and of the
+  // candidate list below (older entries are never read)
+  const std::string key = "tile4/" + device_tag() + "/" + std::to_string(D) + "/" +
                           std::to_string(desc->dom_hi[0] - desc->dom_lo[0] + 1) + "x" +
                           std::to_string(D == 2 ? desc->dom_hi[1] - desc->dom_lo[1] + 1 : 1) + "/" +
                           std::to_string(n) + "/" + std::to_string(R) + "/" + hb;

@@ -98,3 +98,16 @@ def test_a_batch_in_blocks_is_tuned_without_a_grid(tmp_path):
     b.close()
     for g in graphs:
         g.close()
+
+
+def test_the_caches_entries_are_of_the_current_kernels(tmp_path):
+    """An entry of an older sweep or executor does not answer: its tile or shape was the best of other kernels."""
+    ensure_built()
+    cache = tmp_path / "tune.txt"
+    tr = tg.random_rects(grid=(200, 200), n=900, rects=(1, 3), side=(1, 30), seed=5)
+    grt.rt_tune_tile(tr, cache)
+    key = cache.read_text().split(" ")[0]
+    assert key.startswith("tile4/")
+    for old in ("tile", "tile2", "tile3"):
+        cache.write_text(f"{old}/{key.split('/', 1)[1]} 8 8 0.001\n")
+        assert grt.rt_tune_tile(tr, cache)[2] > 0.001
