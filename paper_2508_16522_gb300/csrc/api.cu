@@ -209,6 +209,9 @@ size_t footprint_of(const rt_graph* g) {
 
 bool over_cap(size_t grow_by) { return footprint_of(t_capped) + grow_by > t_capped->mem_cap; }
 
+// whether b.reserve(bytes) would fail with RT_ERR_BUDGET: asked where less will do
+bool past_cap(const DevBuf& b, size_t bytes) { return t_capped && (bytes > b.cap || !b.p) && over_cap(std::max<size_t>(bytes, 256)); }
+
 // applies the graph's memory cap to the buffers this thread grows until the
 // scope ends
 struct CapScope {
@@ -857,7 +860,7 @@ rt_status run_analysis(rt_graph* g) {
     while (fbits < 27 && (1ll << fbits) < 2 * M) ++fbits;
     fslots = fbits - bits_for((uint64_t)(n - 1));  // n <= M / 16 < 2^26, so at least 1
     const size_t fbytes = (size_t)4 << fbits;
-    if (fbytes > g->pfilt.cap && t_capped && over_cap(fbytes - g->pfilt.cap)) fbits = 0;
+    if (past_cap(g->pfilt, fbytes)) fbits = 0;
     else CKR(g->pfilt.reserve(fbytes, s));
   }
   g->pair_filter_bits = fbits;
@@ -867,10 +870,11 @@ rt_status run_analysis(rt_graph* g) {
   // entries make many class cells of a window and many walks back. Its warps
   // take chunks of about a quarter of a warp's share, and small buffer chunks:
   // with the filter few pairs are written, and each warp leaves holes in its
-  // last chunk.
+  // last chunk. (Where the larger pair buffer that goes with them would not
+  // leave the CSR its room under the graph's memory cap, the tiles are swept as
+  // they are.)
   const double cover = M > 0 ? (double)h64[4] / ((double)M * d.tw * d.th) : 0.0;
-  const bool by_windows = M > 0 && cover >= kWindowCover && (fbits > 0 || M >= (int64_t)kWindowTileEntries * ntiles);
-  if (by_windows && !fbits) guess *= 2;
+  bool by_windows = M > 0 && cover >= kWindowCover && (fbits > 0 || M >= (int64_t)kWindowTileEntries * ntiles);
   // entries of a few cells each need no classes (at most one in 64 can then cover
   // a 256-cell tile), unless the tiles hold so few that clearing all cells costs more
   const bool plain = M > 0 && (double)h64[4] <= kPlainCells * (double)M && d.tw * d.th <= kMaxClassCells &&
@@ -883,11 +887,15 @@ rt_status run_analysis(rt_graph* g) {
     const int64_t ww = (int64_t)wblocks * kWindowWarps;
     wspan = (int)std::min<int64_t>(512, (M / (4 * ww) + 15) / 16 * 16);
     wspan = std::max(wspan, 16);
-    while (wchunk < 512 && 32ull * wchunk * (unsigned long long)ww <= guess) wchunk <<= 1;
+    const unsigned long long wguess = fbits ? guess : 2 * guess;
+    while (wchunk < 512 && 32ull * wchunk * (unsigned long long)ww <= wguess) wchunk <<= 1;
+    const unsigned long long more = wguess - guess + (unsigned long long)ww * wchunk;
+    const size_t all = (size_t)((unsigned long long)Pe + guess + W * chunk + more);
+    // the CSR's buffers come after it: 8 bytes a pair and up to 128 a task
+    if (past_cap(g->pairs, all * 16 + (size_t)n * 128)) by_windows = false;
+    else guess += more;
   }
-  unsigned long long cap =
-      (unsigned long long)Pe +
-      (M > 0 ? guess + W * chunk + (unsigned long long)wblocks * kWindowWarps * wchunk : 0ull);
+  unsigned long long cap = (unsigned long long)Pe + (M > 0 ? guess + W * chunk : 0ull);
   CKR(g->pairs.reserve((size_t)std::max<unsigned long long>(cap, 1) * 8, s));
   if (Pe > 0)
     launch_explicit_pairs(g->pred_off.as<int32_t>(), g->pred.as<int32_t>(), n, B, g->pairs.as<uint64_t>(), s);
