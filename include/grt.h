@@ -176,7 +176,9 @@ rt_status rt_graph_clear(rt_graph_t g);
  *  body_arg int32[n] (optional; required for COUNTER): per-task body argument
  *  flags    RT_LAUNCH_HOST / RT_LAUNCH_DEVICE / RT_LAUNCH_DEFER_CHECK
  * The arrays are copied; the caller keeps ownership (pinned host arrays are
- * copied asynchronously and must stay valid until rt_analyze returns). Errors: RT_ERR_INVALID
+ * copied asynchronously and must stay valid until rt_analyze returns; a large
+ * host-validated batch whose stream is idle is checked on the device, and the
+ * call then waits for its own copies). Errors: RT_ERR_INVALID
  * (with host validation nothing is appended), RT_ERR_STATE (graph already
  * analyzed: call rt_graph_clear first), RT_ERR_OOM, RT_ERR_CUDA. */
 rt_status rt_launch_batch(rt_graph_t g, int32_t n, const int32_t* req_off, const int64_t* lo,

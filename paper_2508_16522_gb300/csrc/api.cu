@@ -16,6 +16,7 @@
 #include <time.h>
 #include <cstring>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "grt_internal.cuh"
@@ -484,6 +485,18 @@ bool kernel_reads(const void* p) {
   return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
+// whether the stream has nothing left to do, now or within ns nanoseconds
+bool idle_within(cudaStream_t s, int64_t ns) {
+  const auto until = std::chrono::steady_clock::now() + std::chrono::nanoseconds(ns);
+  for (;;) {
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e == cudaSuccess) return true;
+    cudaGetLastError();
+    if (e != cudaErrorNotReady || std::chrono::steady_clock::now() >= until) return false;
+    std::this_thread::yield();
+  }
+}
+
 // The word that a batch's device checks report to: word 0 gathers the deferred
 // checks' findings until the analysis, word 1 is one call's own.
 rt_status ready_err(rt_graph* g, bool now, uint32_t** err) {
@@ -574,6 +587,9 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
         cudaGetLastError();
         check_now = false;
       }
+      // the check waits for the stream: not for work queued there before this
+      // call, beyond the time that the host's check takes
+      if (check_now) check_now = idle_within(g->s, (int64_t)n + R + Pb);
       if (!check_now) CKR(on_host());
     }
   }
