@@ -473,9 +473,10 @@ rt_status copy_in(void* dst, const void* src, size_t bytes, cudaStream_t s) {
   return RT_OK;
 }
 
-// memory of the current device (a kernel may not reach another device's, which a
-// copy does)
-bool kernel_reads(const void* p) {
+// memory of the current device, aligned for its elements (a kernel may not reach
+// another device's, nor an odd address, which a copy does)
+bool kernel_reads(const void* p, size_t element) {
+  if (reinterpret_cast<uintptr_t>(p) % element != 0) return false;
   cudaPointerAttributes a;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -601,7 +602,7 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     const int32_t* const at[4] = {req_off, req_off + n, pred_off, pred_off ? pred_off + n : nullptr};
     ReportArgs ra;
     for (int k = 0; k < (pred_off ? 4 : 2); ++k) {
-      if (kernel_reads(at[k])) ra.add(g->hpin + k, at[k]);
+      if (kernel_reads(at[k], 4)) ra.add(g->hpin + k, at[k]);
       else CK(cudaMemcpyAsync(g->hpin + k, at[k], 4, cudaMemcpyDefault, s));
     }
     launch_report(ra, s);
@@ -638,7 +639,7 @@ rt_status append_launches(rt_graph_t g, int32_t n, const int32_t* req_off, const
     int64_t* const dhi = g->hi.as<int64_t>() + R0 * D;
     uint8_t* const dpriv = g->priv.as<uint8_t>() + R0;
     // read where they are, when a kernel may
-    const bool direct = dev && kernel_reads(lo) && kernel_reads(hi) && kernel_reads(priv);
+    const bool direct = dev && kernel_reads(lo, c32 ? 4 : 8) && kernel_reads(hi, c32 ? 4 : 8) && kernel_reads(priv, 1);
     const bool check = (on_device_check || check_now) && !bp;  // a placed batch is checked after its placement
     if (check) CKR(ready_err(g, check_now, &err));
     const void *from_lo = lo, *from_hi = hi;
