@@ -284,7 +284,8 @@ rt_status rt_execute_kernels(rt_graph_t g, int32_t mode, int32_t iters, int32_t 
  * graph of any size whose edges and roots reach at most 700 tasks of program
  * order (and whose bodies are short enough for one SM's lanes) runs inside one
  * block (rt_graph_stats then reports 1 block); one whose edges and roots stay
- * within 16384 tasks runs over owned chunks; of the others, one of up to 65534
+ * within 16384 tasks runs over owned chunks, whose warps (up to 256, of up to half
+ * of each SM) start together once all of them have their places; of the others, one of up to 65534
  * tasks and few roots runs inside one block too, from a queue. One block of 8
  * warps, given, also lets a graph that fits run inside one block (of the library's
  * own number of warps). Runs with tickets, a held task or the CHECK body keep the

@@ -99,7 +99,7 @@ struct DevBuf {
 
 struct DeviceInfo {
   bool init = false;
-  int device = -1, num_sms = 0, exec_bps = 0;
+  int device = -1, num_sms = 0, exec_bps = 0, owned_warps = 0, stitch_warps = 0;
 };
 DeviceInfo g_dev;
 std::mutex g_dev_mu;
@@ -115,6 +115,8 @@ rt_status ensure_device() {
   g_dev.num_sms = prop.multiProcessorCount;
   g_dev.exec_bps = exec_max_blocks_per_sm(8);
   if (g_dev.exec_bps < 1) g_dev.exec_bps = 1;
+  g_dev.owned_warps = owned_max_warps();
+  g_dev.stitch_warps = stitch_owned_max_warps();
   g_dev.init = true;
   return RT_OK;
 }
@@ -1223,7 +1225,8 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
                      (one_block || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
                                                                    g->desc.spin_iters, fits.own_warps > 0)));
   const bool block = window || queue;
-  const bool auto_owned = free_shape && !block && fits.own_warps > 0 && body_iters(g) <= kOwnedIters;
+  const bool auto_owned = free_shape && !block && fits.own_warps > 0 && fits.own_warps <= g_dev.owned_warps &&
+                          body_iters(g) <= kOwnedIters;
   const int own_warps = fits.own_warps;
   if (auto_owned) owned = true;
   const bool grow = !owned && !block && (cap * 8 > g->ring.cap || !g->ring.p);
@@ -1671,7 +1674,7 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   const bool long_bodies =
       body_iters(g) > kOwnedIters && ((int64_t)last_root + 1) * replays <= (int64_t)g_dev.num_sms * 64;
   const bool owned =
-      wr > 0 && !tickets && body != RT_BODY_CHECK && g->cfg_blocks == 0 && g->cfg_warps == 0 && !long_bodies;
+      wr > 0 && wr + kStitchOwnedWarps <= g_dev.stitch_warps && !tickets && body != RT_BODY_CHECK && g->cfg_blocks == 0 && g->cfg_warps == 0 && !long_bodies;
   CKR(g->st_count.reserve((size_t)total * 4, s));
   if (!owned) CKR(g->st_ring.reserve((size_t)total * 8, s));
   CKR(g->st_ctrl.reserve(sizeof(ExecCtrl), s));
@@ -1715,7 +1718,7 @@ rt_status rt_execute_stitched(rt_graph_t g, int32_t replays, float* ms_kernel) {
   CK(cudaEventRecord(g->ev[EV_E0], s));
   if (owned) {
     // each replay its own warps, up to two warps a scheduler
-    const int groups = std::max(1, std::min(replays, g_dev.num_sms * 8 / wr));
+    const int groups = std::max(1, std::min(replays, std::min(g_dev.num_sms * 8, g_dev.stitch_warps - kStitchOwnedWarps) / wr));
     launch_stitch_owned(p, g->max_outdeg > kAdjInline ? g->adjx.as<int4>() : nullptr, g->indeg.as<int32_t>(), wr, groups,
                         body == RT_BODY_COUNTER, s);
   } else {

@@ -876,6 +876,11 @@ void launch_exec(ExecParams p, int blocks, int warps, cudaStream_t s) {
   const bool single = p.n_graphs == 1;
   const bool fence = p.need_fence != 0;
   count_launch();
+  if (p.auto_warps > 0) {  // owned chunks picked by the library
+    if (fence) launch_together(k_exec_owned<false, true, 1, false>, blocks, warps * 32, s, p);
+    else launch_together(k_exec_owned<false, false, 1, false>, blocks, warps * 32, s, p);
+    return;
+  }
   if (p.policy == RT_EXEC_OWNED && (single || p.task_graph)) {  // keeps nothing in shared memory
     // the claim width is the group size: lanes per task (1, 2 or 4)
     const int Lg = p.claim >= 4 ? 4 : (p.claim >= 2 ? 2 : 1);
@@ -904,6 +909,15 @@ void launch_exec(ExecParams p, int blocks, int warps, cudaStream_t s) {
     else { if (fence) GRT_EXEC(false, true, false); else GRT_EXEC(false, false, false); }
   }
 #undef GRT_EXEC
+}
+
+int owned_max_warps() {
+  int dev = 0, sms = 0, a = 0, b = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_exec_owned<false, false, 1, false>, 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_exec_owned<false, true, 1, false>, 32, 0);
+  return sms * (std::min(a, b) / 2);
 }
 
 void preload_exec() {

@@ -412,6 +412,28 @@ void launch_rebase_roots(const uint64_t* src, uint64_t* dst, int32_t n, int32_t 
                          cudaStream_t s);
 void launch_seed(ExecParams p, int64_t ring_clear, cudaStream_t s);
 void launch_exec(ExecParams p, int blocks, int warps, cudaStream_t s);
+// A kernel whose warps wait for one another, as one cooperative launch: it starts
+// when all of its blocks have their places, never with some of them while others
+// hold the rest of the device (the warps that had started would then wait for the
+// ones that could not, until the graph's limit). No slower than a plain launch.
+template <class... P, class... A>
+cudaError_t launch_together(void (*kernel)(P...), int blocks, int threads, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)blocks);
+  lc.blockDim = dim3((unsigned)threads);
+  lc.stream = s;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, P(args)...);
+}
+// the warps of owned chunks that the library may take by itself (one replay's, and
+// all replays' of a stitched run): what half of every SM holds, so that they find
+// their places beside a resident server
+int owned_max_warps();
+int stitch_owned_max_warps();
 int exec_max_blocks_per_sm(int warps);
 // small graphs inside one block each (block_exec.cu). The bounds: task ids of 16
 // bits; 2 bytes of shared memory a task for its countdown and 2 for the first

@@ -341,8 +341,10 @@ __global__ void __launch_bounds__(256, 1) k_stitch(StitchParams p) {
 // tasks, one task per lane, polling their counters. A hop costs a reduction and
 // the owner's next poll instead of a trip through the ring, and the replays
 // still overlap: each has its own warps. Every edge leads to a later (replay,
-// task), every warp takes its chunks in that order and all warps are resident,
-// so the first unfinished task is always held with its predecessors done.
+// task), every warp takes its chunks in that order and all warps start together,
+// so the first unfinished task is always held with its predecessors done. (Chunks
+// claimed by whichever warp is free would ask for no more than one of them, but a
+// warp then gets two of a step: random fan-in of 1024 over owned chunks 390 -> 549 us.)
 template <bool FENCE>
 __global__ void __launch_bounds__(256) k_stitch_owned(StitchParams p, const int4* adjx, int wr, int groups) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -480,8 +482,17 @@ void launch_stitch_owned(const StitchParams& p, const int4* adjx, const int32_t*
   count_launch(2);
   k_st_init<<<1024, 256, 0, s>>>(p, indeg, nullptr, nullptr);
   const int blocks = (wr * groups + kStitchOwnedWarps - 1) / kStitchOwnedWarps;
-  if (fence) k_stitch_owned<true><<<blocks, kStitchOwnedWarps * 32, 0, s>>>(p, adjx, wr, groups);
-  else k_stitch_owned<false><<<blocks, kStitchOwnedWarps * 32, 0, s>>>(p, adjx, wr, groups);
+  if (fence) launch_together(k_stitch_owned<true>, blocks, kStitchOwnedWarps * 32, s, p, adjx, wr, groups);
+  else launch_together(k_stitch_owned<false>, blocks, kStitchOwnedWarps * 32, s, p, adjx, wr, groups);
+}
+
+int stitch_owned_max_warps() {
+  int dev = 0, sms = 0, a = 0, b = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_stitch_owned<false>, kStitchOwnedWarps * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_stitch_owned<true>, kStitchOwnedWarps * 32, 0);
+  return sms * (std::min(a, b) / 2) * kStitchOwnedWarps;
 }
 
 void preload_stitch() {
