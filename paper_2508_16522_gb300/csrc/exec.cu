@@ -122,8 +122,9 @@ __global__ void __launch_bounds__(256, 1) k_exec(ExecParams p) {
   // and when a single graph's next run must find its counters re-armed. A
   // release before each published item and an acquire at each poll of a slot
   // cost a hop through the ring most of a microsecond: without them a random
-  // 1024 x 300 Task Bench graph runs in 1.26 ms instead of 1.60, 640 mixed
-  // graphs x 20 replays in 34.8 instead of 46.5.
+  // 1024 x 300 Task Bench graph took 1.26 ms instead of 1.60 on 152 blocks of 2
+  // warps, and 640 mixed graphs x 20 replays 34.8 instead of 46.5, when they ran on
+  // the ring.
   const bool ordered = FENCE || TICKETS || (SINGLE && p.replays > 1);
   uint32_t cnt[kCntCount];  // diagnostics, per warp (lane 0's copy is added to the totals at exit)
 #pragma unroll
@@ -246,7 +247,11 @@ __global__ void __launch_bounds__(256, 1) k_exec(ExecParams p) {
     q.bat[lane][0] = a0;
     q.bat[lane][1] = a1;
     if (has) {
-      if (SINGLE) p.count[v] = a0.z;  // INIT's reset, done by the task itself for the next run
+      // INIT's reset, done by the task itself for the next run: an addition, which
+      // leaves the in-degree however it stands to the decrements of the task's
+      // predecessors (an item polled without acquire is not ordered after them, as a
+      // store would have to be)
+      if (SINGLE && a0.z) red_add_s32(p.count + v, a0.z);
       if (TICKETS) p.tickets[2 * (int64_t)v] = (int32_t)atomicAdd(&ctrl->ticket, 1u);
       if (SINGLE && !FENCE) {
         if (body0 == RT_BODY_SPIN) {  // the one graph's fields live in registers
@@ -571,7 +576,9 @@ __global__ void __launch_bounds__(256, 1) k_exec_owned(ExecParams p) {
       pending &= ~rm;
       if (FENCE) fence_acq_rel_gpu();  // acquire: the predecessors' effects before the bodies
       if (ready && is_head) {
-        p.count[v] = q[0].z;  // INIT's reset for the next run, done by the task itself
+        // INIT's reset for the next run, done by the task itself: after the last
+        // decrement, whose 0 this lane has read from the word
+        st_relaxed_s32(p.count + v, q[0].z);
         if (TICKETS) p.tickets[2 * (int64_t)v] = (int32_t)atomicAdd(&ctrl->ticket, 1u);
         if (batched) {
           const ExecGraph& Gv = p.graphs[gi];  // a batched body sees its graph's own task ids
