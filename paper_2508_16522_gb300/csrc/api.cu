@@ -1998,8 +1998,7 @@ rt_status rt_batch_create(const rt_graph_t* graphs, int32_t n_graphs, void* stre
     rb += g->n_roots;
   }
   if ((st = b->adj.reserve((size_t)std::max<int64_t>(T, 1) * 32, s))) return bail(st);
-  launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(),
-                  nullptr, s);
+  launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(), s);
   if ((st = finish_batch(b, table)) != RT_OK) return bail(st);
   *out = b;
   return RT_OK;
@@ -2113,8 +2112,7 @@ rt_status rt_batch_create_stacked(rt_graph_t g, const int32_t* task_off, int32_t
     tmp.release(s);
     return bail(st);
   }
-  launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(),
-                  nullptr, s);
+  launch_pack_adj(b->row_ptr.as<int32_t>(), b->col.as<int32_t>(), b->indeg.as<int32_t>(), T, b->adj.as<int4>(), s);
   st = finish_batch(b, table);
   tmp.release(s);
   if (st != RT_OK) return bail(st);

@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(256, 1) k_exec(ExecParams p) {
 // issues from 4R to 4R / L. Successors past the record take the warp-shared
 // path through the CSR's columns. No ring, no reservation, no record load on
 // the critical path: a wavefront step costs a reduction reaching L2 and the
-// owner's next poll (issued before the wave's bodies run, and read after).
+// owner's next poll (issued behind the wave's reductions).
 // Every warp takes its chunks in increasing task order and holds its oldest
 // unfinished one, and every edge points to a later task, so the smallest
 // unfinished task is always in a chunk its owner holds, with all its
@@ -671,15 +671,9 @@ __global__ void __launch_bounds__(256, 1) k_exec_owned(ExecParams p) {
 }
 
 // trigger record of each task: {row start, out-degree, in-degree, first
-// kAdjInline successors (-1 padded)}, two int4 per task; optionally the
-// largest out-degree (atomicMax into *maxdeg)
-__global__ void k_pack_adj(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int64_t n,
-                           int4* adj, uint32_t* maxdeg) {
+// kAdjInline successors (-1 padded)}, two int4 per task
+__global__ void k_pack_adj(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int64_t n, int4* adj) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (maxdeg) {  // uniform over the grid: every lane of a warp reaches the reduction
-    const uint32_t m = __reduce_max_sync(0xffffffffu, v < n ? (uint32_t)(row_ptr[v + 1] - row_ptr[v]) : 0u);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(maxdeg, m);
-  }
   if (v >= n) return;
   const int b = row_ptr[v], d = row_ptr[v + 1] - b;
   int c[kAdjInline];
@@ -776,10 +770,10 @@ void launch_check_stacked(const int32_t* row_ptr, const int32_t* col, int64_t T,
 }
 
 void launch_pack_adj(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int64_t n, int4* adj,
-                     uint32_t* maxdeg, cudaStream_t s) {
+                     cudaStream_t s) {
   if (n > 0) {
     count_launch();
-    k_pack_adj<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(row_ptr, col, indeg, n, adj, maxdeg);
+    k_pack_adj<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(row_ptr, col, indeg, n, adj);
   }
 }
 

@@ -403,9 +403,8 @@ struct ReportArgs {
 };
 void launch_report(const ReportArgs& a, cudaStream_t s);
 
-// maxdeg (nullable, zeroed by the caller): receives the largest out-degree
 void launch_pack_adj(const int32_t* row_ptr, const int32_t* col, const int32_t* indeg, int64_t n, int4* adj,
-                     uint32_t* maxdeg, cudaStream_t s);
+                     cudaStream_t s);
 void launch_pack_adjx(const int32_t* row_ptr, const int32_t* col, int64_t n, int4* adjx, cudaStream_t s);
 void launch_fill_task_graph(const ExecGraph* graphs, int32_t G, int32_t* out, cudaStream_t s);
 void launch_max_outdeg(const int32_t* row_ptr, int64_t n, uint32_t* out, cudaStream_t s);

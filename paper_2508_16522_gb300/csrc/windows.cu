@@ -47,6 +47,7 @@ namespace grt {
 
 namespace {
 constexpr unsigned kFullW = 0xffffffffu;
+constexpr int kNew = 16;        // new candidates per window
 constexpr int kMaxCells = 640;  // class cells of a window; more: small boxes, cheaper one by one
 constexpr int kMaxSteps = 512;  // 32-candidate steps of one window's walks
 constexpr int kMaxWalk = 16;    // ... of one walk
@@ -255,17 +256,17 @@ __device__ __forceinline__ bool walk_back(Sink& x, const SweepOut& o, const uint
   return true;
 }
 
-// NEW: new candidates per window (16 or 8; 32 / NEW parts of the warp take
-// different cells); look: at most this many candidates before them.
+// kNew new candidates a window and the 32 - kNew before them; the warp's 32 / kNew
+// parts take different cells.
 // WIDE: tiles of more than 32 columns or rows (and 1-D ones), whose class
 // starts are found among the boxes' own edges instead of in a word of bits.
-template <int NEW, bool WIDE>
+template <bool WIDE>
 __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ payload, const uint32_t* __restrict__ keys,
                                                 const uint32_t* __restrict__ seg_begin,
-                                                const uint32_t* __restrict__ seg_end, int M, int span, int look,
+                                                const uint32_t* __restrict__ seg_end, int M, int span,
                                                 AnalysisDims d, SweepOut o, uint8_t* __restrict__ bail,
                                                 uint32_t* nbail) {
-  constexpr int PARTS = 32 / NEW;
+  constexpr int NEW = kNew, PARTS = 32 / NEW;
   __shared__ uint64_t before[kWindowWarps][32];  // the block before the window, where some cell asked for it
   const int lane = threadIdx.x & 31;
   uint64_t* const first = before[threadIdx.x >> 5];
@@ -273,7 +274,6 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
   const unsigned me = 1u << k;
   const unsigned gt = ~((2u << k) - 1u);
   const unsigned newbits = (1u << NEW) - 1u;
-  const unsigned lookbits = NEW + look >= 32 ? kFullW : (1u << (NEW + look)) - 1u;
   const int tw = d.ndim == 1 ? 1 : d.tw, th = d.ndim == 1 ? d.tw : d.th;
   const unsigned colbits = tw >= 32 ? kFullW : (1u << tw) - 1u;
   const unsigned rowbits = th >= 32 ? kFullW : (1u << th) - 1u;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
         }
       }
       // the oldest whole task, or the task of the last full-tile write before the new ones
-      int hs = 31 - __clz((int)(st0 & lookbits));
+      int hs = 31 - __clz((int)st0);
       bool more = pos + NEW - 1 - hs > sb;
       const unsigned fw = __ballot_sync(kFullW, in && e.priv == kKindWrite && e.x0 == 0 && e.y0 == 0 && e.x1 == fx &&
                                                     e.y1 == fy) &
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(256, 4) k_window(const uint64_t* __restrict__ 
       // ---- the pairs: the parts share each candidate's mask --------------------
 #pragma unroll
       for (int s = NEW; s < 32; s <<= 1) acc |= __shfl_xor_sync(kFullW, acc, s);
-      const unsigned share = PARTS == 2 ? 0x55555555u : 0x11111111u;
+      constexpr unsigned share = 0x55555555u;  // every PARTS-th bit
       emit(x, o, acc & (share << part), task, dst);
       if (b1.lo >= 0) {
 #pragma unroll
@@ -551,22 +551,22 @@ void launch_window(const uint64_t* payload, const uint32_t* keys, const uint32_t
                    cudaStream_t s) {
   count_launch();
   if (wide_tile(d))
-    k_window<16, true><<<blocks, 256, 0, s>>>(payload, keys, seg_begin, seg_end, (int)M, span, 16, d, o, bail, nbail);
+    k_window<true><<<blocks, 256, 0, s>>>(payload, keys, seg_begin, seg_end, (int)M, span, d, o, bail, nbail);
   else
-    k_window<16, false><<<blocks, 256, 0, s>>>(payload, keys, seg_begin, seg_end, (int)M, span, 16, d, o, bail, nbail);
+    k_window<false><<<blocks, 256, 0, s>>>(payload, keys, seg_begin, seg_end, (int)M, span, d, o, bail, nbail);
 }
 
 int window_blocks_per_sm(const AnalysisDims& d) {
   int nb = 0;
-  if (wide_tile(d)) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_window<16, true>, 256, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_window<16, false>, 256, 0);
+  if (wide_tile(d)) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_window<true>, 256, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_window<false>, 256, 0);
   return nb < 1 ? 1 : nb;
 }
 
 void preload_window() {
   cudaFuncAttributes a;
-  cudaFuncGetAttributes(&a, k_window<16, false>);
-  cudaFuncGetAttributes(&a, k_window<16, true>);
+  cudaFuncGetAttributes(&a, k_window<false>);
+  cudaFuncGetAttributes(&a, k_window<true>);
 }
 
 }  // namespace grt
