@@ -143,7 +143,9 @@ typedef struct {
                                pair filter may have (as many, a power of two, for each task), which
                                the first sweep wrote through (a pair found again in
                                another tile is not written again); 0: no filter */
-  int32_t pad1;
+  int32_t windows_left;   /* dense tiles are swept by windows of candidates: how many windows that sweep
+                             gave up, whose tiles it left to the sweep tile by tile; -1: it did not
+                             run; -2: the pairs overflowed its buffer, and all tiles were swept again */
   /* diagnostic counters of the last executor launch: batches, tasks, edges,
    * ring claims, failed claim CASes, items published to the ring, idle polls,
    * waits for a reserved slot, ready successors kept by their warp */

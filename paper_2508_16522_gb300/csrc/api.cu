@@ -152,6 +152,7 @@ struct rt_graph {
   int32_t max_outdeg = 0;  // largest out-degree of the analysed graph
   int32_t max_span = 0, last_root = 0;  // its longest edge (target - source) and last root
   DevBuf pfilt;   // dense inputs: the first sweep's pair-key filter
+  int windows_left = -1;     // of the last analysis (rt_graph_stats)
   int pair_filter_bits = 0;  // log2 of its slots in the last analysis (0: not used)
   DevBuf bucket;  // CSR by buckets: per-task counts, offsets, distinct counts, long-row list, control words
   // the event-based executor (rt_execute_events): in-edges, events, waiter nodes
@@ -883,6 +884,7 @@ rt_status run_analysis(rt_graph* g) {
     else CKR(g->pfilt.reserve(fbytes, s));
   }
   g->pair_filter_bits = fbits;
+  g->windows_left = -1;
   // Entries that cover a fair part of their tiles are swept by windows
   // (windows.cu): on dense inputs (with the filter), or where each tile holds so
   // many entries that its one warp is the analysis's longest chain. Thinner
@@ -972,6 +974,7 @@ rt_status run_analysis(rt_graph* g) {
       if (prof) CK(cudaEventRecord(g->ev[EV_SW1], s));
       trace("analyze: sweep enqueued");
       CKR(count_pairs());
+      if (win) g->windows_left = (int)h64[7];
       if (win && (unsigned long long)h64[3] <= cap && h64[7] != 0) {
         // tiles that the windows left
         o.only = flags1;
@@ -986,6 +989,7 @@ rt_status run_analysis(rt_graph* g) {
       // end (more distinct pairs than twice the entries): swept again from the
       // start by tiles, which do
       if (!win || (unsigned long long)h64[3] <= cap) break;
+      g->windows_left = -2;
     }
     trace("analyze: sweep synced");
     Ptot = (int64_t)h64[3];
@@ -1776,6 +1780,7 @@ rt_status rt_graph_stats(rt_graph_t g, rt_graph_stats_t* out) {
   out->n_pairs = g->n_pairs;
   out->csr_by_buckets = g->csr_by_buckets ? 1 : 0;
   out->pair_filter_bits = g->pair_filter_bits;
+  out->windows_left = g->windows_left;
   out->n_edges = g->n_edges;
   out->n_roots = g->n_roots;
   out->tile_w = g->dims.tw;
