@@ -453,7 +453,7 @@ rt_status rt_tune_tile(const rt_graph_desc* desc, int32_t n, const int32_t* req_
  * two runs each), one block where the graph fits inside it, the owned policy over
  * its grids and then lanes per task (best of three) -- and
  * configures it with the fastest policy and shape (rt_graph_exec_policy,
- * rt_graph_exec_config). The graph's bodies run once per trial: a
+ * rt_graph_exec_config; one block that the library takes by itself is left to it). The graph's bodies run once per trial: a
  * state-changing body sees those runs. Synchronous. */
 rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* best);
 

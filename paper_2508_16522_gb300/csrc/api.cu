@@ -1208,6 +1208,14 @@ ExecFits exec_fits(const rt_graph* g) {
   return f;
 }
 
+// of these, one block for a graph whose launch shape is left to the library
+bool window_best(const rt_graph* g) {
+  return body_iters(g) <= kWindowIters || block_window_small(g->max_span, g->last_root);
+}
+bool queue_best(const rt_graph* g, const ExecFits& f) {
+  return block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body, g->desc.spin_iters, f.own_warps > 0);
+}
+
 // One block of the most warps a launch may have: the shape under which a graph
 // that fits runs inside one block, as the library may choose by itself.
 constexpr int kOneBlockWarps = 8;
@@ -1223,11 +1231,8 @@ rt_status prepare_run(rt_graph* g, int32_t replays, ExecParams* out, int64_t* ri
   const ExecFits fits = exec_fits(g);
   const bool free_shape = g->cfg_blocks == 0 && g->cfg_warps == 0;
   const bool one_block = g->cfg_blocks == 1 && g->cfg_warps == kOneBlockWarps;
-  const bool short_bodies = body_iters(g) <= kWindowIters || block_window_small(g->max_span, g->last_root);
-  const bool window = fits.window && (one_block || (free_shape && short_bodies));
-  const bool queue = fits.queue && !window &&
-                     (one_block || (free_shape && block_exec_alone(g->n, g->n_roots, g->n_edges, g->desc.body,
-                                                                   g->desc.spin_iters, fits.own_warps > 0)));
+  const bool window = fits.window && (one_block || (free_shape && window_best(g)));
+  const bool queue = fits.queue && !window && (one_block || (free_shape && queue_best(g, fits)));
   const bool block = window || queue;
   const bool auto_owned = free_shape && !block && fits.own_warps > 0 && fits.own_warps <= g_dev.owned_warps &&
                           body_iters(g) <= kOwnedIters;
@@ -1408,7 +1413,8 @@ rt_status start_run(rt_graph* g, int32_t replays) {
 namespace grt {
 ExecChoice exec_choice(rt_graph_t g) {
   const ExecFits f = g->analyzed && g->n > 0 ? exec_fits(g) : ExecFits{};
-  return ExecChoice{f.window || f.queue ? kOneBlockWarps : 0, f.own_warps};
+  return ExecChoice{f.window || f.queue ? kOneBlockWarps : 0, f.own_warps,
+                    f.window ? window_best(g) : f.queue && queue_best(g, f)};
 }
 }  // namespace grt
 

@@ -613,9 +613,10 @@ void graph_set_mem_cap(rt_graph_t g, size_t cap);
 rt_status graph_trim(rt_graph_t g);
 // for the tuner: the warps to configure one block with (ring policy) for an
 // analysed graph to run inside it, and the owned chunks' warps that the library
-// would take for it (0: not so)
+// would take for it (0: not so), under the ring policy
 struct ExecChoice {
   int one_block_warps, own_warps;
+  bool one_block_by_itself;  // it takes one block with no shape configured
 };
 ExecChoice exec_choice(rt_graph_t g);
 // in_blocks: the ring policy runs each of the batch's graphs inside one block

@@ -283,7 +283,12 @@ rt_status rt_tune_exec(rt_graph_t g, const char* cache_path, rt_exec_config* bes
                           std::to_string(st.n_edges) + "/" + std::to_string(st.n_roots);
   auto apply = [&](const rt_exec_config& c) -> rt_status {
     rt_status r = rt_graph_exec_policy(g, c.policy);
-    return r != RT_OK ? r : rt_graph_exec_config(g, c.blocks, c.warps, c.claim, c.keep);
+    if (r != RT_OK) return r;
+    // one block that the library takes by itself stays its choice: the graph's next
+    // launches may not fit one
+    const ExecChoice x = exec_choice(g);
+    const bool leave = c.policy == RT_EXEC_RING && c.blocks == 1 && c.warps == x.one_block_warps && x.one_block_by_itself;
+    return rt_graph_exec_config(g, leave ? 0 : c.blocks, leave ? 0 : c.warps, c.claim, c.keep);
   };
   std::vector<double> c;
   if (cache_get(cache_path, key, &c) && c.size() >= 6) {

@@ -111,3 +111,21 @@ def test_the_caches_entries_are_of_the_current_kernels(tmp_path):
     for old in ("tile", "tile2", "tile3"):
         cache.write_text(f"{old}/{key.split('/', 1)[1]} 8 8 0.001\n")
         assert grt.rt_tune_tile(tr, cache)[2] > 0.001
+
+
+def test_a_tuned_graph_takes_larger_launches():
+    """Tuned for launches that run inside one block, then cleared and given ones that do not."""
+    ensure_built()
+    small, large = tg.taskbench(32, 100, "stencil"), tg.taskbench(1024, 100, "stencil")
+    g = grt.Graph(2, large.dom_lo, large.dom_hi)
+    for tr in (small, large):
+        g.clear()
+        g.launch_trace(tr)
+        g.analyze()
+        if tr is small:
+            assert g.tune()["blocks"] == 1
+        g.execute()
+        g.sync()
+        st = g.stats()
+        assert (st["exec_blocks"] == 1) == (tr is small) and st["exec_counters"]["tasks"] == tr.n
+    g.close()
