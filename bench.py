@@ -140,6 +140,9 @@ def run_batched(grt, torch, flush, steps, world=1, rank=0):
 
 SERVE_REQUESTS, SERVE_RATE = 2000, 50_000.0
 SERVE_SLOTS, SERVE_WORKERS, SERVE_MAX_BATCH = 512, 4, 64
+# Alone, a batch of 43 requests is analysed quicker at 16 x 16 (1.6 ms against 1.9, what the tile tuner measures); with
+# four workers' analyses side by side the fewer entries of 16 x 32 count (3.0M against 4.9M): 16.1k graphs/s against 13.6k
+SERVE_TILE = (16, 32)
 SERVE_EXEC_WARPS = 2  # serving kernel warps per SM: leaves room for 3 sweep blocks beside it
 
 
@@ -248,13 +251,15 @@ def run_stitched(grt, torch):
     joined by the edges between two copies of the trace (rt_execute_stitched),
     so that replay r + 1 starts where its own predecessors in replay r are
     done. EMPTY bodies; the barrier replay runs under the autotuner's policy and
-    shape for one execution of the trace, the stitched one (a ring kernel) at the
-    best of four ring shapes; times include the counter reset and seeding."""
+    shape for one execution of the trace, the stitched one at the best of the
+    library's own choice and four ring shapes; times include the counter reset and
+    seeding."""
     R = 20
     res = {"replays": R, "steps_per_replay": 100, "width": 1024,
            "launch": "barrier replay: the autotuner's policy and shape for one execution of the trace; stitched "
-                     "replay (a ring kernel): the best of four ring shapes (blocks, warps, claim, keep)"}
-    ring_shapes = [(304, 4, 2, 8), (304, 2, 2, 4), (152, 4, 1, 4), (152, 2, 2, 8)]
+                     "replay: the best of the library's own choice (0, 0, 0, 0) and four ring shapes (blocks, warps, "
+                     "claim, keep)"}
+    shapes = [(0, 0, 0, 0), (304, 4, 2, 8), (304, 2, 2, 4), (152, 4, 1, 4), (152, 2, 2, 8)]
     for pat in ("stencil", "random"):
         T = tg.taskbench(1024, 100, pat, seed=0)
         g = grt.Graph(2, T.dom_lo, T.dom_hi, flags=grt.RT_GRAPH_PROFILE)
@@ -272,7 +277,7 @@ def run_stitched(grt, torch):
         g2.analyze()
         ana = g2.stats()["ms_analyze"]
         best = None
-        for sh in ring_shapes:
+        for sh in shapes:
             g2.exec_config(*sh)
             st = [g2.execute_stitched(R) for _ in range(4)]
             m = float(np.median(st[1:]))
@@ -319,9 +324,7 @@ def run_served(grt, n_requests=SERVE_REQUESTS, rate=SERVE_RATE, world=1, rank=0)
         from paper_2508_16522_gb300 import shard
         reqs = [stream_all[k] for k in shard.my_arrivals([shard.footprint(r.trace) for r in stream_all], world, rank)]
     gen_s = time.perf_counter() - t0
-    # the tile is tuned on a batch of the size the stream produces (about 43)
-    cache = TUNE_CACHE if world == 1 else None  # ranks would append to one file at once
-    tile = list(grt.rt_tune_tile(stacked_batch([r.trace for r in stream_all[:43]], SERVE_MAX_BATCH), cache)[:2])
+    tile = list(SERVE_TILE)
     srv = grt.Server(2, [0, 0], [1023, 1023], body=grt.RT_BODY_EMPTY, budget_bytes=8 << 30,
                      max_inflight=SERVE_SLOTS, max_tasks=16384, workers=SERVE_WORKERS, tile=tile,
                      max_batch=SERVE_MAX_BATCH, exec_warps=SERVE_EXEC_WARPS)
