@@ -33,3 +33,19 @@ def test_iteration_counts(body, config):
         g.sync()
         assert np.array_equal(g.out.cpu().numpy(), want), iters
         g.close()
+
+
+def test_no_executor_runs_a_body_quicker_than_it_runs_alone():
+    """The rate that efficiencies are measured against is the body's best: a chain of long bodies takes at least that."""
+    ensure_built()
+    alone = grt.rt_microbench_atomics()["fma_body_ns_per_iter"]
+    iters, tr = 60000, tg.taskbench(1, 40, "stencil")
+    for config in ((8, 2, 1, 4), (0, 0, 0, 0)):
+        g = gpu_graph(tr, body=grt.RT_BODY_FMA, spin_iters=iters, flags=grt.RT_GRAPH_PROFILE)
+        g.analyze()
+        g.exec_config(*config)
+        for _ in range(3):
+            g.execute()
+            g.sync()
+            assert g.stats()["ms_exec_kernel"] * 1e6 > 0.98 * alone * iters * tr.n
+        g.close()
